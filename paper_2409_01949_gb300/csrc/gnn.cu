@@ -36,108 +36,216 @@ constexpr int kLayers = 3;
 
 __device__ __forceinline__ float relu(float x) { return x > 0.f ? x : 0.f; }
 
-// out[r][o] (+)= sum_i W[o][i] in[r][i] + bias[o]; optional relu.  One block per
-// 8 rows, thread per output channel.
-__global__ void k_dense_fwd(const float* __restrict__ in, int R, int Din,
-                            const float* __restrict__ W, const float* __restrict__ bias,
-                            int Dout, float* __restrict__ out, int accumulate, int act) {
-  extern __shared__ float xs[];   // [8][Din]
-  const int r0 = blockIdx.x * 8;
-  for (int t = threadIdx.x; t < 8 * Din; t += blockDim.x) {
-    const int r = r0 + t / Din;
-    xs[t] = r < R ? in[(int64_t)r * Din + t % Din] : 0.f;
+// Dense FP32 layer, forward (kNT) or backward in its input:
+//   kNT:  out[r][o] = act(sum_i W1[o][i] in1[r][i] (+ sum_i W2[o][i] in2[r][i]) + bias[o])
+//   else: out_y[r][i] = sum_o W_y[o][i] g[r][o], g = in1 where mask > 0 (the
+//         ReLU's derivative), y = blockIdx.z picking W1 -> out or W2 -> out2;
+//         out2's rows are divided by their node's degree, ready for the
+//         transposed neighbour mean.
+// W [rows of W][ldw].  A CTA forms kNetRows rows x 64 columns from 32-deep
+// slices of both operands in shared memory, 2 x 4 sums a thread.  The layers
+// are products of microseconds: latency decides, so the tile is small enough
+// that a training batch (2728 rows) fills the SMs, and both weights of a
+// message-passing layer share a launch.  A thread-per-output-channel form
+// that read its weight row by strided loads took 58 us a layer at 2728 rows,
+// K = 64.  Loss and gradient of that batch (8 samples x 341 nodes, 18 launches,
+// host copies included): 4.91 ms before these kernels, 0.32 ms with them.
+constexpr int kNetRows = 16;
+constexpr int kNetDepth = 32;
+constexpr int kNetLd = 68;   // leading dimension of the weight slice (16-byte rows, few conflicts)
+
+template <bool kNT>
+__global__ void __launch_bounds__(128) k_net_dense(
+    const float* __restrict__ in1, const float* __restrict__ W1, int D1,
+    const float* __restrict__ in2, const float* __restrict__ W2, int D2,
+    const float* __restrict__ bias, const float* __restrict__ mask, const int* __restrict__ off,
+    int n_nodes, int R, int Dout, int act, float* __restrict__ out, float* __restrict__ out2) {
+  __shared__ float xs[kNetRows][kNetDepth];
+  __shared__ __align__(16) float ws[kNetDepth][kNetLd];
+  const int r0 = blockIdx.x * kNetRows, o0 = blockIdx.y * 64;
+  const int tc = (threadIdx.x & 15) * 4, tr = (threadIdx.x >> 4) * 2;
+  float acc[2][4] = {};
+  const int parts = kNT && W2 ? 2 : 1;
+  for (int part = 0; part < parts; ++part) {
+    const float* in = part ? in2 : in1;
+    const float* W = kNT ? (part ? W2 : W1) : (blockIdx.z ? W2 : W1);
+    const int D = part ? D2 : D1;
+    for (int k0 = 0; k0 < D; k0 += kNetDepth) {
+      __syncthreads();
+      for (int t = threadIdx.x; t < kNetRows * kNetDepth; t += 128) {
+        const int r = r0 + t / kNetDepth, k = k0 + t % kNetDepth;
+        float v = r < R && k < D ? in[(int64_t)r * D + k] : 0.f;
+        if (!kNT && mask && r < R && k < D && !(mask[(int64_t)r * D + k] > 0.f)) v = 0.f;
+        xs[t / kNetDepth][t % kNetDepth] = v;
+      }
+      for (int t = threadIdx.x; t < kNetDepth * 64; t += 128) {
+        // consecutive threads along the weight's rows
+        const int k = kNT ? t % kNetDepth : t / 64, o = kNT ? t / kNetDepth : t % 64;
+        const bool in_w = k0 + k < D && o0 + o < Dout;
+        ws[k][o] = !in_w ? 0.f
+                         : (kNT ? W[(int64_t)(o0 + o) * D + k0 + k]
+                                : W[(int64_t)(k0 + k) * Dout + o0 + o]);
+      }
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < kNetDepth; ++k) {
+        const float4 w = *reinterpret_cast<const float4*>(&ws[k][tc]);
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+          const float x = xs[tr + a][k];
+          acc[a][0] = fmaf(w.x, x, acc[a][0]);
+          acc[a][1] = fmaf(w.y, x, acc[a][1]);
+          acc[a][2] = fmaf(w.z, x, acc[a][2]);
+          acc[a][3] = fmaf(w.w, x, acc[a][3]);
+        }
+      }
+    }
   }
-  __syncthreads();
-  for (int o = threadIdx.x; o < Dout; o += blockDim.x) {
-    const float* w = W + (int64_t)o * Din;
-    for (int rr = 0; rr < 8; ++rr) {
-      const int r = r0 + rr;
-      if (r >= R) break;
-      float acc = 0.f;
-      for (int i = 0; i < Din; ++i) acc += w[i] * xs[rr * Din + i];
-      float* dst = out + (int64_t)r * Dout + o;
-      float v = acc + (accumulate ? *dst : (bias ? bias[o] : 0.f));
-      *dst = act ? relu(v) : v;
+  float* dst = !kNT && blockIdx.z ? out2 : out;
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const int r = r0 + tr + a;
+    if (r >= R) continue;
+    float deg = 1.f;
+    if (!kNT && blockIdx.z) {
+      const int s = r % n_nodes;
+      deg = (float)max(off[s + 1] - off[s], 1);
+    }
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int o = o0 + tc + b;
+      if (o >= Dout) continue;
+      float v = acc[a][b];
+      if (kNT) {
+        if (bias) v += bias[o];
+        if (act) v = relu(v);
+      } else if (blockIdx.z) {
+        v = v / deg;
+      }
+      dst[(int64_t)r * Dout + o] = v;
     }
   }
 }
 
-// dIn[r][i] (+)= sum_o W[o][i] dOut[r][o]
-__global__ void k_dense_bwd_in(const float* __restrict__ dout, int R, int Dout,
-                               const float* __restrict__ W, int Din, float* __restrict__ din,
-                               int accumulate) {
-  extern __shared__ float gs[];   // [8][Dout]
-  const int r0 = blockIdx.x * 8;
-  for (int t = threadIdx.x; t < 8 * Dout; t += blockDim.x) {
-    const int r = r0 + t / Dout;
-    gs[t] = r < R ? dout[(int64_t)r * Dout + t % Dout] : 0.f;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < Din; i += blockDim.x) {
-    for (int rr = 0; rr < 8; ++rr) {
-      const int r = r0 + rr;
-      if (r >= R) break;
-      float acc = 0.f;
-      for (int o = 0; o < Dout; ++o) acc += W[(int64_t)o * Din + i] * gs[rr * Dout + o];
-      float* dst = din + (int64_t)r * Din + i;
-      *dst = acc + (accumulate ? *dst : 0.f);
+// One weight gradient: dW[o][i] = sum_r dout[r][o] in[r][i] (dout where mask >
+// 0; mask null: all of it), db[o] = sum_r dout[r][o], written at w_off and
+// b_off (< 0: none) of a partial gradient.
+struct WGrad {
+  const float* dout;
+  const float* mask;
+  const float* in;
+  int Dout, Din;
+  int64_t w_off, b_off;
+  int tile0;   // the gradient's first 64 x 64 tile in the launch
+};
+constexpr int kWGrads = 2 * kLayers + 2;
+constexpr int kWGradChunks = 64;   // at most this many partial gradients
+struct WGradList {
+  WGrad g[kWGrads];
+};
+
+// Partial gradients of every layer in one launch: CTA (x, y) sums rows
+// [x chunk, (x + 1) chunk) into one 64 x 64 tile of partial gradient x, 4 x 4
+// sums a thread from 32-row slices in shared memory; k_wgrad_sum then adds the
+// partials in order.  Splitting the rows is what fills the chip: with one
+// thread per weight and the whole batch as its serial chain, a layer's 4096
+// weights took 0.85 ms at 2728 rows on 16 CTAs, 85% of the gradient's time.
+__global__ void __launch_bounds__(256) k_wgrad(const __grid_constant__ WGradList L, int R,
+                                               int chunk, int64_t nw, float* __restrict__ part) {
+  __shared__ __align__(16) float ds[32][64];
+  __shared__ __align__(16) float xs[32][64];
+  int q = 0;
+  while (q + 1 < kWGrads && (int)blockIdx.y >= L.g[q + 1].tile0) ++q;
+  const WGrad& G = L.g[q];
+  const int ti = (G.Din + 63) / 64;
+  const int tile = blockIdx.y - G.tile0;
+  const int o0 = (tile / ti) * 64, i0 = (tile % ti) * 64;
+  const int ra = blockIdx.x * chunk, rb = min(R, ra + chunk);
+  const int to = (threadIdx.x >> 4) * 4, tx = (threadIdx.x & 15) * 4;
+  float acc[4][4] = {}, bacc[4] = {};
+  for (int r0 = ra; r0 < rb; r0 += 32) {
+    __syncthreads();
+    for (int t = threadIdx.x; t < 32 * 64; t += 256) {
+      const int rr = t >> 6, c = t & 63, r = r0 + rr;
+      float d = r < rb && o0 + c < G.Dout ? G.dout[(int64_t)r * G.Dout + o0 + c] : 0.f;
+      if (G.mask && r < rb && o0 + c < G.Dout && !(G.mask[(int64_t)r * G.Dout + o0 + c] > 0.f))
+        d = 0.f;
+      ds[rr][c] = d;
+      xs[rr][c] = r < rb && i0 + c < G.Din ? G.in[(int64_t)r * G.Din + i0 + c] : 0.f;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int rr = 0; rr < 32; ++rr) {
+      const float4 d = *reinterpret_cast<const float4*>(&ds[rr][to]);
+      const float4 x = *reinterpret_cast<const float4*>(&xs[rr][tx]);
+      const float dv[4] = {d.x, d.y, d.z, d.w}, xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        bacc[a] += dv[a];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(dv[a], xv[b], acc[a][b]);
+      }
     }
   }
-}
-
-// dW[o][i] += sum_r dOut[r][o] in[r][i];  db[o] += sum_r dOut[r][o]  (fixed order)
-__global__ void k_wgrad(const float* __restrict__ dout, const float* __restrict__ in, int R,
-                        int Dout, int Din, float* __restrict__ dW, float* __restrict__ db) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < Dout * Din) {
-    const int o = idx / Din, i = idx - o * Din;
-    float acc = 0.f;
-    for (int r = 0; r < R; ++r) acc += dout[(int64_t)r * Dout + o] * in[(int64_t)r * Din + i];
-    dW[idx] += acc;
-  }
-  if (db && idx < Dout) {
-    float acc = 0.f;
-    for (int r = 0; r < R; ++r) acc += dout[(int64_t)r * Dout + idx];
-    db[idx] += acc;
+  float* P = part + (int64_t)blockIdx.x * nw;
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    const int o = o0 + to + a;
+    if (o >= G.Dout) continue;
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      if (i0 + tx + b < G.Din) P[G.w_off + (int64_t)o * G.Din + i0 + tx + b] = acc[a][b];
+    if (G.b_off >= 0 && i0 == 0 && tx == 0) P[G.b_off + o] = bacc[a];
   }
 }
 
-// agg[(b,s)][h] = mean_{t in N(s)} A[(b,t)][h]
-__global__ void k_agg(const float* __restrict__ A, int nb_nodes, int B,
-                      const int* __restrict__ off, const int* __restrict__ nb,
-                      float* __restrict__ agg) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)B * nb_nodes * kH) return;
-  const int h = idx % kH;
-  const int64_t rs = idx / kH;
-  const int s = rs % nb_nodes, b = rs / nb_nodes;
-  const int e0 = off[s], e1 = off[s + 1];
-  float acc = 0.f;
-  for (int e = e0; e < e1; ++e) acc += A[((int64_t)b * nb_nodes + nb[e]) * kH + h];
-  agg[idx] = e1 > e0 ? acc / (float)(e1 - e0) : 0.f;
-}
-
-// dA[(b,s)][h] += sum_{t in N(s)} G[(b,t)][h] / |N(t)|   (transpose of the mean)
-__global__ void k_aggT(const float* __restrict__ G, int nb_nodes, int B,
-                       const int* __restrict__ off, const int* __restrict__ nb,
-                       float* __restrict__ dA) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)B * nb_nodes * kH) return;
-  const int h = idx % kH;
-  const int64_t rs = idx / kH;
-  const int s = rs % nb_nodes, b = rs / nb_nodes;
-  float acc = 0.f;
-  for (int e = off[s]; e < off[s + 1]; ++e) {
-    const int t = nb[e];
-    acc += G[((int64_t)b * nb_nodes + t) * kH + h] / (float)(off[t + 1] - off[t]);
-  }
-  dA[idx] += acc;
-}
-
-// dZ = dA * (A > 0)
-__global__ void k_relu_mask(const float* __restrict__ A, float* __restrict__ dA, int64_t n) {
+// dW = the sum of the partial gradients, in order
+__global__ void k_wgrad_sum(const float* __restrict__ part, int chunks, int64_t nw,
+                            float* __restrict__ dW) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n && !(A[i] > 0.f)) dA[i] = 0.f;
+  if (i >= nw) return;
+  float v = 0.f;
+#pragma unroll 8
+  for (int c = 0; c < chunks; ++c) v += part[(int64_t)c * nw + i];
+  dW[i] = v;
+}
+
+// out[(b,s)][h] (+)= sum_{t in N(s)} A[(b,t)][h], over |N(s)| with `mean`.  A
+// CTA per row: 16 lanes of four channels, the neighbour list dealt round-robin
+// to 8 groups of them and the group sums added in order, so that a coarse
+// node's list of hundreds is not one thread's serial chain.
+__global__ void __launch_bounds__(128) k_agg(const float* __restrict__ A, int nb_nodes,
+                                             const int* __restrict__ off,
+                                             const int* __restrict__ nb, int mean,
+                                             float* __restrict__ out) {
+  __shared__ __align__(16) float4 sh[8][16];
+  const int64_t rs = blockIdx.x;
+  const int s = (int)(rs % nb_nodes);
+  const int64_t row0 = rs - s;   // node 0 of this sample
+  const int e0 = off[s], e1 = off[s + 1];
+  const int l = threadIdx.x & 15, g = threadIdx.x >> 4;
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+  for (int e = e0 + g; e < e1; e += 8) {
+    const float4 a = reinterpret_cast<const float4*>(A + (row0 + nb[e]) * kH)[l];
+    v.x += a.x, v.y += a.y, v.z += a.z, v.w += a.w;
+  }
+  sh[g][l] = v;
+  __syncthreads();
+  if (g != 0) return;
+#pragma unroll
+  for (int q = 1; q < 8; ++q) {
+    const float4 a = sh[q][l];
+    v.x += a.x, v.y += a.y, v.z += a.z, v.w += a.w;
+  }
+  float4* dst = reinterpret_cast<float4*>(out + rs * kH) + l;
+  if (mean) {
+    const float deg = (float)max(e1 - e0, 1);
+    *dst = make_float4(v.x / deg, v.y / deg, v.z / deg, v.w / deg);
+  } else {
+    const float4 a = *dst;
+    *dst = make_float4(a.x + v.x, a.y + v.y, a.z + v.z, a.w + v.w);
+  }
 }
 
 // dY = 2 w_b (Y - T) / B;  loss partial per block
@@ -457,30 +565,32 @@ double gnn_pass(elmfb_ctx* h, int B, const float* X, const float* T, const float
   const int64_t R = (int64_t)B * n;
   Gnn g{h, K, n, gnn_weight_count(K)};
   g.bind(h->d_gnn_w.as<float>());
-  // activations: A0..A3, AGG1..3 [R][H]; scratch dA, tmp [R][H]
-  h->d_gnn_act.alloc((size_t)R * kH * (2 * kLayers + 3) * sizeof(float), st);
+  // activations A0..A3 and neighbour means AG1..3, their gradients dA0..dA3
+  // and one scratch, each [R][H]
+  h->d_gnn_act.alloc((size_t)R * kH * (3 * kLayers + 3) * sizeof(float), st);
   float* A[kLayers + 1];
   float* AG[kLayers];
+  float* dA[kLayers + 1];
   float* base = h->d_gnn_act.as<float>();
   for (int l = 0; l <= kLayers; ++l) A[l] = base + (int64_t)l * R * kH;
   for (int l = 0; l < kLayers; ++l) AG[l] = base + (int64_t)(kLayers + 1 + l) * R * kH;
-  float* dA = base + (int64_t)(2 * kLayers + 1) * R * kH;
-  float* tmp = dA + R * kH;
-  const unsigned rb = (unsigned)ceil_div(R, 8);
-  const unsigned eb = (unsigned)ceil_div(R * kH, 256);
+  for (int l = 0; l <= kLayers; ++l) dA[l] = base + (int64_t)(2 * kLayers + 1 + l) * R * kH;
+  float* tmp = base + (int64_t)(3 * kLayers + 2) * R * kH;
+  const unsigned rb = (unsigned)ceil_div(R, kNetRows);
   const int* off = h->d_gnn_off.as<int>();
   const int* nb = h->d_gnn_nb.as<int>();
-  k_dense_fwd<<<rb, 128, 8 * K * sizeof(float), st>>>(X, (int)R, K, g.W_in, g.b_in, kH, A[0], 0, 1);
+  auto forward = [&](const float* in1, const float* W1, int D1, const float* in2,
+                     const float* W2, const float* bias, int Dout, int act, float* out) {
+    k_net_dense<true><<<dim3(rb, (unsigned)ceil_div(Dout, 64)), 128, 0, st>>>(
+        in1, W1, D1, in2, W2, kH, bias, nullptr, nullptr, n, (int)R, Dout, act, out, nullptr);
+  };
+  forward(X, g.W_in, K, nullptr, nullptr, g.b_in, kH, 1, A[0]);
   for (int l = 0; l < kLayers; ++l) {
-    k_agg<<<eb, 256, 0, st>>>(A[l], n, B, off, nb, AG[l]);
-    k_dense_fwd<<<rb, 128, 8 * kH * sizeof(float), st>>>(A[l], (int)R, kH, g.W_self[l], g.b_l[l],
-                                                          kH, A[l + 1], 0, 0);
-    k_dense_fwd<<<rb, 128, 8 * kH * sizeof(float), st>>>(AG[l], (int)R, kH, g.W_nb[l], nullptr,
-                                                          kH, A[l + 1], 1, 1);
+    k_agg<<<(unsigned)R, 128, 0, st>>>(A[l], n, off, nb, 1, AG[l]);
+    forward(A[l], g.W_self[l], kH, AG[l], g.W_nb[l], g.b_l[l], kH, 1, A[l + 1]);
   }
-  k_dense_fwd<<<rb, 128, 8 * kH * sizeof(float), st>>>(A[kLayers], (int)R, kH, g.W_out, g.b_out,
-                                                        K, Y, 0, 0);
-  count_launch(h, 2 + 3 * kLayers);
+  forward(A[kLayers], g.W_out, kH, nullptr, nullptr, g.b_out, K, 0, Y);
+  count_launch(h, 2 + 2 * kLayers);
   double loss = 0.0;
   if (T) {
     h->d_gnn_lp.alloc(kDotBlocks * sizeof(double), st);
@@ -492,32 +602,41 @@ double gnn_pass(elmfb_ctx* h, int B, const float* X, const float* T, const float
     if (dW) {
       Gnn gd{h, K, n, g.nw};
       gd.bind(dW);
-      CUDA_CHECK(cudaMemsetAsync(dW, 0, g.nw * sizeof(float), st));
-      // output layer
-      k_wgrad<<<(unsigned)ceil_div((int64_t)K * kH, 256), 256, 0, st>>>(dY, A[kLayers], (int)R, K,
-                                                                         kH, gd.W_out, gd.b_out);
-      k_dense_bwd_in<<<rb, 128, 8 * K * sizeof(float), st>>>(dY, (int)R, K, g.W_out, kH, dA, 0);
+      // gradients of the activations, last layer first; dA[l] of a layer with
+      // a ReLU is masked where it is read
+      k_net_dense<false><<<dim3(rb, 1, 1), 128, 0, st>>>(dY, g.W_out, K, nullptr, nullptr, 0,
+                                                         nullptr, nullptr, off, n, (int)R, kH, 0,
+                                                         dA[kLayers], nullptr);
       for (int l = kLayers - 1; l >= 0; --l) {
-        k_relu_mask<<<eb, 256, 0, st>>>(A[l + 1], dA, R * kH);   // dA now holds dZ_l
-        k_wgrad<<<(unsigned)ceil_div(kH * kH, 256), 256, 0, st>>>(dA, A[l], (int)R, kH, kH,
-                                                                  gd.W_self[l], gd.b_l[l]);
-        k_wgrad<<<(unsigned)ceil_div(kH * kH, 256), 256, 0, st>>>(dA, AG[l], (int)R, kH, kH,
-                                                                  gd.W_nb[l], nullptr);
-        k_dense_bwd_in<<<rb, 128, 8 * kH * sizeof(float), st>>>(dA, (int)R, kH, g.W_nb[l], kH,
-                                                                 tmp, 0);
-        // dA_{l-1} = dZ W_self + aggT(dZ W_nb): write into the tmp2 region (reuse A? no)
-        float* dprev = AG[l];   // AG[l] no longer needed once its gradient is taken
-        k_dense_bwd_in<<<rb, 128, 8 * kH * sizeof(float), st>>>(dA, (int)R, kH, g.W_self[l],
-                                                                 kH, dprev, 0);
-        k_aggT<<<eb, 256, 0, st>>>(tmp, n, B, off, nb, dprev);
-        CUDA_CHECK(cudaMemcpyAsync(dA, dprev, R * kH * sizeof(float), cudaMemcpyDeviceToDevice,
-                                   st));
-        count_launch(h, 6);
+        // dA_l = dZ W_self + (transposed mean)(dZ W_nb)
+        k_net_dense<false><<<dim3(rb, 1, 2), 128, 0, st>>>(
+            dA[l + 1], g.W_self[l], kH, nullptr, g.W_nb[l], 0, nullptr, A[l + 1], off, n, (int)R,
+            kH, 0, dA[l], tmp);
+        k_agg<<<(unsigned)R, 128, 0, st>>>(tmp, n, off, nb, 0, dA[l]);
       }
-      k_relu_mask<<<eb, 256, 0, st>>>(A[0], dA, R * kH);
-      k_wgrad<<<(unsigned)ceil_div((int64_t)kH * K, 256), 256, 0, st>>>(dA, X, (int)R, kH, K,
-                                                                         gd.W_in, gd.b_in);
-      count_launch(h, 4);
+      // every weight gradient at once
+      WGradList wl;
+      int tiles = 0, nq = 0;
+      auto add = [&](const float* dout, const float* mask, int Dout, const float* in, int Din,
+                     const float* w, const float* b) {
+        wl.g[nq++] = {dout, mask, in, Dout, Din, w - dW, b ? b - dW : -1, tiles};
+        tiles += (int)(ceil_div(Dout, 64) * ceil_div(Din, 64));
+      };
+      add(dY, nullptr, K, A[kLayers], kH, gd.W_out, gd.b_out);
+      for (int l = kLayers - 1; l >= 0; --l) {
+        add(dA[l + 1], A[l + 1], kH, A[l], kH, gd.W_self[l], gd.b_l[l]);
+        add(dA[l + 1], A[l + 1], kH, AG[l], kH, gd.W_nb[l], nullptr);
+      }
+      add(dA[0], A[0], kH, X, K, gd.W_in, gd.b_in);
+      const int chunk = (int)(ceil_div(ceil_div(R, kWGradChunks), 32) * 32);
+      const int chunks = (int)ceil_div(R, chunk);
+      DevBuf dpart;
+      dpart.alloc((size_t)chunks * g.nw * sizeof(float), st);
+      k_wgrad<<<dim3((unsigned)chunks, (unsigned)tiles), 256, 0, st>>>(wl, (int)R, chunk, g.nw,
+                                                                       dpart.as<float>());
+      k_wgrad_sum<<<(unsigned)ceil_div(g.nw, 256), 256, 0, st>>>(dpart.as<float>(), chunks, g.nw,
+                                                                 dW);
+      count_launch(h, 3 + 2 * kLayers);
     }
     std::vector<double> lp(kDotBlocks);
     CUDA_CHECK(cudaMemcpyAsync(lp.data(), h->d_gnn_lp.p, kDotBlocks * sizeof(double),

@@ -171,3 +171,48 @@ def test_fcg_block_jacobi_matches_paper_protocol_error():
     print(f"FCG block-Jacobi rel L2 {err:.3e} after {info.iterations} its; "
           f"oracle LSQR-15000 {g['lsqr']['rel_l2']:.3e}")
     assert err <= 1.01 * g["lsqr"]["rel_l2"]
+
+
+@pytest.mark.parametrize("K,B", [(1, 1), (33, 3), (64, 1), (100, 4)])
+def test_gnn_gradient_at_ragged_sizes(K, B):
+    """Forward pass, loss and every weight gradient where the 16-row and
+    64-column tiles are ragged (K = 1, 33, 100; 21 B rows, 84 rows past two
+    row chunks), against the same network in FP64 with torch's autograd.  All
+    sums are FP32 of at most 128 terms, the gradients' of at most 84: 2^-24
+    times that chain length is 8e-6 of the terms' magnitude, so 1e-4 of the
+    largest value covers the five layers."""
+    import torch
+    P = WL.poisson2d(levels=(1, 2, 4), features=K, n_side=24, n_boundary_side=12)
+    H = 64
+    nbrs = _oracle_graph(P)
+    rng = np.random.default_rng(7)
+    w = (0.3 * rng.standard_normal(OG.n_weights(K, H))).astype(np.float32)
+    X = rng.standard_normal((B, P.n_subdomains, K)).astype(np.float32)
+    T = rng.standard_normal((B, P.n_subdomains, K)).astype(np.float32)
+    wb = (0.5 + rng.random(B)).astype(np.float32)
+    with E.Solver.from_problem(P, precision=E.FP32) as s:
+        s.assemble_problem(P)
+        s.gnn_set_weights(w)
+        Y, grad, loss = s.gnn_eval(X, T, wb, grad=True)
+    wt = torch.from_numpy(w).double().requires_grad_(True)
+    mean = torch.zeros((P.n_subdomains, P.n_subdomains), dtype=torch.float64)
+    for i, nb in enumerate(nbrs):
+        mean[i, nb] = 1.0 / len(nb)
+    o = 0
+
+    def take(*shape):
+        nonlocal o
+        n = int(np.prod(shape))
+        o += n
+        return wt[o - n:o].reshape(shape)
+    A = torch.relu(torch.from_numpy(X).double() @ take(H, K).T + take(H))
+    for _ in range(3):
+        ws, wn, b = take(H, H), take(H, H), take(H)
+        A = torch.relu(A @ ws.T + mean @ A @ wn.T + b)
+    Yo = A @ take(K, H).T + take(K)
+    Lo = (torch.from_numpy(wb).double() * ((Yo - torch.from_numpy(T).double()) ** 2).sum((1, 2))).mean()
+    Lo.backward()
+    Yo, go = Yo.detach().numpy(), wt.grad.numpy()
+    assert np.allclose(Y, Yo, rtol=0, atol=1e-4 * np.abs(Yo).max())
+    assert loss == pytest.approx(Lo.item(), rel=1e-4)
+    assert np.allclose(grad, go, rtol=0, atol=1e-4 * np.abs(go).max())
