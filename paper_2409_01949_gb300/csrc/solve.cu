@@ -27,6 +27,8 @@
 // from run to run.
 #include <algorithm>
 #include <cmath>
+
+#include <cooperative_groups.h>
 #include <cstdlib>
 #include <map>
 #include <mutex>
@@ -2760,92 +2762,124 @@ void block_jacobi_setup(elmfb_ctx* h, double shift, bool identity, double abs_sh
 
 namespace {
 
-// Number of eigenvalues below lam of the Golub-Kahan tridiagonal of B_k: the
-// (2k+1) x (2k+1) symmetric matrix with zero diagonal and off-diagonal
-// alpha_1, beta_2, alpha_2, beta_3, ..., alpha_k, beta_{k+1}, whose eigenvalues
-// are +-sigma_i(B_k) and 0 (Golub & Kahan 1965).  Sturm sequence of the LDL^T
-// factorisation of T - lam I, tiny pivots replaced by -pivmin.
-__device__ int gk_sturm_count(const double* __restrict__ gk, int k, double lam, double pivmin) {
-  double d = -lam;
-  int cnt = d < 0.0;
-  for (int i = 0; i < 2 * k; ++i) {
-    const int j = i >> 1;
-    const double e = (i & 1) ? gk[2 * (j + 1) + 1] : gk[2 * j];   // beta_{j+2} : alpha_{j+1}
-    if (fabs(d) < pivmin) d = -pivmin;
-    d = -lam - e * e / d;
-    cnt += d < 0.0;
-  }
-  return cnt;
+// Extreme singular values of B_k: the (2k+1) x (2k+1) Golub-Kahan tridiagonal
+// T of B_k (zero diagonal, off-diagonal alpha_1, beta_2, alpha_2, beta_3, ...,
+// alpha_k, beta_{k+1}) has the eigenvalues +-sigma_i(B_k) and 0 (Golub & Kahan
+// 1965).  Multisection of the number of its eigenvalues below a trial point
+// lam: 256 points a round for each extreme, the two side by side, spread
+// geometrically while the interval is wide and evenly once it is narrow, to
+// 1e-10 relative: out[0] = sigma_max (the point where the count reaches
+// 2k+1), out[1] = sigma_min (where it reaches k+2).  k = 0: zeros.
+//
+// The count is that of the sign changes in the leading principal minors of
+// T - lam I (Givens 1954), p_{i+1} = -lam p_i - e_i^2 p_{i-1}, which carry the
+// same relative backward error in lam and e_i as the pivots p_{i+1} / p_i of
+// the LDL^T recurrence and need no division; T is scaled by a power of two to
+// norm <= 1 and the pair (p_i, p_{i+1}) back to order 1 every four steps.
+// GB300 issues an FP64 warp instruction over 64 cycles of a sub-partition, so
+// FP64 instructions per step decide the time: a cluster of 8 CTAs with one
+// warp per extreme has each warp on a sub-partition of its own.  The LDL^T
+// form in one 512-thread CTA took 122 us at k = 4 and 450 us at k = 20; this
+// one saves 115 us of a k = 4 solve and 400 us of a k = 20 one.
+constexpr int kBidiagCtas = 8;
+constexpr int kBidiagPts = 32 * kBidiagCtas;
+constexpr int kBidiagStage = 512;   // squared off-diagonal entries staged at a time
+
+__device__ __forceinline__ double bidiag_point(double lo, double hi, int i) {
+  const float f = (float)(i + 1) / (kBidiagPts + 1);
+  if (!(lo > 0.0)) return hi * (double)f;
+  const float r = (float)(hi / lo);
+  if (r > 1.001f) return lo * (double)exp2f(f * log2f(r));
+  return lo + (hi - lo) * (double)f;
 }
 
-// Extreme singular values of B_k by multisection of the Sturm count (one
-// block: 256 trial points per round for each extreme, the two searched side
-// by side; geometric spacing once the interval is off 0; to 1e-10 relative):
-// out[0] = sigma_max (the point where the count reaches 2k+1), out[1] =
-// sigma_min (where it reaches k+2).  k = 0: zeros.
-__global__ void __launch_bounds__(512) k_bidiag_extremes(const double* __restrict__ gk, int k,
-                                                        double* __restrict__ out) {
-  // two groups of 256 threads, one per extreme: each round every thread
-  // counts at one of 256 points spread geometrically over the group's
-  // interval, and the interval shrinks to the pair of points where the count
-  // crosses the target
-  constexpr int kPts = 256;
-  __shared__ double lam_s[2][kPts];
-  __shared__ int nb_w[16];
-  __shared__ double lo_s[2], hi_s[2];
-  __shared__ int done_s[2];
-  const int g = threadIdx.x / kPts, i = threadIdx.x % kPts;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (k <= 0) {
-    if (threadIdx.x < 2) out[threadIdx.x] = 0.0;
+__global__ void __cluster_dims__(kBidiagCtas, 1, 1) __launch_bounds__(64)
+    k_bidiag_extremes(const double* __restrict__ gk, int k, double* __restrict__ out) {
+  namespace cg = cooperative_groups;
+  __shared__ int cnt[2][2][kBidiagCtas];   // [round parity][extreme][CTA]: points below
+  __shared__ double e2[kBidiagStage];
+  __shared__ double red[2];
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank();
+  const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (k <= 0) {   // the same for the whole cluster
+    if (rank == 0 && threadIdx.x < 2) out[threadIdx.x] = 0.0;
     return;
   }
-  double bound = 0.0, emax2 = 0.0, eprev = 0.0;
-  for (int q = 0; q < 2 * k; ++q) {
+  const int n = 2 * k;   // off-diagonal entries
+  auto entry = [&](int q) -> double {
     const int j = q >> 1;
-    const double e = fabs((q & 1) ? gk[2 * (j + 1) + 1] : gk[2 * j]);
-    bound = fmax(bound, eprev + e);
-    eprev = e;
-    emax2 = fmax(emax2, e * e);
-  }
-  bound = fmax(bound, eprev) * (1.0 + 1e-12) + 1e-300;
-  const double pivmin = 2.2250738585072014e-308 * fmax(1.0, emax2);
+    return fabs((q & 1) ? gk[2 * (j + 1) + 1] : gk[2 * j]);
+  };
+  // ||T|| <= the largest sum of neighbouring entries
+  double bound = 0.0;
+  for (int q = threadIdx.x; q <= n; q += 64)
+    bound = fmax(bound, (q > 0 ? entry(q - 1) : 0.0) + (q < n ? entry(q) : 0.0));
+  for (int o = 16; o > 0; o >>= 1) bound = fmax(bound, __shfl_xor_sync(0xffffffffu, bound, o));
+  if (lane == 0) red[g] = bound;
+  cl.sync();   // and every CTA runs: its shared memory may be written from here on
+  bound = fmax(red[0], red[1]) * (1.0 + 1e-12) + 1e-300;
+  // a power of two >= bound (1 for an infinite bound)
+  const int ex = isfinite(bound) ? ilogb(bound) + 1 : 0;
+  const double up = scalbn(1.0, min(-ex, 1000));
   const int target = g == 0 ? 2 * k + 1 : k + 2;   // sigma_max, sigma_min
-  if (threadIdx.x < 2) {
-    lo_s[threadIdx.x] = 0.0;
-    hi_s[threadIdx.x] = bound;
-    done_s[threadIdx.x] = 0;
-  }
-  __syncthreads();
-  for (int round = 0; round < 200 && !(done_s[0] && done_s[1]); ++round) {
-    const double lo = lo_s[g], hi = hi_s[g];
-    const double f = (double)(i + 1) / (kPts + 1);
-    const double lam = lo > 0.0 ? lo * pow(hi / lo, f) : hi * f;
-    lam_s[g][i] = lam;
-    const bool below = !done_s[g] && gk_sturm_count(gk, k, lam, pivmin) < target;
-    const unsigned m = __ballot_sync(0xffffffffu, below);
-    if (lane == 0) nb_w[warp] = __popc(m);
-    __syncthreads();
-    if (i == 0 && !done_s[g]) {
-      // points 0..nb-1 lie below the crossing; the new interval is [lam_{nb-1}, lam_nb]
-      int nb = 0;
-      for (int w = 0; w < kPts / 32; ++w) nb += nb_w[g * (kPts / 32) + w];
-      double nlo = lo, nhi = hi;
-      if (nb > 0) nlo = lam_s[g][nb - 1];
-      if (nb < kPts) nhi = lam_s[g][nb];
-      lo_s[g] = nlo;
-      hi_s[g] = nhi;
-      done_s[g] = !(nhi > nlo * (1.0 + 1e-10));
+  double lo = 0.0, hi = bound;
+  bool done = false;
+  for (int round = 0; round < 200; ++round) {
+    const double lam = bidiag_point(lo, hi, rank * 32 + lane) * up;
+    double p0 = 0.0, p1 = 1.0;   // p_{-1}, p_0
+    bool neg = false;            // sign of p_i
+    int below = 0;               // eigenvalues below lam
+    for (int q0 = -1; q0 < n; q0 += kBidiagStage) {
+      __syncthreads();
+      for (int q = threadIdx.x; q < kBidiagStage; q += 64) {
+        const double e = q0 + q >= 0 && q0 + q < n ? entry(q0 + q) * up : 0.0;
+        e2[q] = e * e;
+      }
+      __syncthreads();
+      if (done) continue;   // warp-uniform
+      const int m = min(kBidiagStage, n - q0);
+      for (int q = 0; q < m; ++q) {
+        const double p2 = fma(-lam, p1, -(e2[q] * p0));
+        // a zero minor takes the sign that counts one change over the pair
+        const bool s2 = p2 < 0.0 || (p2 == 0.0 && !neg);
+        below += s2 != neg;
+        neg = s2;
+        p0 = p1;
+        p1 = p2;
+        if ((q & 3) == 3) {
+          const int h0 = __double2hiint(p0) & 0x7ff00000, h1 = __double2hiint(p1) & 0x7ff00000;
+          const int he = min(max(max(h0, h1), 0x00100000), 0x7fd00000);
+          const double sc = __hiloint2double(0x7fe00000 - he, 0);
+          p0 *= sc;
+          p1 *= sc;
+        }
+      }
     }
-    __syncthreads();
+    const unsigned bl = __ballot_sync(0xffffffffu, !done && below < target);
+    if (lane < kBidiagCtas) *cl.map_shared_rank(&cnt[round & 1][g][rank], lane) = __popc(bl);
+    cl.sync();
+    if (!done) {
+      int nb = 0;
+      for (int r = 0; r < kBidiagCtas; ++r) nb += cnt[round & 1][g][r];
+      // points 0..nb-1 lie below the crossing: the new interval
+      const double a = nb > 0 ? bidiag_point(lo, hi, nb - 1) : lo;
+      const double b = nb < kBidiagPts ? bidiag_point(lo, hi, nb) : hi;
+      lo = a;
+      hi = b;
+      done = !(hi > lo * (1.0 + 1e-10));
+    }
+    // every CTA sees the same counts, so all of them leave in the same round
+    if (__syncthreads_and(done)) break;
   }
-  if (threadIdx.x < 2) out[threadIdx.x] = 0.5 * (lo_s[threadIdx.x] + hi_s[threadIdx.x]);
+  if (rank == 0 && lane == 0) out[g] = 0.5 * (lo + hi);
+  cl.sync();   // no CTA leaves while another may still write its counts
 }
 
 }  // namespace
 
 void bidiag_extremes(elmfb_ctx* h, const double* gk, int k, double* out2) {
-  k_bidiag_extremes<<<1, 512, 0, h->stream>>>(gk, k, out2);
+  k_bidiag_extremes<<<kBidiagCtas, 64, 0, h->stream>>>(gk, k, out2);
   check_launch("k_bidiag_extremes");
   count_launch(h);
 }

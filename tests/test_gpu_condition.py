@@ -107,3 +107,19 @@ def test_qr_rank_and_r11_match_oracle():
     assert abs(info.rank - rank) <= 1
     assert info.sigma_max == pytest.approx(abs(R[0, 0]), rel=1e-13)
     assert 1e-13 * info.sigma_max < info.sigma_min <= info.sigma_max
+
+
+@pytest.mark.parametrize("k", [1, 255, 256, 300])
+def test_extreme_singular_values_past_one_stage(k):
+    """The count of eigenvalues below a trial point walks the 2k off-diagonal
+    entries 512 at a time: k = 255 and 256 end at and just past the first
+    stage, k = 300 inside the second, k = 1 has a single step.  sigma_max to
+    the search's 1e-10 relative width, sigma_min to 1e-9 as above."""
+    P = _small()
+    with E.Solver.from_problem(P, precision=E.FP64) as s:
+        s.assemble_problem(P)
+        info = s.solve(preconditioner=E.PREC_NONE, max_iter=k, atol=0.0, btol=0.0, check_every=k)
+        al, be = s.bidiagonal()
+    sv = np.linalg.svd(OL.bidiagonal(al[:k], be[:k + 1]), compute_uv=False)
+    assert info.sigma_max == pytest.approx(sv.max(), rel=1e-10)
+    assert info.sigma_min == pytest.approx(sv.min(), rel=1e-9)
