@@ -2,7 +2,8 @@
 
 Each translation unit under ``csrc/`` is compiled by nvcc in parallel and the
 objects are linked into ``paper_2409_01949_gb300/libelmfb.so``.  Objects go to
-``paper_2409_01949_gb300/_build/``.  A unit is recompiled when it or a header
+``paper_2409_01949_gb300/_build/``, the table of the fixed-point tanh
+(``tanh_table.py``) too.  A unit is recompiled when it or a header
 changed after its object.
 """
 from __future__ import annotations
@@ -14,6 +15,8 @@ import shutil
 import subprocess
 import sys
 
+from . import tanh_table
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
@@ -22,7 +25,7 @@ LIB = os.path.join(HERE, "libelmfb.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
-         "-I" + os.path.join(ROOT, "include")]
+         "-I" + os.path.join(ROOT, "include"), "-I" + BUILD]
 
 
 def _nvcc() -> str:
@@ -43,7 +46,10 @@ def build(verbose: bool = False, force: bool = False, extra_flags=()) -> str:
     nvcc = _nvcc()
     os.makedirs(BUILD, exist_ok=True)
     sources = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
-    headers = sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + \
+    table = os.path.join(BUILD, "tanh_table.inc")
+    if _stale(table, [tanh_table.__file__]):
+        tanh_table.write(table)
+    headers = [table] + sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + \
         [os.path.join(ROOT, "include", "elmfb.h")]
     jobs = []
     objs = []
@@ -70,5 +76,5 @@ def build(verbose: bool = False, force: bool = False, extra_flags=()) -> str:
     return LIB
 
 
-if __name__ == "__main__":
+if __name__ == "__main__":   # python -m paper_2409_01949_gb300.build
     print(build(verbose="-v" in sys.argv, force="-f" in sys.argv))

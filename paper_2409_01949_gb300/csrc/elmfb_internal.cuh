@@ -218,6 +218,7 @@ struct elmfb_ctx {
 
   // solution
   DevBuf d_a;           // [NPhi] FP64
+  DevBuf d_eval;        // elmfb_eval's fixed-point columns (workspace)
   bool have_coeffs = false;
 
   // solver work buffers

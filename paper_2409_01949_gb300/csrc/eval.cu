@@ -1,10 +1,11 @@
 // Model evaluation and error norms.
 //
 // u_hat(x) = (1/L) sum_l sum_j w_j(x) sum_k a_ljk phi_ljk(x)   (paper Eq.
-// multilevel_solution), evaluated in FP64: one warp per point.  Lane j forms
-// the window of covering subdomain j, the lanes then share the features of
-// each covering subdomain.  The covering subdomains of a point are
-// those of its cell (the common refinement of all supports).
+// multilevel_solution): one warp per point.  Lane j forms the window of
+// covering subdomain j in FP64, the lanes then share the features of each
+// covering subdomain, in fixed point that is more accurate than FP64
+// (fixed.cuh).  The covering subdomains of a point are those of its cell (the
+// common refinement of all supports).
 //
 // Error norms (paper Eq. l1_error): e_L1 = sum |u_hat - u| / (M std(u)) with
 // the population standard deviation, plus the relative L2 error and the max
@@ -13,8 +14,12 @@
 #include <cmath>
 
 #include "elmfb_internal.cuh"
+#include "fixed.cuh"
+#include "tanh_table.cuh"
 
 namespace {
+
+constexpr double kPiHi = 3.141592653589793116, kPiLo = 1.2246467991473532e-16;   // pi = hi + lo
 
 __device__ __forceinline__ double warp_sum_d(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -145,6 +150,236 @@ __global__ void __launch_bounds__(256) k_eval(const double* __restrict__ xs, int
   if (lane == 0) out[pt] = total / L * ansatz_value(an, x, dim);
 }
 
+// ---- the fixed-point form -------------------------------------------------
+// One column as k_eval_fx reads it: weights, bias and coefficient in fixed
+// point.  The coefficients of a subdomain share an exponent: a = a_fx
+// 2^(ea - 59) with 2^ea above the largest, so that the K terms a_k phi_k are
+// summed as 64-bit integers in units of 2^(ea - 58).
+struct __align__(16) EvalCol {
+  int4 w;    // w0.hi, w0.lo, w1.hi, w1.lo
+  int4 ba;   // bias (low, high word), a.hi, a.lo
+};
+constexpr int kWide = -100000;       // no shared exponent: the subdomain is evaluated in FP64
+constexpr int kNone = kWide + 1;     // all coefficients zero
+
+// Columns of subdomain blockIdx.x in fixed point and their exponent ea, or
+// kWide where a coefficient is not finite or the exponent out of range, kNone
+// where all are zero.
+__global__ void __launch_bounds__(128) k_eval_pack(const double* __restrict__ W,
+                                                   const double* __restrict__ B,
+                                                   const double* __restrict__ a, int dim, int K,
+                                                   int wexp, EvalCol* __restrict__ cols,
+                                                   int* __restrict__ expo) {
+  __shared__ double red[4];
+  const int64_t q0 = (int64_t)blockIdx.x * K;
+  double mx = 0.0;
+  bool bad = false;
+  for (int f = threadIdx.x; f < K; f += blockDim.x) {
+    const double v = fabs(a[q0 + f]);
+    bad |= !(v <= 1.7976931348623157e308);
+    mx = fmax(mx, v);
+  }
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+  bad = __syncthreads_or(bad);
+  mx = fmax(fmax(red[0], red[1]), fmax(red[2], red[3]));
+  const int ea = mx > 0.0 ? ilogb(mx) + 1 : 0;
+  bad |= ea < -900 || ea > 900;
+  if (threadIdx.x == 0) expo[blockIdx.x] = bad ? kWide : (mx > 0.0 ? ea : kNone);
+  const double ws = scalbn(1.0, 61 - wexp), bs = scalbn(1.0, 60 - wexp);
+  const double as = bad ? 0.0 : scalbn(1.0, 59 - ea);
+  for (int f = threadIdx.x; f < K; f += blockDim.x) {
+    const int64_t q = q0 + f;
+    const fx::Val w0 = fx::split(__double2ll_rn(W[q * dim] * ws));
+    const fx::Val w1 = fx::split(dim == 2 ? __double2ll_rn(W[q * dim + 1] * ws) : 0ll);
+    const int64_t b = __double2ll_rn(B[q] * bs);
+    const fx::Val av = fx::split(bad ? 0ll : __double2ll_rn(a[q] * as));
+    cols[q].w = make_int4(w0.hi, w0.lo, w1.hi, w1.lo);
+    cols[q].ba = make_int4((int)(uint32_t)b, (int)(b >> 32), av.hi, av.lo);
+  }
+}
+
+// 1-D window factor 4 cos^4(pi x / 2) at x = xh + xl, |x| < 1, to within a unit
+// in the last place: the terms of u_hat are summed without rounding, so the
+// windows are what its accuracy comes down to.  With u = 1 - |x|, cos(pi x / 2)
+// is sin(pi u / 2) near the edge, else 1 - 2 sin^2(pi x / 4); the sine by its
+// Taylor polynomial (|argument| <= pi / 4, next term below 2^-63), sine, cosine
+// and its square as sums hi + lo.
+__device__ __forceinline__ double window_factor64(double xh, double xl) {
+  const double ax = fabs(xh);
+  const double u = (1.0 - ax) - (xh < 0.0 ? -xl : xl);
+  const bool edge = u < 0.5;
+  const double v = edge ? 0.5 * u : 0.25 * ax;   // xl is below v's last place there
+  const double x = v * kPiHi, z = x * x;
+  double p = 2.8114572543455206e-15;          // 1 / 17!
+  p = fma(p, z, -7.6471637318198164e-13);     // -1 / 15!
+  p = fma(p, z, 1.6059043836821613e-10);      // 1 / 13!
+  p = fma(p, z, -2.5052108385441720e-08);     // -1 / 11!
+  p = fma(p, z, 2.7557319223985893e-06);      // 1 / 9!
+  p = fma(p, z, -1.9841269841269841e-04);     // -1 / 7!
+  p = fma(p, z, 8.3333333333333332e-03);      // 1 / 5!
+  p = fma(p, z, -1.6666666666666666e-01);     // -1 / 3!
+  // what x's rounding left out, pi's low part included
+  const double t = fma(x * z, p, fma(v, kPiLo, fma(v, kPiHi, -x)));
+  double ch = x + t, cl = t - (ch - x);
+  if (!edge) {
+    const double s = ch;
+    ch = fma(-2.0 * s, s, 1.0);
+    cl = fma(-2.0 * s, s, 1.0 - ch) - 4.0 * s * cl;
+  }
+  const double c2 = ch * ch, c2l = fma(ch, ch, -c2) + 2.0 * ch * cl;
+  const double c4 = c2 * c2, c4l = fma(c2, c2, -c4) + 2.0 * c2 * c2l;
+  return 4.0 * (c4 + c4l);
+}
+
+// a number that orders as the double does
+__device__ __forceinline__ int64_t order_key(double v) {
+  const int64_t b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+
+// Warp per point, as k_eval's m <= 32 form (every cell's covering subdomains
+// fit a warp).  Terms and their sums are integers; per point and lane about 100
+// FP64 instructions remain (the windows, their partition of unity and the
+// final sum), which the FP64 pipe issues in 6400 cycles of a sub-partition
+// beside the integer pipes' work: 130 instructions a term, a third of them
+// multiply-adds, and three 16-byte table loads.  The FP64 form spent 3200
+// cycles of a sub-partition on a warp of terms, almost all in tanh: 262144
+// points of a 7-level 2-D model with K = 64 took 31.2 ms and take 3.15 ms, 1000
+// points of a 1-D model 45 us and 29 us (the whole call); the error against a
+// 113-bit evaluation is the same, 2.3e-16 of the result in the mean (the
+// windows' part of it).
+template <bool kTwo>
+__global__ void __launch_bounds__(256) k_eval_fx(
+    const double* __restrict__ xs, int64_t n, int K, int L, const double* __restrict__ bnd,
+    int nc0, int nc1, const SubGeom* __restrict__ sub, const int* __restrict__ cell_level_off,
+    const int* __restrict__ cover_sub, const EvalCol* __restrict__ cols,
+    const int* __restrict__ expo, int shift, int rows, int room, const double* __restrict__ W,
+    const double* __restrict__ B, const double* __restrict__ a, double* __restrict__ out,
+    const Ansatz an) {
+  constexpr int dim = kTwo ? 2 : 1;
+  extern __shared__ __align__(16) int4 tab[];
+  for (int i = threadIdx.x; i < 3 * rows; i += blockDim.x) tab[i] = kTanhTable[i];
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const int64_t pt = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (pt >= n) return;
+  const double x[2] = {xs[pt * dim], kTwo ? xs[pt * dim + 1] : 0.0};
+  int cell = 0;
+  {
+    const double* bb = bnd;
+    int stride = 1;
+#pragma unroll
+    for (int i = 0; i < dim; ++i) {
+      const int nc = i == 0 ? nc0 : nc1;
+      const int64_t key = order_key(x[i]);   // integer comparisons: the FP64 pipe is the busy one
+      int lo = 0, hi = nc;
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (order_key(bb[mid]) <= key) lo = mid;
+        else hi = mid;
+      }
+      cell += lo * stride;
+      stride = nc0;
+      bb += nc + 1;
+    }
+  }
+  const int* lo_l = cell_level_off + (int64_t)cell * (L + 1);
+  const int e0 = lo_l[0], m = lo_l[L] - e0;
+  // lane j: covering entry e0 + j, its window factor and scaled input
+  double wj = 0.0, xd[2] = {0.0, 0.0}, xl[2] = {0.0, 0.0};
+  int sj = 0, gb = 0, ge = 0, ea = 0;   // its level's entries gb .. ge - 1
+  if (lane < m) {
+    sj = cover_sub[e0 + lane];
+    const SubGeom g = sub[sj];
+    gb = lo_l[g.level] - e0;
+    ge = lo_l[g.level + 1] - e0;
+    ea = expo[sj];
+    wj = 1.0;
+#pragma unroll
+    for (int i = 0; i < dim; ++i) {
+      // dx / sigma = xd + xl
+      const double dx = x[i] - g.mu[i];
+      xd[i] = dx * g.inv_sigma_d[i];
+      xl[i] = fma(-xd[i], g.sigma_d[i], dx) * g.inv_sigma_d[i];
+      wj *= fabs(dx) < g.sigma_d[i] ? window_factor64(xd[i], xl[i]) : 0.0;
+    }
+  }
+  // partition of unity: the sum over the level's entries, which are
+  // neighbouring lanes (each lane reads its own level's)
+  double S = 0.0;
+  const int len = __reduce_max_sync(0xffffffffu, ge - gb);
+  for (int k = 0; k < len; ++k) {
+    const double v = __shfl_sync(0xffffffffu, wj, min(gb + k, 31));
+    if (gb + k < ge) S += v;
+  }
+  const double cw = S > 0.0 && wj != 0.0 ? wj / (S * L) : 0.0;
+  const fx::Val x0 = fx::split(__double2ll_rn(xd[0] * 0x1p61) + __double2ll_rn(xl[0] * 0x1p61));
+  const fx::Val x1 =
+      fx::split(kTwo ? __double2ll_rn(xd[1] * 0x1p61) + __double2ll_rn(xl[1] * 0x1p61) : 0ll);
+  // cw = cm 2^(ec - 61), cm in [2^60, 2^61): an entry's sum times cm has the
+  // exponent ea + ec, and all are aligned to the largest of the point, `room`
+  // bits lower so that they cannot overflow
+  const int64_t cb = __double_as_longlong(cw);
+  const int ex = (int)(cb >> 52);
+  const fx::Val cm = fx::split(((cb & 0xfffffffffffffll) | 0x10000000000000ll) << 8);
+  const bool is_wide = cw != 0.0 && ea == kWide;
+  const bool is_live = ex > 0 && ea > kNone;
+  const int en = is_live ? ea + ex - 1022 : kWide;
+  const int emax = __reduce_max_sync(0xffffffffu, en);
+  const int down = min(emax - en + room, 62);
+  const unsigned live = __ballot_sync(0xffffffffu, is_live);
+  const unsigned wide = __ballot_sync(0xffffffffu, is_wide);
+  int64_t acc = 0;
+  for (int j = 0; j < m; ++j) {
+    if (!((live >> j) & 1u)) continue;
+    const int s = __shfl_sync(0xffffffffu, sj, j);
+    const fx::Val y0 = {__shfl_sync(0xffffffffu, x0.hi, j), __shfl_sync(0xffffffffu, x0.lo, j)};
+    fx::Val y1 = {0, 0};
+    if (kTwo)
+      y1 = {__shfl_sync(0xffffffffu, x1.hi, j), __shfl_sync(0xffffffffu, x1.lo, j)};
+    const EvalCol* col = cols + (int64_t)s * K;
+    int64_t sum = 0;
+#pragma unroll 2
+    for (int f = lane; f < K; f += 32) {
+      const int4 w = col[f].w, ba = col[f].ba;
+      const int64_t b = (int64_t)(((uint64_t)(uint32_t)ba.y << 32) | (uint32_t)ba.x);
+      const int64_t arg = fx::argument({w.x, w.y}, y0, {w.z, w.w}, y1, b, kTwo);
+      sum = fx::mul_add({ba.z, ba.w}, fx::split(fx::tanh61(arg, shift, tab, rows)), sum);
+    }
+    const fx::Val c = {__shfl_sync(0xffffffffu, cm.hi, j), __shfl_sync(0xffffffffu, cm.lo, j)};
+    const int d = __shfl_sync(0xffffffffu, down, j);
+    acc += (fx::mul_add(fx::split(sum), c, 0) + (((int64_t)1 << d) >> 1)) >> d;   // to nearest
+  }
+  double part = live ? (double)acc * scalbn(1.0, emax - 57 + room) : 0.0;
+  if (wide) {   // subdomains whose coefficients have no shared exponent
+    for (int j = 0; j < m; ++j) {
+      if (!((wide >> j) & 1u)) continue;
+      const int s = __shfl_sync(0xffffffffu, sj, j);
+      const double c = __shfl_sync(0xffffffffu, cw, j);
+      const double y0 = __shfl_sync(0xffffffffu, xd[0], j);
+      const double y1 = __shfl_sync(0xffffffffu, xd[1], j);
+      for (int f = lane; f < K; f += 32) {
+        const int64_t q = (int64_t)s * K + f;
+        const double arg = W[q * dim] * y0 + (kTwo ? W[q * dim + 1] * y1 : 0.0) + B[q];
+        part += c * (a[q] * tanh(arg));
+      }
+    }
+  }
+  const double total = warp_sum_d(part);
+  if (lane == 0) out[pt] = total * ansatz_value(an, x, dim);
+}
+
+// Bits to keep free below the aligned sums: a term is below 2^58 units, so an
+// entry's K / 32 terms a lane times cm / 2^62 below (K / 32) 2^57, and m
+// entries add up.
+int eval_room(int K, int m) {
+  const int64_t terms = ceil_div(K, 32) * m;
+  int room = 0;
+  while ((int64_t)64 << room < terms) ++room;
+  return room;
+}
+
 // pass 1: sum u, sum |d|, sum d^2, sum u^2, max |d|  (per block)
 __global__ void k_err_pass1(const double* __restrict__ uh, const double* __restrict__ ur,
                             int64_t n, double* __restrict__ part) {
@@ -204,23 +439,78 @@ __global__ void k_err_pass2(const double* __restrict__ ur, int64_t n,
 
 }  // namespace
 
+// p lies in this device's own memory and is aligned, so that a kernel may use
+// it in place
+static bool in_place(const elmfb_ctx* h, const void* p, size_t align) {
+  if ((uintptr_t)p % align != 0) return false;
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == h->device;
+}
+
 void eval_model(elmfb_ctx* h, const double* xs, int64_t n, double* out) {
   if (n == 0) return;
   cudaStream_t st = h->stream;
   stage_begin(h, 6);
+  // points and results in device memory are used where they are (unless they
+  // overlap), others staged
+  const size_t xb = n * h->dim * sizeof(double), ob = n * sizeof(double);
+  const char *x0 = (const char*)xs, *o0 = (const char*)out;
+  const bool apart = x0 + xb <= o0 || o0 + ob <= x0;
   DevBuf dx, dout;
-  dx.alloc(n * h->dim * sizeof(double), st);
-  dout.alloc(n * sizeof(double), st);
-  CUDA_CHECK(cudaMemcpyAsync(dx.p, xs, n * h->dim * sizeof(double), cudaMemcpyDefault, st));
-  const int64_t threads = n * 32;
-  k_eval<<<(unsigned)ceil_div(threads, 256), 256, 0, st>>>(
-      dx.as<double>(), n, h->dim, h->K, h->L, h->d_bnd.as<double>(), h->nc[0], h->nc[1],
-      h->d_sub.as<SubGeom>(), h->d_cell_level_off.as<int>(), h->d_cover_sub.as<int>(),
-      h->d_W64.as<double>(), h->d_b64.as<double>(), h->d_a.as<double>(), dout.as<double>(),
-      make_ansatz(h->cfg));
-  check_launch("k_eval");
-  count_launch(h);
-  CUDA_CHECK(cudaMemcpyAsync(out, dout.p, n * sizeof(double), cudaMemcpyDefault, st));
+  const double* x = xs;
+  double* o = out;
+  if (!apart || !in_place(h, xs, sizeof(double))) {
+    dx.alloc(xb, st);
+    CUDA_CHECK(cudaMemcpyAsync(dx.p, xs, xb, cudaMemcpyDefault, st));
+    x = dx.as<double>();
+  }
+  if (!apart || !in_place(h, out, sizeof(double))) {
+    dout.alloc(ob, st);
+    o = dout.as<double>();
+  }
+  // Fixed point wherever a point's covering subdomains fit a warp and the
+  // weight scale is in its range (fixed.cuh); FP64 otherwise: below the range
+  // FP64's error, relative to the small arguments, is the smaller one.
+  const double a = h->cfg.weight_scale;
+  const int wexp = a > 0.0 ? fx::weight_exp(a) : fx::kMinExp - 1;
+  if (h->max_cover <= 32 && wexp >= fx::kMinExp && wexp <= fx::kMaxExp) {
+    const int rows = fx::tanh_rows(h->dim, wexp);
+    const size_t smem = (size_t)rows * 3 * sizeof(int4);
+    // columns, then exponents: a workspace of the handle, rewritten on each call
+    h->d_eval.alloc((size_t)h->NPhi * sizeof(EvalCol) + (size_t)h->n_sub * sizeof(int), st);
+    EvalCol* const cols = h->d_eval.as<EvalCol>();
+    int* const expo = reinterpret_cast<int*>(cols + h->NPhi);
+    k_eval_pack<<<(unsigned)h->n_sub, 128, 0, st>>>(
+        h->d_W64.as<double>(), h->d_b64.as<double>(), h->d_a.as<double>(), h->dim, h->K, wexp,
+        cols, expo);
+    // few points: half-size blocks, so that they spread over more SMs
+    const int threads = n < 152 * 16 ? 128 : 256;
+#define ELMFB_EVAL_FX(TWO)                                                                     \
+  k_eval_fx<TWO><<<(unsigned)ceil_div(n * 32, threads), threads, smem, st>>>(                  \
+      x, n, h->K, h->L, h->d_bnd.as<double>(), h->nc[0], h->nc[1], h->d_sub.as<SubGeom>(),     \
+      h->d_cell_level_off.as<int>(), h->d_cover_sub.as<int>(), cols, expo, 55 - wexp, rows,    \
+      eval_room(h->K, h->max_cover), h->d_W64.as<double>(), h->d_b64.as<double>(),      \
+      h->d_a.as<double>(), o, make_ansatz(h->cfg))
+    if (h->dim == 2) ELMFB_EVAL_FX(true);
+    else ELMFB_EVAL_FX(false);
+#undef ELMFB_EVAL_FX
+    check_launch("k_eval_fx");
+    count_launch(h, 2);
+  } else {
+    const int64_t threads = n * 32;
+    k_eval<<<(unsigned)ceil_div(threads, 256), 256, 0, st>>>(
+        x, n, h->dim, h->K, h->L, h->d_bnd.as<double>(), h->nc[0], h->nc[1],
+        h->d_sub.as<SubGeom>(), h->d_cell_level_off.as<int>(), h->d_cover_sub.as<int>(),
+        h->d_W64.as<double>(), h->d_b64.as<double>(), h->d_a.as<double>(), o,
+        make_ansatz(h->cfg));
+    check_launch("k_eval");
+    count_launch(h);
+  }
+  if (dout.p) CUDA_CHECK(cudaMemcpyAsync(out, dout.p, ob, cudaMemcpyDefault, st));
   stage_end(h, 6);
 }
 

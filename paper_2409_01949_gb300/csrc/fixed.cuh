@@ -1,0 +1,100 @@
+// Fixed-point arithmetic of the FP64-accurate feature evaluation.
+//
+// GB300 issues an FP64 warp instruction over 64 cycles of a sub-partition, a
+// 32 x 32 + 64 bit integer multiply-add over a few, so a tanh in FP64 (about
+// 50 such instructions with its argument) costs about 3000 cycles a warp and
+// the integer form below about 200.  Every quantity of a feature is bounded
+// (|x| <= 1 in a support, |w|, |b| <= the weight scale, |tanh| <= 1), so 62-bit
+// fixed point loses nothing: the absolute error of the tanh is below 2^-57
+// (2^-60 in the mean square), its argument's below 2^-59 times the weight scale (rounded up to a power of
+// two), against 2^-54 and 2^-53 times the argument's terms in FP64.
+//
+// A value v is held as v = hi 2^31 + lo, 0 <= lo < 2^31, so that every partial
+// product is one signed multiply-add; the lo x lo product (less than one unit
+// after the shift) is left out.
+#pragma once
+
+#include <math.h>
+#include <stdint.h>
+
+#if defined(__CUDACC__)
+#define FX_FN __host__ __device__ __forceinline__
+#else
+#define FX_FN inline
+struct int4 { int x, y, z, w; };
+struct int2 { int x, y; };
+#endif
+
+namespace fx {
+
+struct Val {
+  int hi, lo;
+};
+
+FX_FN Val split(int64_t v) { return {(int)(v >> 31), (int)(v & 0x7fffffff)}; }
+
+// c + a b / 2^62, to the nearest unit (but for the lo x lo product): rounding
+// down would put half a unit of the same sign on every one of the thousands of
+// terms of a sum
+FX_FN int64_t mul_add(Val a, Val b, int64_t c) {
+  const int64_t cross = (int64_t)a.hi * b.lo + ((int64_t)a.lo * b.hi + (1 << 30));
+  return (int64_t)a.hi * b.hi + c + (cross >> 31);
+}
+
+// The weight scale a as a power of two: weights and biases are at most
+// 2^wexp(a) in magnitude.  Fixed point is used for kMinExp <= wexp <= kMaxExp:
+// below, FP64's error (relative to its terms) is the smaller one; above, the
+// interval index would run out of bits.
+constexpr int kMinExp = -4, kMaxExp = 16;
+
+// wexp(a), the least e with a <= 2^e (a > 0)
+FX_FN int weight_exp(double a) {
+  int e;
+  const double m = frexp(a, &e);
+  return m == 0.5 ? e - 1 : e;
+}
+
+// A feature's argument s = w0 x0 + w1 x1 + b with w in units of 2^(wexp - 61),
+// x in units of 2^-61 and b in units of 2^(wexp - 60); s has b's unit and at
+// most three terms, so it stays below 2^62.
+FX_FN int64_t argument(Val w0, Val x0, Val w1, Val x1, int64_t b, bool two) {
+  int64_t cross = (int64_t)w0.hi * x0.lo + ((int64_t)w0.lo * x0.hi + (1 << 30));
+  int64_t s = (int64_t)w0.hi * x0.hi + b;
+  if (two) {
+    cross += (int64_t)w1.hi * x1.lo + (int64_t)w1.lo * x1.hi;
+    s += (int64_t)w1.hi * x1.hi;
+  }
+  return s + (cross >> 31);
+}
+
+// tanh(s) in units of 2^-61, s in units of 2^(wexp - 60); `shift` = 55 - wexp is
+// the width of an interval of 1/32.  tab holds `rows` rows of the table
+// (tanh_table.py), the last of them for everything past the others.
+FX_FN int64_t tanh61(int64_t s, int shift, const int4* tab, int rows) {
+  const uint64_t m = (uint64_t)(s < 0 ? -s : s);
+  const uint64_t j64 = m >> shift;
+  const int j = j64 < (uint64_t)rows ? (int)j64 : rows - 1;
+  // the place in the interval as r in [-1, 1), units of 2^-62
+  const Val r = split((int64_t)((m << (64 - shift)) >> 1) - ((int64_t)1 << 62));
+  const int4 a = tab[3 * j], b = tab[3 * j + 1], d = tab[3 * j + 2];
+  auto word = [](int lo, int hi) { return (int64_t)(((uint64_t)(uint32_t)hi << 32) | (uint32_t)lo); };
+  // the upper coefficients fit 32 bits, and the high half of r is enough
+  int t = (int)(((int64_t)(d.y >> 16) * r.hi) >> 31) + d.w;   // c7 r + c6
+  t = (int)(((int64_t)t * r.hi) >> 31) + d.z;                 // ... r + c5
+  int64_t v = (((int64_t)t * r.hi) >> 31) + word(d.x, (int)(short)d.y);   // ... + c4
+  v = mul_add(split(v), r, word(b.z, b.w));
+  v = mul_add(split(v), r, word(b.x, b.y));
+  v = mul_add(split(v), r, word(a.z, a.w));
+  v = mul_add(split(v), r, word(a.x, a.y));
+  return s < 0 ? -v : v;
+}
+
+constexpr int kTanhRows = 32 * 22 + 1;   // tanh_table.py: 32 a unit up to 22, and the closing row
+
+// rows that arguments up to (dim + 1) 2^wexp reach, the closing row included
+FX_FN int tanh_rows(int dim, int wexp) {
+  const int64_t n = wexp >= 0 ? (int64_t)(dim + 1) * 32 << wexp : ((int64_t)(dim + 1) * 32 >> -wexp) + 1;
+  return n + 1 < kTanhRows ? (int)n + 1 : kTanhRows;
+}
+
+}  // namespace fx

@@ -1,0 +1,116 @@
+"""Model evaluation: the fixed-point kernel and the FP64 one it replaces where
+a point's covering subdomains fit a warp and the weight scale is in range.
+
+Tolerance, against the oracle's FP64 evaluation: the windows of a level sum to
+1 and |tanh| <= 1, so the terms of u_hat add up to at most S = max_j ||a_j||_1
+per level; either side rounds the argument (dim + 1 terms of at most the
+weight scale a, plus the scaled coordinate, whose centre subtraction carries
+2^-53 / sigma <= 2^-53 n / 1 of the box) and a few products, 16 of them in all:
+|difference| <= 16 2^-53 S (1 + (dim + 1) a n_max).
+"""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+import paper_2409_01949_gb300 as E
+import workloads as WL
+from oracle import evaluate as OE
+
+pytestmark = pytest.mark.gpu
+
+
+def _problem(dim, levels, K, scale, **kw):
+    f = WL.poisson1d if dim == 1 else WL.poisson2d
+    return f(levels=levels, features=K, weight_scale=scale, **kw)
+
+
+def _points(P, n, seed=3):
+    """Random points, then support edges, centres and corners."""
+    r = np.random.default_rng(seed)
+    x = r.random((n, P.dim))
+    nl = P.levels[-1]
+    special = np.array([0.0, 1.0, 0.5, 0.5 / nl, 1.5 / nl, 1.0 / nl, 1.0 - 0.5 / nl])
+    m = min(n, special.size)
+    x[:m, 0] = np.clip(special[:m], 0.0, 1.0)
+    return x
+
+
+def _tol(P, a):
+    S = np.abs(a).reshape(-1, P.features).sum(axis=1).max()
+    return 16 * 2.0 ** -53 * S * (1 + (P.dim + 1) * P.weight_scale * max(P.levels))
+
+
+# weight scales: 1/16 and 2^16 are the ends of the fixed-point range, 0.06 and
+# 70000 just outside it (FP64), 0.3 and 5 not powers of two; K past 32 and
+# multiples of it; 40 covering subdomains (delta = 2.9, five levels of nine)
+# do not fit a warp
+@pytest.mark.parametrize("dim,levels,K,scale,delta,n", [
+    (1, (1,), 1, 1.0, 2.0, 1), (1, (16,), 64, 1.0, 2.0, 1000), (1, (1, 2, 4, 8), 33, 0.3, 2.9, 77),
+    (1, (5,), 256, 1.0 / 16, 1.5, 9), (1, (8,), 32, 0.06, 2.0, 50), (1, (8,), 40, 5.0, 2.0, 50),
+    (1, (4,), 16, 65536.0, 2.0, 200), (1, (4,), 16, 70000.0, 2.0, 50),
+    (2, (1, 2, 4), 128, 1.0, 2.0, 333), (2, (3,), 100, 2.0, 2.9, 64), (2, (1, 2, 4, 8, 16), 31, 1.0, 2.0, 2500),
+    (2, (3, 4, 5, 6, 7), 8, 1.0, 2.9, 40),
+])
+def test_eval_matches_oracle(dim, levels, K, scale, delta, n):
+    P = _problem(dim, levels, K, scale, delta=delta)
+    rng = np.random.default_rng(1)
+    a = rng.standard_normal(P.n_columns) * 10.0 ** rng.uniform(-3, 3, P.n_columns)
+    X = _points(P, n)
+    with E.Solver.from_problem(P) as s:
+        s.set_coeffs(a)
+        u = s.eval(X)
+    assert np.abs(u - OE.u_hat(P, a, X)).max() <= _tol(P, a)
+
+
+def test_coefficients_outside_the_fixed_point_range():
+    """A subdomain whose coefficients are too large for a shared exponent, or
+    not finite, is evaluated in FP64: points it does not cover keep their
+    values, points it covers see what FP64 gives."""
+    P = _problem(1, (8,), 32, 1.0)
+    rng = np.random.default_rng(2)
+    a = rng.standard_normal(P.n_columns)
+    X = np.linspace(0.01, 0.99, 57)[:, None]
+    ref = OE.u_hat(P, a, X)
+    with E.Solver.from_problem(P) as s:
+        for v in (1e300, 1e-300, np.inf, np.nan):
+            b = a.copy()
+            b[5 * 32 + 3] = v           # subdomain 5 covers (4.5/8, 6.5/8)
+            s.set_coeffs(b)
+            u = s.eval(X)
+            inside = np.abs(X[:, 0] - 5.5 / 8) < 1.0 / 8
+            assert np.abs(u[~inside] - ref[~inside]).max() <= _tol(P, a)
+            if np.isfinite(v):
+                assert np.abs(u - OE.u_hat(P, b, X)).max() <= _tol(P, b)
+            else:
+                assert not np.isfinite(u[inside]).any()
+        s.set_coeffs(np.zeros_like(a))
+        assert np.all(s.eval(X) == 0.0)
+        # a subdomain of zeros sets no exponent for neighbours of tiny coefficients
+        b = 1e-40 * a
+        b[5 * 32:6 * 32] = 0.0
+        s.set_coeffs(b)
+        assert np.abs(s.eval(X) - OE.u_hat(P, b, X)).max() <= _tol(P, b)
+
+
+def test_points_and_results_in_place_overlapping_or_unaligned():
+    """Device buffers are used where they are; overlapping ones and ones not
+    aligned to doubles are staged.  All give the values of host arrays."""
+    import torch
+    P = _problem(1, (4, 8), 24, 1.0)
+    a = np.random.default_rng(4).standard_normal(P.n_columns)
+    X = _points(P, 301)
+    with E.Solver.from_problem(P) as s:
+        s.set_coeffs(a)
+        ref = s.eval(X)
+        x = torch.from_numpy(X).cuda()
+        assert np.array_equal(s.eval(x, torch.empty(301, dtype=torch.float64, device="cuda")).cpu().numpy(), ref)
+        buf = torch.zeros(302, dtype=torch.float64, device="cuda")
+        buf[:301] = x[:, 0]
+        torch.cuda.synchronize()
+        L = E.lib()
+        assert L.elmfb_eval(s.h, C.c_void_p(buf.data_ptr()), 301, C.c_void_p(buf.data_ptr() + 8)) == E.OK
+        assert np.array_equal(buf[1:].cpu().numpy(), ref)
+        raw = torch.zeros(301 * 8 + 4, dtype=torch.uint8, device="cuda")
+        assert L.elmfb_eval(s.h, C.c_void_p(x.data_ptr()), 301, C.c_void_p(raw.data_ptr() + 4)) == E.OK
+        assert np.array_equal(raw[4:].cpu().numpy().tobytes(), ref.tobytes())
