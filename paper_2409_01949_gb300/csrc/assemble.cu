@@ -15,7 +15,8 @@
 // subdomains, and its row offset inside each of their panels, then follow from
 // its cell alone.
 //
-// K1 evaluates the operator analytically.  With t = 1 - phi^2 and
+// K1 evaluates the operator analytically (k_assemble; FP64-accurate entries at
+// the usual weight scales in fixed point, k_assemble_fx).  With t = 1 - phi^2 and
 // d_i = w_i / sigma_i (= d s / d x_i),
 //     d_i phi = t d_i,    d_ii phi = -2 phi t d_i^2,
 // and the product rule of Op[w phi] collects into
@@ -35,12 +36,15 @@
 // tanh is formed from expm1: e = expm1(2|s|), phi = sign(s) e/(e+2) and
 // 1 - phi^2 = 4 (e+1)/(e+2)^2, free of cancellation for every s.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <numeric>
 
 #include <cuda_bf16.h>
 
 #include "elmfb_internal.cuh"
+#include "fixed.cuh"
+#include "tanh_table.cuh"
 
 namespace {
 
@@ -538,6 +542,368 @@ __global__ void __launch_bounds__(128) k_assemble(
   }
 }
 
+// The entry of one feature in FP64 for the rows that the fixed-point form does
+// not take (terms that are not finite, or so large or small that an exponent
+// could leave the double's range).
+__device__ __noinline__ double entry64(double w0, double w1, double b, double x0, double x1,
+                                       double is0, double is1, double A, double be0, double be1,
+                                       double ga0, double ga1) {
+  double phi, t;
+  tanh_pair<double>(w0 * x0 + w1 * x1 + b, &phi, &t);
+  const double d0 = w0 * is0, d1 = w1 * is1;
+  const double B = be0 * d0 + be1 * d1;
+  const double C = ga0 * (d0 * d0) + ga1 * (d1 * d1);
+  return t * (B - 2.0 * phi * C) + phi * A;
+}
+
+// K1 for FP64 entries and FP32 pairs (kSplit) in fixed point (fixed.cuh): phase
+// 1 as k_assemble, in FP64; phase 2 in integers.  A row's terms share an
+// exponent er, 2^er above the largest of |A|, |beta_i w / sigma_i|, 2 |gamma_i
+// (w / sigma_i)^2| over |w| <= 2^wexp, and become
+//     M = phi A + (1 - phi^2) D = D + phi (A - phi D),  D = B - phi C,
+//     B = sum beta_i u_i,  C = sum 2 gamma_i u_i^2,  u = w / 2^wexp,
+// in units of 2^(er - 59): every term of a row is held to
+// 2^-59 of the row's largest, where FP64 rounds each operation to 2^-53 of its
+// result.  The sum is rounded once, to a double or to an FP32 pair.
+//
+// The FP64 form is bound by the FP64 pipe (47 instructions an entry, 3020
+// cycles of a sub-partition for a warp's 32 entries); this one by integer issue
+// (ncu: 50% issue-active, the multiply-add pipe 51%), with phase 1's FP64 work
+// beside it.  400^2 points, levels 1..16, K = 128: assembly and one LSQR step
+// 29.5 -> 10.1 ms; the oscillator (20000 points, levels 1..64, K = 96, pairs),
+// four LSQR steps: 4.18 -> 1.63 ms.  Entries against a 113-bit evaluation: 1.5e-16
+// -> 0.9e-16 of the system's norm in FP64, the pairs' 48 bits as before.
+//
+// 1-D window factor f = 4 c^4 with (s, c) = sincos(pi x / 2), x = dx / sigma, its
+// derivatives (file header), and x in units of 2^-61.  Sine and cosine come
+// from one argument y <= pi / 4 -- pi u / 2 with u = 1 - |x| near the edge, else
+// pi |x| / 2 -- by their Taylor polynomials (next terms below 2^-58 of 1), with
+// x = xh + xl carried beyond FP64, so that no branch is taken twice.
+__device__ __forceinline__ void window_axis(double dx, double sigma, double inv, double& f,
+                                            double& fp, double& fpp, int64_t& x61) {
+  const double xh = dx * inv, xl = fma(-xh, sigma, dx) * inv;
+  x61 = __double2ll_rn(xh * 0x1p61) + __double2ll_rn(xl * 0x1p61);
+  f = fp = fpp = 0.0;
+  if (!(fabs(dx) < sigma)) return;
+  const double u = (1.0 - fabs(xh)) - (xh < 0.0 ? -xl : xl);
+  const bool edge = u < 0.5;
+  const double v = 0.5 * (edge ? u : fabs(xh));
+  const double y = v * kPiD, z = y * y;
+  const double yl = fma(v, 1.2246467991473532e-16, fma(v, kPiD, -y));   // pi v - y
+  double p = 2.8114572543455206e-15;          // 1 / 17!
+  p = fma(p, z, -7.6471637318198164e-13);     // -1 / 15!
+  p = fma(p, z, 1.6059043836821613e-10);      // 1 / 13!
+  p = fma(p, z, -2.5052108385441720e-08);     // -1 / 11!
+  p = fma(p, z, 2.7557319223985893e-06);      // 1 / 9!
+  p = fma(p, z, -1.9841269841269841e-04);     // -1 / 7!
+  p = fma(p, z, 8.3333333333333332e-03);      // 1 / 5!
+  p = fma(p, z, -1.6666666666666666e-01);     // -1 / 3!
+  const double sy = y + fma(y * z, p, yl);
+  double q = 4.7794773323873853e-14;          // 1 / 16!
+  q = fma(q, z, -1.1470745597729725e-11);     // -1 / 14!
+  q = fma(q, z, 2.0876756987868099e-09);      // 1 / 12!
+  q = fma(q, z, -2.7557319223985888e-07);     // -1 / 10!
+  q = fma(q, z, 2.4801587301587302e-05);      // 1 / 8!
+  q = fma(q, z, -1.3888888888888889e-03);     // -1 / 6!
+  q = fma(q, z, 4.1666666666666664e-02);      // 1 / 4!
+  const double cy = 1.0 + (fma(q * z, z, -y * yl) - 0.5 * z);
+  const double c = edge ? sy : cy, s = edge ? cy : sy;
+  const double g = kPiD * inv, c2 = c * c;
+  f = 4.0 * c2 * c2;
+  fp = -8.0 * (c2 * g) * (c * (dx < 0.0 ? -s : s));
+  fpp = 4.0 * c2 * (3.0 - 4.0 * c2) * g * g;   // 3 s^2 - c^2, s^2 = 1 - c^2
+}
+
+struct RowTerms {   // one row of phase 2, as four 16-byte words
+  int4 a;    // A59.hi, A59.lo, er (kRow64: in FP64), -
+  int4 b;    // beta'' of axis 0 (hi, lo), axis 1
+  int4 c;    // 2 gamma'' of axis 0, axis 1
+  int4 x;    // scaled coordinates
+};
+constexpr int kRow64 = INT_MIN;
+
+constexpr int kFxFeatures = 2;   // a lane's features of one pass over a panel's rows
+
+template <bool kSplit, bool kTwo>
+__global__ void __launch_bounds__(64, 8) k_assemble_fx(
+    const int4* __restrict__ tiles, int64_t n_tiles, int K, int nl_max,
+    const SubGeom* __restrict__ sub, const int* __restrict__ cover_sub,
+    const int* __restrict__ entry_cell, const int* __restrict__ cell_count,
+    const int* __restrict__ cell_pstart, const int64_t* __restrict__ entry_base,
+    const int* __restrict__ cover_off, const double* __restrict__ xs, const int* __restrict__ rcls,
+    const RowClass* __restrict__ c_cls, const double* __restrict__ W,
+    const double* __restrict__ Bias, double* __restrict__ panels, const Ansatz an,
+    float* __restrict__ panels32, int wexp, int rows) {
+  constexpr int dim = kTwo ? 2 : 1;
+  extern __shared__ __align__(16) unsigned char k1_smem[];
+  int4* tab = reinterpret_cast<int4*>(k1_smem);
+  for (int i = threadIdx.x; i < 3 * rows; i += blockDim.x) tab[i] = kTanhTable[i];
+  __syncthreads();
+  const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
+  const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + wq;
+  if (t >= n_tiles) return;
+  RowTerms* rowt = reinterpret_cast<RowTerms*>(tab + 3 * rows) + wq * 32;
+  double* fac = reinterpret_cast<double*>(reinterpret_cast<RowTerms*>(tab + 3 * rows) +
+                                          (blockDim.x >> 5) * 32) +
+                (size_t)wq * nl_max * kFacVals * 32;
+  const int4 tile = tiles[t];
+  const int e0 = tile.x, nl = tile.y, p0 = tile.z;
+  const int c = entry_cell[e0];
+  const int cnt = cell_count[c];
+  const int pad = cell_pstart[c + 1] - cell_pstart[c];
+  const int nrows = min(32, pad - p0);
+  const int64_t rstride = (int64_t)(cover_off[c + 1] - cover_off[c]) * K;
+  const bool valid = lane < nrows && p0 + lane < cnt;
+  const int64_t R = (int64_t)cell_pstart[c] + p0 + lane;
+  double x[2] = {0.0, 0.0};
+  if (valid) {
+    x[0] = xs[R * dim];
+    if (kTwo) x[1] = xs[R * dim + 1];
+  }
+
+  // phase 1a: the level's window factors and their sums
+  double S = 0, dS[2] = {0, 0}, ddS[2] = {0, 0};
+  for (int k = 0; k < nl; ++k) {
+    double f[2] = {1, 1}, fp[2] = {0, 0}, fpp[2] = {0, 0};
+    int64_t x61[2] = {0, 0};
+    if (valid) {
+      const SubGeom& g = sub[cover_sub[e0 + k]];
+#pragma unroll
+      for (int i = 0; i < dim; ++i)
+        window_axis(x[i] - g.mu[i], g.sigma_d[i], g.inv_sigma_d[i], f[i], fp[i], fpp[i], x61[i]);
+    } else {
+      f[0] = 0.0;
+    }
+    const double w = f[0] * f[1], dw[2] = {fp[0] * f[1], f[0] * fp[1]};
+    const double ddw[2] = {fpp[0] * f[1], f[0] * fpp[1]};
+    S += w;
+    for (int i = 0; i < dim; ++i) {
+      dS[i] += dw[i];
+      ddS[i] += ddw[i];
+    }
+    double* fk = fac + (size_t)k * kFacVals * 32 + lane;
+    fk[0] = w;
+    fk[32] = dw[0];
+    fk[64] = dw[1];
+    fk[96] = ddw[0];
+    fk[128] = ddw[1];
+    fk[160] = __longlong_as_double(x61[0]);
+    fk[192] = __longlong_as_double(x61[1]);
+  }
+  const double iS = S > 0.0 ? 1.0 / S : 0.0;
+  RowClass rc{};
+  double Aa = 1.0, dA[2] = {0.0, 0.0}, ddA[2] = {0.0, 0.0};
+  if (valid) {
+    rc = c_cls[rcls[R]];
+    if (an.w > 0.0) ansatz_at(an, x, dim, Aa, dA, ddA);
+  }
+  const double wsc = scalbn(1.0, wexp);
+  const double w_in = scalbn(1.0, 61 - wexp), b_in = scalbn(1.0, 60 - wexp);
+
+  for (int k = 0; k < nl; ++k) {
+    const int e = e0 + k;
+    const int s = cover_sub[e];
+    const double is0 = sub[s].inv_sigma_d[0], is1 = kTwo ? sub[s].inv_sigma_d[1] : 0.0;
+    // phase 1b: this panel's normalised window (quotient rule over the level)
+    const double* fk = fac + (size_t)k * kFacVals * 32 + lane;
+    const double wo = fk[0], dwo[2] = {fk[32], fk[64]}, ddwo[2] = {fk[96], fk[128]};
+    // w = om S, so om' = (w' - om S') / S and om'' = (w'' - 2 om' S' - om S'') / S:
+    // exactly 1, 0, 0 where one subdomain covers the point
+    double om = wo * iS, dom[2] = {0, 0}, ddom[2] = {0, 0};
+    om = fma(fma(-om, S, wo), iS, om);
+    for (int i = 0; i < dim; ++i) {
+      dom[i] = (dwo[i] - om * dS[i]) * iS;
+      ddom[i] = (ddwo[i] - 2.0 * dom[i] * dS[i] - om * ddS[i]) * iS;
+    }
+    if (an.w > 0.0) {   // hard-constraint ansatz, as in k_assemble
+      for (int i = 0; i < dim; ++i) {
+        ddom[i] = ddA[i] * om + 2.0 * dA[i] * dom[i] + Aa * ddom[i];
+        dom[i] = dA[i] * om + Aa * dom[i];
+      }
+      om = Aa * om;
+    }
+    double A = 0, be0 = 0, be1 = 0, ga0 = 0, ga1 = 0;
+    const int64_t y0 = __double_as_longlong(fk[160]), y1 = __double_as_longlong(fk[192]);
+    if (valid) {
+      const double sc = rc.scale;
+      A = sc * (rc.c2[0] * ddom[0] + rc.c1[0] * dom[0] + rc.c0 * om +
+                (kTwo ? rc.c1[1] * dom[1] + rc.c2[1] * ddom[1] : 0.0));
+      be0 = sc * (rc.c1[0] * om + 2.0 * rc.c2[0] * dom[0]);
+      ga0 = sc * rc.c2[0] * om;
+      if (kTwo) {
+        be1 = sc * (rc.c1[1] * om + 2.0 * rc.c2[1] * dom[1]);
+        ga1 = sc * rc.c2[1] * om;
+      }
+    }
+
+    __syncwarp();   // the previous panel's row terms have been read
+    {
+      const double s0 = is0 * wsc, s1 = is1 * wsc;
+      const double B0 = be0 * s0, B1 = be1 * s1;
+      const double C0 = 2.0 * ga0 * (s0 * s0), C1 = 2.0 * ga1 * (s1 * s1);
+      auto expo = [](double v) { return (__double2hiint(v) >> 20) & 0x7ff; };
+      const int ef = max(max(expo(A), max(expo(B0), expo(B1))), max(expo(C0), expo(C1)));
+      const bool zero = A == 0.0 && B0 == 0.0 && B1 == 0.0 && C0 == 0.0 && C1 == 0.0;
+      const bool fits = zero || (ef > 150 && ef < 1900);
+      const int er = zero ? 0 : ef - 1022;
+      const double q = fits ? scalbn(1.0, 60 - er) : 0.0;
+      auto fixed = [&](double v) { return fx::split(fits ? __double2ll_rn(v * q) : 0ll); };
+      const fx::Val a = fixed(0.5 * A), b0 = fixed(B0), b1 = fixed(B1), c0 = fixed(C0),
+                    c1 = fixed(C1);
+      const fx::Val v0 = fx::split(y0), v1 = fx::split(y1);
+      rowt[lane].a = make_int4(a.hi, a.lo, fits ? er : kRow64, 0);
+      rowt[lane].b = make_int4(b0.hi, b0.lo, b1.hi, b1.lo);
+      rowt[lane].c = make_int4(c0.hi, c0.lo, c1.hi, c1.lo);
+      rowt[lane].x = make_int4(v0.hi, v0.lo, v1.hi, v1.lo);
+    }
+    __syncwarp();
+    double* out = panels + entry_base[e] * (int64_t)K + (int64_t)p0 * rstride;
+    // 64 features at a time: two a lane keep the registers for four blocks an SM
+    for (int f0 = 0; f0 < K; f0 += 32 * kFxFeatures) {
+      // this lane's features f0 + lane + 32 i: weights, their squares, bias
+      fx::Val w0[kFxFeatures], w1[kFxFeatures], q0[kFxFeatures], q1[kFxFeatures];
+      int64_t bb[kFxFeatures];
+#pragma unroll
+      for (int i = 0; i < kFxFeatures; ++i) {
+        const int f = f0 + lane + 32 * i;
+        const int64_t q = (int64_t)s * K + f;
+        const bool on = f < K;
+        w0[i] = fx::split(on ? __double2ll_rn(W[q * dim] * w_in) : 0ll);
+        q0[i] = fx::split(fx::mul_add(w0[i], w0[i], 0) << 1);
+        w1[i] = fx::split(on && kTwo ? __double2ll_rn(W[q * dim + 1] * w_in) : 0ll);
+        q1[i] = fx::split(fx::mul_add(w1[i], w1[i], 0) << 1);
+        bb[i] = on ? __double2ll_rn(Bias[q] * b_in) : 0ll;
+      }
+
+      // phase 2: row by row, every lane its own features
+      for (int r = 0; r < nrows; ++r) {
+        const int4 ra = rowt[r].a, rb = rowt[r].b, rg = rowt[r].c, rx = rowt[r].x;
+        double* orow = out + (int64_t)r * rstride;
+        if (ra.z == kRow64) {
+          const double uA = __shfl_sync(0xffffffffu, A, r);
+          const double ub0 = __shfl_sync(0xffffffffu, be0, r), ub1 = __shfl_sync(0xffffffffu, be1, r);
+          const double ug0 = __shfl_sync(0xffffffffu, ga0, r), ug1 = __shfl_sync(0xffffffffu, ga1, r);
+          const double ux0 = (double)__shfl_sync(0xffffffffu, y0, r) * 0x1p-61;
+          const double ux1 = (double)__shfl_sync(0xffffffffu, y1, r) * 0x1p-61;
+          for (int f = f0 + lane; f < min(K, f0 + 32 * kFxFeatures); f += 32) {
+            const int64_t q = (int64_t)s * K + f;
+            const double v = entry64(W[q * dim], kTwo ? W[q * dim + 1] : 0.0, Bias[q], ux0, ux1, is0,
+                                     is1, uA, ub0, ub1, ug0, ug1);
+            if (kSplit) {
+              const float hi = __double2float_rn(v);
+              reinterpret_cast<float2*>(orow)[f] = make_float2(hi, __double2float_rn(v - (double)hi));
+              if (panels32) panels32[(orow - panels) + f] = hi;
+            } else {
+              orow[f] = v;
+            }
+          }
+          continue;
+        }
+#pragma unroll
+        for (int i = 0; i < kFxFeatures; ++i) {
+          if (f0 + 32 * i >= K) break;   // warp-uniform
+          const int64_t arg = fx::argument(w0[i], {rx.x, rx.y}, w1[i], {rx.z, rx.w}, bb[i], kTwo);
+          const int64_t phi = fx::tanh61(arg, 54 - wexp, tab, rows);
+          const fx::Val p = fx::split(phi << 1);   // units of 2^-62
+          // B and C, then D = B - phi C (2^(er - 59))
+          int64_t xb = (int64_t)rb.x * w0[i].lo + ((int64_t)rb.y * w0[i].hi + (1 << 30));
+          int64_t xc = (int64_t)rg.x * q0[i].lo + ((int64_t)rg.y * q0[i].hi + (1 << 30));
+          int64_t B = (int64_t)rb.x * w0[i].hi, C = (int64_t)rg.x * q0[i].hi;
+          if (kTwo) {
+            xb += (int64_t)rb.z * w1[i].lo + (int64_t)rb.w * w1[i].hi;
+            xc += (int64_t)rg.z * q1[i].lo + (int64_t)rg.w * q1[i].hi;
+            B += (int64_t)rb.z * w1[i].hi;
+            C += (int64_t)rg.z * q1[i].hi;
+          }
+          B += xb >> 31;
+          C += xc >> 31;
+          const int64_t D = B - fx::mul_add(p, fx::split(C), 0);
+          // M = D + phi (A - phi D) (2^(er - 59))
+          const int64_t A59 = ((int64_t)ra.x << 31) + ra.y;
+          const int64_t M =
+              fx::mul_add(p, fx::split(A59 - fx::mul_add(p, fx::split(D), 0)), D);
+          const int f = f0 + lane + 32 * i;
+          if (f >= K) continue;
+          // M 2^(er - 59) as n 2^(ex - 63), n's top bit set
+          const uint64_t m = (uint64_t)(M < 0 ? -M : M);
+          const int lz = __clzll((long long)m);
+          const uint64_t nrm = m << (lz & 63);
+          const int ex = ra.z + 4 - lz;
+          const uint64_t odd = (nrm >> 11) & 1;
+          const uint64_t man = (nrm >> 11) + ((nrm & 0x7ff) + odd > 0x400);   // to nearest even
+          const uint64_t sign = (uint64_t)M & 0x8000000000000000ull;
+          if (kSplit) {
+            float2 hl;
+            if (ex > -72 && ex < 100 && m != 0) {   // both parts in FP32's normal range
+              // the double's top 24 bits to nearest even, and the rest
+              const uint32_t h24 = (uint32_t)(man >> 29), rest = (uint32_t)man & 0x1fffffffu;
+              const uint32_t up = rest + (h24 & 1) > 0x10000000u;
+              const uint32_t sg = (uint32_t)(sign >> 32);
+              hl.x = __uint_as_float((((uint32_t)(ex + 126) << 23) + h24 + up) | sg);
+              const float lo = __int2float_rn((int)rest - (int)(up << 29)) *
+                               __uint_as_float((uint32_t)(ex - 52 + 127) << 23);
+              hl.y = __uint_as_float(__float_as_uint(lo) ^ sg);
+            } else {
+              const double v = m == 0 ? 0.0
+                                      : __longlong_as_double((long long)(
+                                            (((uint64_t)(ex + 1022) << 52) + man) | sign));
+              hl.x = __double2float_rn(v);
+              hl.y = __double2float_rn(v - (double)hl.x);
+            }
+            reinterpret_cast<float2*>(orow)[f] = hl;
+            if (panels32) panels32[(orow - panels) + f] = hl.x;
+          } else {
+            orow[f] = m == 0 ? 0.0
+                             : __longlong_as_double(
+                                   (long long)((((uint64_t)(ex + 1022) << 52) + man) | sign));
+          }
+        }
+      }
+    }
+  }
+}
+
+// FP64-accurate entries in fixed point: weight scales 1/16 .. 1, at which
+// arguments stay within +-3 and 1 - phi^2 above 2^-7, so that its 2^-60 absolute
+// error is no larger than FP64's relative one; larger and smaller scales keep
+// the FP64 form.  False: not taken.
+bool launch_assemble_fx(elmfb_ctx* h, bool split, double* panels, float* panels32,
+                        const Ansatz& an) {
+  const double a = h->cfg.weight_scale;
+  const int wexp = a > 0.0 ? fx::weight_exp(a) : 1;
+  if (wexp < fx::kMinExp || wexp > 0) return false;
+  const int rows = fx::tanh_rows(h->dim, wexp), warps = 2;
+  const size_t smem = (size_t)rows * 3 * sizeof(int4) + warps * 32 * sizeof(RowTerms) +
+                      (size_t)warps * h->nl_max * kFacVals * 32 * sizeof(double);
+  if (smem > 220 * 1024) return false;
+  prof_begin(h, KID_ASSEMBLE, (double)h->NPR * h->K * (8.0 + (panels32 ? 4.0 : 0.0)) +
+                                  (double)h->NR * (8.0 * h->dim + 4.0));
+#define ELMFB_K1FX(SP, TWO)                                                                   \
+  do {                                                                                       \
+    ensure_dyn_smem((const void*)k_assemble_fx<SP, TWO>, smem);                              \
+    k_assemble_fx<SP, TWO>                                                                   \
+        <<<(unsigned)ceil_div(h->n_ltiles, warps), warps * 32, smem, h->stream>>>(           \
+            h->d_ltiles.as<int4>(), h->n_ltiles, h->K, h->nl_max, h->d_sub.as<SubGeom>(),    \
+            h->d_cover_sub.as<int>(), h->d_entry_cell.as<int>(), h->d_cell_count.as<int>(),  \
+            h->d_cell_pstart.as<int>(), h->d_entry_base.as<int64_t>(),                       \
+            h->d_cover_off.as<int>(), h->d_x.as<double>(), h->d_rcls.as<int>(),              \
+            h->d_cls.as<RowClass>(), h->d_W64.as<double>(), h->d_b64.as<double>(), panels,   \
+            an, panels32, wexp, rows);                                                       \
+  } while (0)
+  if (h->dim == 2) {
+    if (split) ELMFB_K1FX(true, true);
+    else ELMFB_K1FX(false, true);
+  } else {
+    if (split) ELMFB_K1FX(true, false);
+    else ELMFB_K1FX(false, false);
+  }
+#undef ELMFB_K1FX
+  prof_end(h, KID_ASSEMBLE);
+  check_launch("k_assemble_fx");
+  count_launch(h);
+  return true;
+}
+
 template <class T>
 void launch_assemble(elmfb_ctx* h) {
   const int K = h->K;
@@ -561,6 +927,9 @@ void launch_assemble(elmfb_ctx* h) {
   if (smem > 220 * 1024)
     ELMFB_THROW(ELMFB_ERR_UNSUPPORTED, "assembly: too many covering subdomains per level");
   const Ansatz an = make_ansatz(h->cfg);
+  if constexpr (sizeof(T) == 8) {
+    if (launch_assemble_fx(h, split, pout, p32, an)) return;
+  }
 #define ELMFB_K1_ARGS                                                                        \
   h->d_ltiles.as<int4>(), h->n_ltiles, h->dim, K, h->nl_max, h->d_sub.as<SubGeom>(),         \
       h->d_cover_sub.as<int>(), h->d_cover_start.as<int>(), h->d_entry_cell.as<int>(),       \

@@ -490,11 +490,14 @@ void eval_model(elmfb_ctx* h, const double* xs, int64_t n, double* out) {
     // few points: half-size blocks, so that they spread over more SMs
     const int threads = n < 152 * 16 ? 128 : 256;
 #define ELMFB_EVAL_FX(TWO)                                                                     \
-  k_eval_fx<TWO><<<(unsigned)ceil_div(n * 32, threads), threads, smem, st>>>(                  \
-      x, n, h->K, h->L, h->d_bnd.as<double>(), h->nc[0], h->nc[1], h->d_sub.as<SubGeom>(),     \
-      h->d_cell_level_off.as<int>(), h->d_cover_sub.as<int>(), cols, expo, 55 - wexp, rows,    \
-      eval_room(h->K, h->max_cover), h->d_W64.as<double>(), h->d_b64.as<double>(),      \
-      h->d_a.as<double>(), o, make_ansatz(h->cfg))
+  do {                                                                                         \
+    ensure_dyn_smem((const void*)k_eval_fx<TWO>, smem);                                        \
+    k_eval_fx<TWO><<<(unsigned)ceil_div(n * 32, threads), threads, smem, st>>>(                \
+        x, n, h->K, h->L, h->d_bnd.as<double>(), h->nc[0], h->nc[1], h->d_sub.as<SubGeom>(),   \
+        h->d_cell_level_off.as<int>(), h->d_cover_sub.as<int>(), cols, expo, 54 - wexp, rows,  \
+        eval_room(h->K, h->max_cover), h->d_W64.as<double>(), h->d_b64.as<double>(),           \
+        h->d_a.as<double>(), o, make_ansatz(h->cfg));                                          \
+  } while (0)
     if (h->dim == 2) ELMFB_EVAL_FX(true);
     else ELMFB_EVAL_FX(false);
 #undef ELMFB_EVAL_FX

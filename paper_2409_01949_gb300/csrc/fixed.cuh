@@ -67,8 +67,8 @@ FX_FN int64_t argument(Val w0, Val x0, Val w1, Val x1, int64_t b, bool two) {
   return s + (cross >> 31);
 }
 
-// tanh(s) in units of 2^-61, s in units of 2^(wexp - 60); `shift` = 55 - wexp is
-// the width of an interval of 1/32.  tab holds `rows` rows of the table
+// tanh(s) in units of 2^-61, s in units of 2^(wexp - 60); `shift` = 54 - wexp is
+// the width of an interval of 1/64.  tab holds `rows` rows of the table
 // (tanh_table.py), the last of them for everything past the others.
 FX_FN int64_t tanh61(int64_t s, int shift, const int4* tab, int rows) {
   const uint64_t m = (uint64_t)(s < 0 ? -s : s);
@@ -78,22 +78,21 @@ FX_FN int64_t tanh61(int64_t s, int shift, const int4* tab, int rows) {
   const Val r = split((int64_t)((m << (64 - shift)) >> 1) - ((int64_t)1 << 62));
   const int4 a = tab[3 * j], b = tab[3 * j + 1], d = tab[3 * j + 2];
   auto word = [](int lo, int hi) { return (int64_t)(((uint64_t)(uint32_t)hi << 32) | (uint32_t)lo); };
-  // the upper coefficients fit 32 bits, and the high half of r is enough
-  int t = (int)(((int64_t)(d.y >> 16) * r.hi) >> 31) + d.w;   // c7 r + c6
-  t = (int)(((int64_t)t * r.hi) >> 31) + d.z;                 // ... r + c5
-  int64_t v = (((int64_t)t * r.hi) >> 31) + word(d.x, (int)(short)d.y);   // ... + c4
-  v = mul_add(split(v), r, word(b.z, b.w));
+  // c4 and up fit 32 bits, and the high half of r is enough for them
+  int t = (int)(((int64_t)d.z * r.hi) >> 31) + d.y;                // c6 r + c5
+  t = (int)(((int64_t)t * r.hi) >> 31) + d.x;                      // ... r + c4
+  int64_t v = (((int64_t)t * r.hi) >> 31) + word(b.z, b.w);        // ... r + c3
   v = mul_add(split(v), r, word(b.x, b.y));
   v = mul_add(split(v), r, word(a.z, a.w));
   v = mul_add(split(v), r, word(a.x, a.y));
   return s < 0 ? -v : v;
 }
 
-constexpr int kTanhRows = 32 * 22 + 1;   // tanh_table.py: 32 a unit up to 22, and the closing row
+constexpr int kTanhRows = 64 * 22 + 1;   // tanh_table.py: 64 a unit up to 22, and the closing row
 
 // rows that arguments up to (dim + 1) 2^wexp reach, the closing row included
 FX_FN int tanh_rows(int dim, int wexp) {
-  const int64_t n = wexp >= 0 ? (int64_t)(dim + 1) * 32 << wexp : ((int64_t)(dim + 1) * 32 >> -wexp) + 1;
+  const int64_t n = wexp >= 0 ? (int64_t)(dim + 1) * 64 << wexp : ((int64_t)(dim + 1) * 64 >> -wexp) + 1;
   return n + 1 < kTanhRows ? (int)n + 1 : kTanhRows;
 }
 

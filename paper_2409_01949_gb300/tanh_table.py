@@ -1,30 +1,29 @@
 """Writes the table of the fixed-point tanh (csrc/fixed.cuh) as a C++ include.
 
-Row j holds the degree-7 polynomial of tanh on [j/32, (j+1)/32) in the variable
-r = 64 (s - (j + 1/2)/32) in [-1, 1): the Taylor polynomial of degree 20 about the
-interval's middle, from the recurrence of T' = 1 - T^2, lowered to degree 7 by
+Row j holds the degree-6 polynomial of tanh on [j/64, (j+1)/64) in the variable
+r = 128 (s - (j + 1/2)/64) in [-1, 1): the Taylor polynomial of degree 20 about the
+interval's middle, from the recurrence of T' = 1 - T^2, lowered to degree 6 by
 subtracting the leading multiples of Chebyshev polynomials (economisation,
-Lanczos 1938); the dropped terms are below 2^-60.  Coefficients are integers in
+Lanczos 1938); the dropped terms are below 2^-58.  Coefficients are integers in
 units of 2^-61.  The last row is the constant 1 - 2^-61, for s >= 22 where
 1 - tanh(s) < 2^-62.
 
-A row is three 16-byte words: (c0, c1), (c2, c3), then c4's low 32 bits, c7 in
-the upper and the rest of c4 in the lower half of one word, c5, c6.
+A row is three 16-byte words: (c0, c1), (c2, c3) in 64 bits each, then c4, c5, c6.
 """
 from __future__ import annotations
 
 import decimal
 import os
 
-ROWS_PER_UNIT = 32
+ROWS_PER_UNIT = 64
 LIMIT = 22
-DEGREE = 7
+DEGREE = 6
 BITS = 61
 TAYLOR = 20
 
 
 def row(j: int):
-    """The eight integer coefficients of interval j."""
+    """The seven integer coefficients of interval j."""
     D = decimal.Decimal
     s0 = D(2 * j + 1) / (2 * ROWS_PER_UNIT)
     e = (-2 * s0).exp()
@@ -50,11 +49,9 @@ def words(c):
     """A row as twelve 32-bit words."""
     def split(v):
         return [v & 0xFFFFFFFF, (v >> 32) & 0xFFFFFFFF]
-    assert -2 ** 47 <= c[4] < 2 ** 47 and -2 ** 15 <= c[7] < 2 ** 15
-    assert all(-2 ** 31 <= v < 2 ** 31 for v in c[5:7])
+    assert all(-2 ** 31 <= v < 2 ** 31 for v in c[4:])
     w = split(c[0]) + split(c[1]) + split(c[2]) + split(c[3])
-    w += [c[4] & 0xFFFFFFFF, ((c[7] & 0xFFFF) << 16) | ((c[4] >> 32) & 0xFFFF),
-          c[5] & 0xFFFFFFFF, c[6] & 0xFFFFFFFF]
+    w += [v & 0xFFFFFFFF for v in c[4:]] + [0]
     return w
 
 

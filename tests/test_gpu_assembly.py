@@ -160,3 +160,52 @@ def test_empty_boundary_set_and_boundary_points():
     with E.Solver.from_problem(P) as s:
         s.assemble(sets)
         assert s.sizes().n_rows == 32
+
+
+# weight scales at and past the ends of the fixed-point range (1/16 .. 1), a
+# scale that is no power of two, K at the edges of the 64-feature passes, one
+# axis and two
+@pytest.mark.parametrize("dim,K,a", [(1, 1, 1.0), (1, 32, 1.0 / 16), (1, 65, 0.7), (1, 96, 0.05),
+                                     (2, 31, 1.0), (2, 64, 0.06), (2, 100, 0.3), (2, 8, 1.5)])
+@pytest.mark.parametrize("prec", [E.FP64, E.DF32])
+def test_entries_over_weight_scales(dim, K, a, prec):
+    """FP64 entries and FP32 pairs against the oracle at 100 times the FP64
+    unit (48-bit pairs: 2^-48) of the block's term scale: the arithmetic after
+    the windows is a dozen roundings, the windows' second derivatives lose two
+    digits at most to the quotient rule's cancellation."""
+    mk = WL.poisson1d if dim == 1 else WL.poisson2d
+    kw = dict(n_interior=150) if dim == 1 else dict(n_side=20, n_boundary_side=9)
+    P = mk(levels=(1, 3, 4), features=K, weight_scale=a, delta=2.3, **kw)
+    with E.Solver.from_problem(P, precision=prec) as s:
+        s.assemble_problem(P)
+        M, _ = s.get_rows(np.arange(P.n_rows))
+    ref = OS.assemble(P, fmt="dense", with_bound=True)
+    tol = 100 * 2.0 ** -53 if prec == E.FP64 else 2.0 ** -48 + 100 * 2.0 ** -53
+    assert np.all(np.abs(M - ref["M"]) <= tol * _scale(ref["bound"], K))
+
+
+@pytest.mark.parametrize("c", [1e-290, 1e-150, 1.0, 1e150, 1e290])
+def test_entries_scale_with_the_operator(c):
+    """Entries are linear in the operator's coefficients: rows of terms far
+    outside the fixed-point exponents (1e-290, 1e290) go through FP64 and agree
+    with the scaled entries of the unscaled operator to a few roundings."""
+    P = WL.poisson1d(levels=(2, 5), features=40, n_interior=64)
+    out = []
+    for k in (1.0, c):
+        with E.Solver.from_problem(P, precision=E.FP64) as s:
+            s.assemble([dict(points=P.interior.points, rhs=P.interior.rhs, c0=0.5 * k,
+                             c1=(0.25 * k, 0.0), c2=(-k, 0.0))])
+            out.append(s.get_rows(np.arange(64))[0])
+    # 64 ulp of each row's largest entry: the two sides may round in different forms
+    top = np.abs(out[0]).max(axis=1, keepdims=True)
+    assert np.all(np.abs(out[1] / c - out[0]) <= 64 * 2.0 ** -53 * top)
+
+
+def test_nonfinite_operator_gives_nonfinite_entries():
+    P = WL.poisson1d(levels=(4,), features=12, n_interior=30)
+    for bad in (np.inf, np.nan):
+        with E.Solver.from_problem(P, precision=E.FP64) as s:
+            s.assemble([dict(points=P.interior.points, rhs=P.interior.rhs, c0=bad, c2=(-1.0, 0.0))])
+            M, _ = s.get_rows(np.arange(30))
+        inside = np.abs((np.arange(4) + 0.5) / 4 - P.interior.points) < 0.25
+        assert not np.isfinite(M.reshape(30, 4, 12)[inside]).any()
