@@ -529,15 +529,16 @@ __global__ void __launch_bounds__(128) k_assemble(
       }
     }
     if (WRITE_T) {
-      // feature-major BF16 copy: feature f, rows rho0 .. rho0+nrows in 16-byte pieces
+      // the BF16 copy: 8 rows of a feature are 16 bytes of its 16-row block, the
+      // next feature's beside them
       __syncwarp();
       const int64_t rho0 = panel_off[s] + cover_start[e] + p0;
-      const int pieces = nrows / 8;   // nrows is 16 or 32
-      for (int idx = lane; idx < K * pieces; idx += 32) {
-        const int f = idx / pieces, q = idx - f * pieces;
-        const uint4 val = *reinterpret_cast<const uint4*>(tsm + (size_t)f * 32 + q * 8);
-        *reinterpret_cast<uint4*>(pt + (int64_t)f * NPR + rho0 + q * 8) = val;
-      }
+      const int bytes = gram_block_bytes(K);
+      uint8_t* blk = reinterpret_cast<uint8_t*>(pt) + (rho0 >> 4) * bytes;
+      for (int q = 0; q < nrows / 8; ++q)   // nrows is 16 or 32
+        for (int f = lane; f < K; f += 32)
+          *reinterpret_cast<uint4*>(blk + (int64_t)(q >> 1) * bytes + (q & 1) * (bytes / 2) + f * 16) =
+              *reinterpret_cast<const uint4*>(tsm + (size_t)f * 32 + q * 8);
     }
   }
 }
@@ -950,7 +951,7 @@ void launch_assemble(elmfb_ctx* h) {
     else ELMFB_K1_LAUNCH(F, false, false, false, nullptr, nullptr);                          \
     break;
   // algorithmic bytes: every panel entry written once (twice in mixed precision:
-  // FP32 row-major and BF16 feature-major), point data read once
+  // FP32 row-major and in BF16), point data read once
   prof_begin(h, KID_ASSEMBLE,
              (double)h->NPR * K * (sizeof(T) + (wt ? 2.0 : 0.0) + (p32 ? 4.0 : 0.0)) +
                  (double)h->NR * (h->dim * 8.0 + 4.0));
@@ -1231,9 +1232,10 @@ void assemble_system(elmfb_ctx* h, int n_sets, const elmfb_rowset* sets) {
   h->gnn_nb.clear();
   h->gnn_trained = false;
   if (h->cfg.precision == ELMFB_MIXED) {
-    h->d_pt.alloc(h->NPR * h->K * 2, st);
+    const size_t pt_bytes = (size_t)(h->NPR / 16) * gram_block_bytes(h->K);
+    h->d_pt.alloc(pt_bytes, st);
     // padding tail of 16-row tiles is written by the kernel; clear once for safety
-    CUDA_CHECK(cudaMemsetAsync(h->d_pt.p, 0, h->NPR * h->K * 2, st));
+    CUDA_CHECK(cudaMemsetAsync(h->d_pt.p, 0, pt_bytes, st));
   }
   if (h->eval64() || h->dual()) launch_assemble<double>(h);
   else launch_assemble<float>(h);

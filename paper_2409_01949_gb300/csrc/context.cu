@@ -356,6 +356,16 @@ cudaMemPool_t library_pool() {
   return pool;
 }
 
+bool usable_in_place(const elmfb_ctx* h, const void* p, size_t align) {
+  if ((uintptr_t)p % align != 0) return false;
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == h->device;
+}
+
 void ensure_dyn_smem(const void* func, size_t bytes, bool max_carveout) {
   static std::mutex mu;
   static std::map<std::pair<int, const void*>, size_t> limit;

@@ -63,6 +63,11 @@ struct DevBuf {
   template <class T> T* as() const { return reinterpret_cast<T*>(p); }
 };
 
+// The BF16 copy of the panels as the tensor cores read it: 16 panel rows (panel
+// rows 16 q .. 16 q + 15, all of one cell) are one block, element (feature k, row
+// r) at byte (r / 8) (block / 2) + (k / 8) 128 + (k % 8) 16 + (r % 8) 2.
+__host__ __device__ constexpr int gram_block_bytes(int K) { return ((K + 7) & ~7) * 32; }
+
 // Row padding of a cell of the common refinement and the row-class limit.
 constexpr int kCellPad = 16;            // cell row groups are padded to this multiple
 constexpr int kMaxClasses = ELMFB_MAX_ROWSETS;
@@ -201,11 +206,11 @@ struct elmfb_ctx {
   DevBuf d_entry_cell;
   DevBuf d_flags;       // device status flags (int[4])
 
-  // BF16 feature-major panel copy PT[k][rho] (mixed precision) and Gram blocks
+  // BF16 panel copy (mixed precision; gram_block_bytes) and Gram blocks
   DevBuf d_pt;
   std::vector<std::pair<int, int>> gram_pair_ij;   // sorted (i <= j)
-  int64_t gram_runs = 0;
-  DevBuf d_gram_pairs, d_gram_runs, d_gram;        // d_gram: [pair][K][K] FP32
+  int gram_ctas = 0, gram_multi = 0, gram_parts = 0;
+  DevBuf d_gram_tasks, d_gram_task_off, d_gram_runs, d_gram_multi, d_gram;   // d_gram: [pair][K][K] FP32
   bool have_gram = false;
 
   // learned preconditioner: subdomain graph, weights, Adam moments, work buffers
@@ -423,6 +428,10 @@ void prof_harvest(elmfb_ctx* h, size_t keep = 0);   // all but the last `keep` r
 // forget the timed launches of kernel kid from ordinal `from` on (launches
 // that returned at once after LSQR stopped on the device)
 void prof_drop_from(elmfb_ctx* h, int kid, int64_t from);
+
+// p lies in this device's own memory and is aligned, so that a kernel may use
+// it in place
+bool usable_in_place(const elmfb_ctx* h, const void* p, size_t align);
 
 // helpers
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }

@@ -439,18 +439,6 @@ __global__ void k_err_pass2(const double* __restrict__ ur, int64_t n,
 
 }  // namespace
 
-// p lies in this device's own memory and is aligned, so that a kernel may use
-// it in place
-static bool in_place(const elmfb_ctx* h, const void* p, size_t align) {
-  if ((uintptr_t)p % align != 0) return false;
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return at.type == cudaMemoryTypeDevice && at.device == h->device;
-}
-
 void eval_model(elmfb_ctx* h, const double* xs, int64_t n, double* out) {
   if (n == 0) return;
   cudaStream_t st = h->stream;
@@ -463,12 +451,12 @@ void eval_model(elmfb_ctx* h, const double* xs, int64_t n, double* out) {
   DevBuf dx, dout;
   const double* x = xs;
   double* o = out;
-  if (!apart || !in_place(h, xs, sizeof(double))) {
+  if (!apart || !usable_in_place(h, xs, sizeof(double))) {
     dx.alloc(xb, st);
     CUDA_CHECK(cudaMemcpyAsync(dx.p, xs, xb, cudaMemcpyDefault, st));
     x = dx.as<double>();
   }
-  if (!apart || !in_place(h, out, sizeof(double))) {
+  if (!apart || !usable_in_place(h, out, sizeof(double))) {
     dout.alloc(ob, st);
     o = dout.as<double>();
   }

@@ -9,21 +9,42 @@
 // runs (one per shared cell, merged where both panels continue contiguously),
 // each a multiple of 16 rows.
 //
-// Operands come from the BF16 feature-major copy of the panels written by the
-// assembly kernel in mixed precision: PT[k][rho] (rho = panel row).  For one
-// pair, A = P_i^T (features x rows) and B = P_j^T are both K-major along the
-// contraction, loaded by 2-D TMA boxes of 64 rows x K features with 128-byte
-// swizzle into a 4-stage shared-memory ring.  One thread issues
-// tcgen05.mma (M = 128, N = K rounded up to 16, 16 rows per instruction) into
-// a TMEM accumulator, releasing each stage with tcgen05.commit; all four warps
-// then read the accumulator with tcgen05.ld and store the FP32 block.  Rows of
-// a box beyond its run are skipped by issuing only the valid 16-row steps.
+// Operands come from the BF16 copy of the panels written by the assembly kernel in
+// mixed precision, laid out as the tensor cores read it: per 16 panel rows one
+// block of 8 x 8 core matrices (8 features x 8 rows, 128 contiguous bytes),
+// features fastest, then the two row halves.  For one pair, A = P_i^T (features x
+// rows) and B = P_j^T are both K-major along the contraction; a box of up to 64
+// rows is one contiguous bulk copy into a shared-memory ring, and each of its 16-row
+// blocks one MMA step without swizzle.  One thread issues tcgen05.mma (M = 128,
+// N = K rounded up to 16) into a TMEM accumulator, releasing each stage with
+// tcgen05.commit.  Feature rows of a tile past K hold whatever the ring holds:
+// they reach only accumulator rows and columns past K, which are never read.
+// (As a feature-major matrix, 64-row boxes of it read by 2-D TMA were 128-byte
+// pieces 4 MB apart: 4.3 GB of DRAM reads for 0.57 GB of panels at 400^2 points,
+// K = 128, at a third of the DRAM rate.)
+//
+// A pair's rows are cut into tasks of a bounded number of rows, and one persistent
+// CTA per SM walks its list of them: a producer warp, an MMA warp and four
+// epilogue warps, with two accumulators, so that the ring runs on across tasks
+// while the last one's block is stored.  A pair of several tasks sums their blocks
+// in order (k_gram_sum).  Cells are visited in square blocks of 32 MB of panels
+// and tasks dealt in the order of their first cell, each to the CTA with the least
+// work so far, so that all CTAs are in the same place at the same time and the
+// panels stay in L2: with one CTA per pair, pair after pair, the coarse panels'
+// pairs each streamed the whole domain, and the level-1 pair alone was 2525 boxes
+// of one CTA.  400^2 points, levels 1..16, K = 128 (6297 pairs): 1.64 -> 0.85 ms,
+// 330 -> 640 TFLOP/s; the tiles arrive at 10 TB/s from L2, which bounds it (half
+// the ring costs 4%, so it is not latency): fewer tile reads per block would need
+// several pairs per accumulator set.
+//
 // Every mbarrier wait is bounded; a timeout raises flags[2].
 #include <algorithm>
-#include <map>
+#include <cmath>
 #include <cstring>
-
-#include <cudaTypedefs.h>
+#include <functional>
+#include <numeric>
+#include <queue>
+#include <unordered_map>
 
 #include <new>
 #include <stdexcept>
@@ -33,178 +54,341 @@
 
 namespace {
 
-constexpr int kStages = 4;
-constexpr int kBoxRows = 64;                 // contraction rows per box (128 B of BF16)
-constexpr int kTileBytes = 128 * 128;        // 128 feature rows x 128 B
-constexpr int kGramThreads = 128;
-constexpr size_t kGramSmem = 2 * kStages * kTileBytes + 1024;
+constexpr int kBoxRows = 64;                 // contraction rows per box
+constexpr int kMaxGramStages = 12;
+constexpr int kGramThreads = 192;            // producer, MMA, four epilogue warps
+constexpr size_t kGramRing = 192 * 1024;
+// ring, 1 KB alignment, and the rest of a 128-row tile past the last stage's K rows
+constexpr size_t kGramSmem = kGramRing + 16 * 1024 + 1024;
 
+// a box of 64 rows of one panel: four blocks
+__host__ __device__ constexpr int gram_tile_bytes(int K) { return 4 * gram_block_bytes(K); }
+
+// tasks: (first run, end run, diagonal, block: >= 0 a block of G, else partial ~block)
 __global__ void __launch_bounds__(kGramThreads, 1)
-    k_gram_tc(const __grid_constant__ CUtensorMap tmap, const int4* __restrict__ pairs,
-              const int4* __restrict__ runs, int K, int N, float* __restrict__ G,
-              int* __restrict__ flags) {
+    k_gram_tc(const uint8_t* __restrict__ pt, const int4* __restrict__ tasks,
+              const int* __restrict__ task_off, const int4* __restrict__ runs, int K, int N, int S,
+              float* __restrict__ G, float* __restrict__ part, int* __restrict__ flags) {
   extern __shared__ uint8_t smraw[];
-  __shared__ __align__(8) uint64_t full[kStages];
-  __shared__ __align__(8) uint64_t empty[kStages];
-  __shared__ __align__(8) uint64_t done;
+  __shared__ __align__(8) uint64_t full[kMaxGramStages];
+  __shared__ __align__(8) uint64_t empty[kMaxGramStages];
+  __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], done;
   __shared__ uint32_t tmem_slot;
   uint8_t* sm = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int4 task = pairs[blockIdx.x];   // (first run, end run, diagonal, -)
-  const bool diag = task.z != 0;
+  const int tile_bytes = gram_tile_bytes(K), block_bytes = gram_block_bytes(K);
+  const int t0 = task_off[blockIdx.x], t1 = task_off[blockIdx.x + 1];   // this CTA's tasks
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < S; ++s) {
       sm100::mbar_init(&full[s], 1);
       sm100::mbar_init(&empty[s], 1);
     }
+    for (int b = 0; b < 2; ++b) {
+      sm100::mbar_init(&acc_full[b], 1);
+      sm100::mbar_init(&acc_empty[b], 4);   // one arrival per epilogue warp
+    }
     sm100::mbar_init(&done, 1);
     sm100::fence_mbar_init();
-    sm100::prefetch_tensormap(&tmap);
   }
-  if (warp == 2) sm100::tmem_alloc(&tmem_slot, 128);
-  // zero the tiles once: feature rows >= K are never written by TMA
-  for (int i = threadIdx.x; i < 2 * kStages * kTileBytes / 16; i += blockDim.x)
-    reinterpret_cast<uint4*>(sm)[i] = make_uint4(0, 0, 0, 0);
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  if (warp == 2) sm100::tmem_alloc(&tmem_slot, 256);
   sm100::tc_fence_before();
   __syncthreads();
   sm100::tc_fence_after();
   const uint32_t tmem = tmem_slot;
-  const uint32_t idesc = sm100::idesc_bf16_f32(128, N);
-  const uint32_t box_bytes = (uint32_t)K * 128u;
-  int nboxes = 0;
-  for (int r = task.x; r < task.y; ++r) nboxes += (runs[r].z + kBoxRows - 1) / kBoxRows;
+  bool ok = true;
 
   if (warp == 0 && lane == 0) {
-    // TMA producer
-    int b = 0;
-    bool ok = true;
-    for (int r = task.x; r < task.y && ok; ++r) {
-      const int4 run = runs[r];
-      for (int off = 0; off < run.z; off += kBoxRows, ++b) {
-        const int stage = b % kStages, round = b / kStages;
-        if (round > 0 && !sm100::mbar_wait(&empty[stage], (round - 1) & 1)) {
-          atomicOr(&flags[2], 1);
-          ok = false;
-          break;
+    // producer: box b goes to stage b mod S once box b - S has left it
+    int st = 0, ph = 1, issued = 0;
+    for (int t = t0; t < t1 && ok; ++t) {
+      const int4 task = tasks[t];
+      int4 next = runs[task.x];   // one record ahead, so that its load is not waited for
+      for (int r = task.x; r < task.y && ok; ++r) {
+        const int4 run = next;
+        next = runs[min(r + 1, task.y - 1)];
+        for (int off = 0; off < run.z; off += kBoxRows) {
+          if (!sm100::mbar_wait(&empty[st], ph)) {   // the first round passes at once
+            ok = false;
+            break;
+          }
+          uint8_t* a = sm + (size_t)st * 2 * tile_bytes;
+          const uint32_t bytes = (uint32_t)(min(kBoxRows, run.z - off) / 16 * block_bytes);
+          sm100::mbar_arrive_expect_tx(&full[st], task.z ? bytes : 2 * bytes);
+          sm100::bulk_load(a, pt + (int64_t)((run.x + off) >> 4) * block_bytes, bytes, &full[st]);
+          if (!task.z)
+            sm100::bulk_load(a + tile_bytes, pt + (int64_t)((run.y + off) >> 4) * block_bytes,
+                             bytes, &full[st]);
+          ++issued;
+          if (++st == S) {
+            st = 0;
+            ph ^= 1;
+          }
         }
-        uint8_t* a = sm + stage * 2 * kTileBytes;
-        sm100::mbar_arrive_expect_tx(&full[stage], diag ? box_bytes : 2 * box_bytes);
-        sm100::tma_load_2d(a, &tmap, run.x + off, 0, &full[stage]);
-        if (!diag) sm100::tma_load_2d(a + kTileBytes, &tmap, run.y + off, 0, &full[stage]);
       }
     }
+    // no copy of this CTA is left in flight when it ends
+    for (int b = max(0, issued - S); b < issued; ++b)
+      if (!sm100::mbar_wait(&full[b % S], (b / S) & 1)) ok = false;
+    if (!ok) atomicOr(&flags[2], 1);
   } else if (warp == 1 && lane == 0) {
-    // MMA issuer
-    int b = 0;
-    uint32_t acc = 0;
-    bool ok = true;
-    for (int r = task.x; r < task.y && ok; ++r) {
-      const int4 run = runs[r];
-      for (int off = 0; off < run.z; off += kBoxRows, ++b) {
-        const int stage = b % kStages, round = b / kStages;
-        if (!sm100::mbar_wait(&full[stage], round & 1)) {
-          atomicOr(&flags[2], 1);
-          ok = false;
-          break;
-        }
-        sm100::tc_fence_after();
-        const uint8_t* a = sm + stage * 2 * kTileBytes;
-        const uint64_t ad = sm100::sdesc_k_sw128(sm100::smem_u32(a));
-        const uint64_t bd = sm100::sdesc_k_sw128(sm100::smem_u32(diag ? a : a + kTileBytes));
-        const int ksteps = min(kBoxRows, run.z - off) / 16;
-        for (int ks = 0; ks < ksteps; ++ks) {
-          // advance 16 BF16 (32 B) along the contraction inside the swizzle atom
-          sm100::mma_bf16(tmem, ad + 2 * ks, bd + 2 * ks, idesc, acc);
-          acc = 1;
-        }
-        sm100::mma_commit(&empty[stage]);
+    // MMA issuer: task q of this CTA accumulates in TMEM buffer q mod 2
+    const uint32_t idesc = sm100::idesc_bf16_f32(128, N);
+    int st = 0, ph = 0, q = 0;
+    for (int t = t0; t < t1 && ok; ++t, ++q) {
+      const int4 task = tasks[t];
+      const int buf = q & 1;
+      if (!sm100::mbar_wait(&acc_empty[buf], ((q >> 1) & 1) ^ 1)) {
+        ok = false;
+        break;
       }
+      sm100::tc_fence_after();
+      const uint32_t acc_at = tmem + (uint32_t)buf * 128u;
+      uint32_t acc = 0;
+      int next = runs[task.x].z;
+      for (int r = task.x; r < task.y && ok; ++r) {
+        const int len = next;
+        next = runs[min(r + 1, task.y - 1)].z;
+        for (int off = 0; off < len; off += kBoxRows) {
+          if (!sm100::mbar_wait(&full[st], ph)) {
+            ok = false;
+            break;
+          }
+          sm100::tc_fence_after();
+          const uint8_t* a = sm + (size_t)st * 2 * tile_bytes;
+          const uint32_t lead = (uint32_t)block_bytes / 2;   // between the row halves
+          const uint64_t ad = sm100::sdesc_k_plain(sm100::smem_u32(a), lead, 128);
+          const uint64_t bd =
+              sm100::sdesc_k_plain(sm100::smem_u32(task.z ? a : a + tile_bytes), lead, 128);
+          const int ksteps = min(kBoxRows, len - off) / 16;
+          for (int ks = 0; ks < ksteps; ++ks) {
+            const uint64_t step = (uint64_t)(ks * (block_bytes >> 4));
+            sm100::mma_bf16(acc_at, ad + step, bd + step, idesc, acc);
+            acc = 1;
+          }
+          sm100::mma_commit(&empty[st]);
+          if (++st == S) {
+            st = 0;
+            ph ^= 1;
+          }
+        }
+      }
+      sm100::mma_commit(&acc_full[buf]);
     }
     sm100::mma_commit(&done);
+    if (!ok) atomicOr(&flags[2], 1);
+  } else if (warp >= 2) {
+    // epilogue: warp w reads TMEM lanes 32 (w mod 4) .. + 31 (= rows of the block)
+    const int quad = warp & 3, m = 32 * quad + lane;
+    const bool vec = K % 4 == 0;
+    int q = 0;
+    for (int t = t0; t < t1 && ok; ++t, ++q) {
+      const int block = tasks[t].w, buf = q & 1;
+      if (!sm100::mbar_wait(&acc_full[buf], (q >> 1) & 1)) {
+        ok = false;
+        break;
+      }
+      sm100::tc_fence_after();
+      float* out = (block >= 0 ? G + (int64_t)block * K * K : part + (int64_t)~block * K * K) +
+                   (int64_t)m * K;
+      if (32 * quad < K) {
+        for (int c0 = 0; c0 < N; c0 += 16) {
+          uint32_t v[16];
+          sm100::tmem_ld16(tmem + (uint32_t)buf * 128u + ((uint32_t)(32 * quad) << 16) + (uint32_t)c0,
+                           v);
+          sm100::tmem_ld_wait();
+          if (m < K && vec) {
+#pragma unroll
+            for (int j = 0; j < 16; j += 4)
+              if (c0 + j < K)
+                *reinterpret_cast<float4*>(out + c0 + j) =
+                    make_float4(__uint_as_float(v[j]), __uint_as_float(v[j + 1]),
+                                __uint_as_float(v[j + 2]), __uint_as_float(v[j + 3]));
+          } else if (m < K) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              if (c0 + j < K) out[c0 + j] = __uint_as_float(v[j]);
+          }
+          __syncwarp();   // the next load is warp-aligned
+        }
+      }
+      sm100::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) sm100::mbar_arrive(&acc_empty[buf]);
+    }
+    if (!ok && lane == 0) atomicOr(&flags[2], 1);
   }
   __syncwarp();
-  // epilogue: warp w reads TMEM lanes 32w .. 32w+31 (= rows of G_ij)
-  const bool got = sm100::mbar_wait(&done, 0);
-  sm100::tc_fence_after();
-  if (!got && threadIdx.x == 0) atomicOr(&flags[2], 1);
-  const int m = 32 * warp + lane;
-  float* Gp = G + (int64_t)blockIdx.x * K * K;
-  for (int c0 = 0; c0 < N; c0 += 16) {
-    uint32_t v[16];
-    sm100::tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0, v);
-    sm100::tmem_ld_wait();
-    if (m < K) {
-#pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if (c0 + j < K) Gp[(int64_t)m * K + c0 + j] = nboxes > 0 && got ? __uint_as_float(v[j]) : 0.f;
-    }
-  }
+  // every MMA has completed before TMEM is given back
+  if (!sm100::mbar_wait(&done, 0) && threadIdx.x == 0) atomicOr(&flags[2], 1);
   sm100::tc_fence_before();
   __syncthreads();
-  if (warp == 2) sm100::tmem_dealloc(tmem, 128);
+  sm100::tc_fence_after();
+  if (warp == 2) sm100::tmem_dealloc(tmem, 256);
 }
 
-// cuTensorMapEncodeTiled from the driver, resolved at run time through the
-// runtime's entry-point query (the library does not link libcuda directly).
-PFN_cuTensorMapEncodeTiled_v12000 encode_tiled() {
-  // thread-safe one-time lookup (function-local static initialisation)
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      return nullptr;
-    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  }();
-  if (!fn) ELMFB_THROW(ELMFB_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
-  return fn;
+// G of the pairs cut into several tasks: (pair, first partial, partials, -), the
+// partial blocks added in order
+__global__ void __launch_bounds__(256) k_gram_sum(const int4* __restrict__ multi, int KK,
+                                                  const float* __restrict__ part,
+                                                  float* __restrict__ G) {
+  const int4 q = multi[blockIdx.x];
+  const int e = blockIdx.y * 256 + threadIdx.x;
+  if (e >= KK) return;
+  const float* p = part + (int64_t)q.y * KK + e;
+  float v = 0.f;
+#pragma unroll 8
+  for (int c = 0; c < q.z; ++c) v += p[(int64_t)c * KK];
+  G[(int64_t)q.x * KK + e] = v;
+}
+
+// out[n] = Gram block (which[n].x: its index, < 0 a zero block; which[n].y: transposed)
+__global__ void __launch_bounds__(256) k_gram_blocks(const int2* __restrict__ which, int K,
+                                                     const float* __restrict__ G,
+                                                     double* __restrict__ out) {
+  const int2 q = which[blockIdx.x];
+  const int e = blockIdx.y * 256 + threadIdx.x;
+  if (e >= K * K) return;
+  const int a = e / K, b = e - a * K;
+  out[(int64_t)blockIdx.x * K * K + e] =
+      q.x < 0 ? 0.0 : (double)G[(int64_t)q.x * K * K + (q.y ? b * K + a : e)];
 }
 
 }  // namespace
 
-// Build the pair / run lists (host) for the assembled system.
+// Pairs (i <= j) with shared rows, their tasks and the runs of each (host),
+// for the assembled system.
 void gram_build_pairs(elmfb_ctx* h) {
-  struct RunL {
-    int a, b, len;
+  struct Run {
+    int a, b, len, at;   // panel rows of i and j; the place of the run's first cell
   };
-  std::map<std::pair<int, int>, std::vector<RunL>> pr;
-  for (int c = 0; c < h->n_cells; ++c) {
-    if (h->cell_count[c] == 0) continue;
+  // pairs numbered as the cells meet them, then sorted by (i, j)
+  std::unordered_map<uint64_t, int> number;
+  std::vector<uint64_t> keys;
+  std::vector<std::vector<Run>> runs_of;
+  number.reserve(16 * (size_t)h->n_sub);
+  int64_t total = 0;
+  // the cells in square blocks of about 32 MB of panels
+  const double cell_mb = (double)h->NPR * gram_block_bytes(h->K) / 16 / std::max(h->n_cells, 1) / 1e6;
+  const int side = h->dim == 2 ? std::max(1, (int)std::sqrt(32.0 / std::max(cell_mb, 1e-6)))
+                               : std::max(h->nc[0], 1);
+  std::vector<int> visit;
+  visit.reserve(h->n_cells);
+  for (int by = 0; by < h->nc[1]; by += side)
+    for (int bx = 0; bx < h->nc[0]; bx += side)
+      for (int y = by; y < std::min(by + side, h->nc[1]); ++y)
+        for (int x = bx; x < std::min(bx + side, h->nc[0]); ++x)
+          if (h->cell_count[y * h->nc[0] + x] > 0) visit.push_back(y * h->nc[0] + x);
+  for (int at = 0; at < (int)visit.size(); ++at) {
+    const int c = visit[at];
     const int pad = h->cell_pstart[c + 1] - h->cell_pstart[c];
     for (int e1 = h->cover_off[c]; e1 < h->cover_off[c + 1]; ++e1)
       for (int e2 = e1; e2 < h->cover_off[c + 1]; ++e2) {
         const int s1 = h->cover_sub[e1], s2 = h->cover_sub[e2];
         const int a = (int)(h->panel_off[s1] + h->cover_start[e1]);
         const int b = (int)(h->panel_off[s2] + h->cover_start[e2]);
-        auto& v = pr[{s1, s2}];
+        const uint64_t key = ((uint64_t)(uint32_t)s1 << 32) | (uint32_t)s2;
+        const auto [it, fresh] = number.try_emplace(key, (int)keys.size());
+        if (fresh) {
+          keys.push_back(key);
+          runs_of.emplace_back();
+        }
+        auto& v = runs_of[it->second];
         if (!v.empty() && v.back().a + v.back().len == a && v.back().b + v.back().len == b)
           v.back().len += pad;
         else
-          v.push_back({a, b, pad});
+          v.push_back({a, b, pad, at});
+        total += pad;
       }
   }
+  std::vector<int> order(keys.size());
+  std::iota(order.begin(), order.end(), 0);
+  std::sort(order.begin(), order.end(), [&](int x, int y) { return keys[x] < keys[y]; });
   h->gram_pair_ij.clear();
-  std::vector<int4> pairs, runs;
-  for (auto& kv : pr) {
-    pairs.push_back(make_int4((int)runs.size(), (int)(runs.size() + kv.second.size()),
-                              kv.first.first == kv.first.second ? 1 : 0, 0));
-    for (auto& r : kv.second) runs.push_back(make_int4(r.a, r.b, r.len, 0));
-    h->gram_pair_ij.push_back(kv.first);
+  // Rows per task: at most 4096 (64 boxes; at K = 128 a partial block is then 3%
+  // of the operands read for it), fewer where that leaves under 16 tasks a CTA.
+  const int64_t cap = std::min<int64_t>(
+      4096, std::max<int64_t>(256, total / (152 * 16) / kBoxRows * kBoxRows));
+  struct Task {
+    int4 t;
+    int at;
+    int boxes;   // tiles read
+  };
+  std::vector<Task> tasks;
+  std::vector<int4> runs, multi;
+  int n_part = 0;
+  for (size_t p = 0; p < order.size(); ++p) {
+    const uint64_t key = keys[order[p]];
+    h->gram_pair_ij.push_back({(int)(key >> 32), (int)(uint32_t)key});
+    const auto& v = runs_of[order[p]];
+    const int diag = (key >> 32) == (uint32_t)key;
+    const size_t t0 = tasks.size();
+    int64_t rows = cap;   // open a task at the first run
+    for (const Run& r : v)
+      for (int off = 0; off < r.len;) {
+        if (rows >= cap) {
+          tasks.push_back({make_int4((int)runs.size(), 0, diag, 0), r.at, 0});
+          rows = 0;
+        }
+        // a cut inside a run stays on a box
+        const int room = (int)(cap - rows);
+        const int take = r.len - off <= room ? r.len - off
+                                             : std::max(room / kBoxRows * kBoxRows, kBoxRows);
+        const int len = std::min(take, r.len - off);
+        runs.push_back(make_int4(r.a + off, r.b + off, len, 0));
+        tasks.back().t.y = (int)runs.size();
+        tasks.back().boxes += (int)ceil_div(len, kBoxRows) * (2 - diag);
+        off += len;
+        rows += len;
+      }
+    const int n = (int)(tasks.size() - t0);
+    for (int k = 0; k < n; ++k) tasks[t0 + k].t.w = n == 1 ? (int)p : ~(n_part + k);
+    if (n > 1) {
+      multi.push_back(make_int4((int)p, n_part, n, 0));
+      n_part += n;
+    }
   }
-  h->n_gram_pairs = (int64_t)pairs.size();
-  h->gram_runs = (int64_t)runs.size();
+  std::stable_sort(tasks.begin(), tasks.end(),
+                   [](const Task& x, const Task& y) { return x.at < y.at; });
+  int sms = 0;
+  CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+  const int ctas = (int)std::min<size_t>(tasks.size(), sms);
+  std::vector<int> owner(tasks.size()), task_off(ctas + 1, 0);
+  {
+    typedef std::pair<int64_t, int> Load;   // tiles so far, CTA
+    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> idle;
+    for (int c = 0; c < ctas; ++c) idle.push({0, c});
+    for (size_t k = 0; k < tasks.size(); ++k) {
+      const Load l = idle.top();
+      idle.pop();
+      owner[k] = l.second;
+      task_off[l.second + 1]++;
+      idle.push({l.first + tasks[k].boxes + 8, l.second});   // 8: a task's own cost
+    }
+    for (int c = 0; c < ctas; ++c) task_off[c + 1] += task_off[c];
+  }
+  std::vector<int4> flat(tasks.size());
+  {
+    std::vector<int> fill(task_off.begin(), task_off.end() - 1);
+    for (size_t k = 0; k < tasks.size(); ++k) flat[fill[owner[k]]++] = tasks[k].t;
+  }
+  h->d_gram_task_off.alloc(task_off.size() * sizeof(int), h->stream);
+  CUDA_CHECK(cudaMemcpyAsync(h->d_gram_task_off.p, task_off.data(), task_off.size() * sizeof(int),
+                             cudaMemcpyHostToDevice, h->stream));
+  h->gram_ctas = ctas;
+  h->n_gram_pairs = (int64_t)order.size();
+  h->gram_multi = (int)multi.size();
+  h->gram_parts = n_part;
   auto up = [&](DevBuf& d, const std::vector<int4>& v) {
     d.alloc(std::max<size_t>(v.size(), 1) * sizeof(int4), h->stream);
     if (!v.empty())
       CUDA_CHECK(cudaMemcpyAsync(d.p, v.data(), v.size() * sizeof(int4), cudaMemcpyHostToDevice,
                                  h->stream));
   };
-  up(h->d_gram_pairs, pairs);
+  up(h->d_gram_tasks, flat);
   up(h->d_gram_runs, runs);
+  up(h->d_gram_multi, multi);
 }
 
 void gram_compute(elmfb_ctx* h) {
@@ -216,28 +400,25 @@ void gram_compute(elmfb_ctx* h) {
   const int K = h->K;
   const int N = (K + 15) & ~15;
   h->d_gram.alloc(std::max<int64_t>(h->n_gram_pairs, 1) * K * K * sizeof(float), st);
-  // tensor map over PT[K][NPR] (BF16, rows innermost)
-  CUtensorMap tm;
-  cuuint64_t gdim[2] = {(cuuint64_t)h->NPR, (cuuint64_t)K};
-  cuuint64_t gstride[1] = {(cuuint64_t)h->NPR * 2};
-  cuuint32_t box[2] = {(cuuint32_t)kBoxRows, (cuuint32_t)K};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = encode_tiled()(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, h->d_pt.p, gdim,
-                                      gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                      CU_TENSOR_MAP_SWIZZLE_128B,
-                                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS)
-    ELMFB_THROW(ELMFB_ERR_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
+  DevBuf dpart;
+  dpart.alloc((size_t)h->gram_parts * K * K * sizeof(float), st);
   ensure_dyn_smem((const void*)k_gram_tc, kGramSmem);
   CUDA_CHECK(cudaMemsetAsync(h->d_flags.p, 0, 16 * sizeof(int), st));
   stage_begin(h, 3);
   // algorithmic work: 2 K^2 flops per shared row per pair; bytes: BF16 rows read once
   prof_begin(h, KID_GRAM_TC, (double)h->NPR * K * 2.0 + (double)h->n_gram_pairs * K * K * 4.0);
-  if (h->n_gram_pairs > 0)
-    k_gram_tc<<<(unsigned)h->n_gram_pairs, kGramThreads, kGramSmem, st>>>(
-        tm, h->d_gram_pairs.as<int4>(), h->d_gram_runs.as<int4>(), K, N, h->d_gram.as<float>(),
+  if (h->gram_ctas > 0) {
+    const int S = (int)std::min<size_t>(kMaxGramStages, kGramRing / (2 * gram_tile_bytes(K)));
+    k_gram_tc<<<(unsigned)h->gram_ctas, kGramThreads, kGramSmem, st>>>(
+        h->d_pt.as<uint8_t>(), h->d_gram_tasks.as<int4>(), h->d_gram_task_off.as<int>(),
+        h->d_gram_runs.as<int4>(), K, N, S, h->d_gram.as<float>(), dpart.as<float>(),
         h->d_flags.as<int>());
+    if (h->gram_multi > 0) {
+      k_gram_sum<<<dim3((unsigned)h->gram_multi, (unsigned)ceil_div(K * K, 256)), 256, 0, st>>>(
+          h->d_gram_multi.as<int4>(), K * K, dpart.as<float>(), h->d_gram.as<float>());
+      count_launch(h);
+    }
+  }
   prof_end(h, KID_GRAM_TC);
   check_launch("k_gram_tc");
   count_launch(h);
@@ -279,23 +460,34 @@ int elmfb_get_gram(elmfb_t h, int64_t n, const int* ij, double* out) {
     const int K = h->K;
     std::vector<int> hij(2 * n);
     CUDA_CHECK(cudaMemcpy(hij.data(), ij, 2 * n * sizeof(int), cudaMemcpyDefault));
-    std::vector<float> blk((size_t)K * K);
-    std::vector<double> res((size_t)n * K * K, 0.0);
+    if (n == 0) return ELMFB_OK;
+    std::vector<int2> which(n);
     for (int64_t q = 0; q < n; ++q) {
       int i = hij[2 * q], j = hij[2 * q + 1];
-      bool tr = i > j;
+      const bool tr = i > j;
       if (tr) std::swap(i, j);
       auto it = std::lower_bound(h->gram_pair_ij.begin(), h->gram_pair_ij.end(),
                                  std::make_pair(i, j));
-      if (it == h->gram_pair_ij.end() || *it != std::make_pair(i, j)) continue;   // zero block
-      const int64_t p = it - h->gram_pair_ij.begin();
-      CUDA_CHECK(cudaMemcpy(blk.data(), h->d_gram.as<float>() + p * K * K, K * K * sizeof(float),
-                            cudaMemcpyDeviceToHost));
-      for (int a = 0; a < K; ++a)
-        for (int b = 0; b < K; ++b)
-          res[(size_t)q * K * K + a * K + b] = tr ? blk[b * K + a] : blk[a * K + b];
+      const bool found = it != h->gram_pair_ij.end() && *it == std::make_pair(i, j);
+      which[q] = make_int2(found ? (int)(it - h->gram_pair_ij.begin()) : -1, tr);
     }
-    CUDA_CHECK(cudaMemcpy(out, res.data(), res.size() * sizeof(double), cudaMemcpyDefault));
+    // in place in device memory, else through a staging buffer
+    cudaStream_t st = h->stream;
+    const size_t bytes = (size_t)n * K * K * sizeof(double);
+    DevBuf dw, dout;
+    dw.alloc(n * sizeof(int2), st);
+    CUDA_CHECK(cudaMemcpyAsync(dw.p, which.data(), n * sizeof(int2), cudaMemcpyHostToDevice, st));
+    double* o = out;
+    if (!usable_in_place(h, out, sizeof(double))) {
+      dout.alloc(bytes, st);
+      o = dout.as<double>();
+    }
+    k_gram_blocks<<<dim3((unsigned)n, (unsigned)ceil_div(K * K, 256)), 256, 0, st>>>(
+        dw.as<int2>(), K, h->d_gram.as<float>(), o);
+    check_launch("k_gram_blocks");
+    count_launch(h);
+    if (dout.p) CUDA_CHECK(cudaMemcpyAsync(out, dout.p, bytes, cudaMemcpyDefault, st));
+    stream_sync(h);
     return ELMFB_OK;
   } catch (const elmfb_error& e) {
     h->err = e.msg;

@@ -1,5 +1,5 @@
 // Inline-PTX helpers for the Blackwell (sm_100 family, here sm_103a) async
-// machinery used by the tensor-core kernels: mbarriers, TMA tensor loads,
+// machinery used by the tensor-core kernels: mbarriers, bulk copies,
 // TMEM allocation, tcgen05.mma / commit / ld.  Every wait is bounded: after
 // kSpinLimit polls it gives up and reports failure to the caller.
 #pragma once
@@ -54,14 +54,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
 }
 
 // ---------------------------------------------------------------- TMA
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int32_t x,
-                                            int32_t y, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-      : "memory");
-}
 // 1-D bulk copy global -> shared, completing `bytes` on the mbarrier
 // (addresses 16-byte aligned, size a multiple of 16)
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes,
@@ -93,9 +85,6 @@ __device__ __forceinline__ void bulk_load_hint(void* dst, const void* src, uint3
 // later async-proxy (bulk copy) accesses
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
 // ---------------------------------------------------------------- TMEM
@@ -130,6 +119,17 @@ __device__ __forceinline__ uint64_t sdesc_k_sw128(uint32_t saddr) {
   d |= (uint64_t)(1024u >> 4) << 32;
   d |= 1ull << 46;
   d |= 2ull << 61;
+  return d;
+}
+// The same without swizzle: core matrices of 8 rows x 16 bytes, contiguous;
+// `lead` bytes between neighbours along the contraction, `stride` bytes between
+// neighbours along the rows.
+__device__ __forceinline__ uint64_t sdesc_k_plain(uint32_t saddr, uint32_t lead, uint32_t stride) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+  d |= (uint64_t)((lead >> 4) & 0x3FFFu) << 16;
+  d |= (uint64_t)((stride >> 4) & 0x3FFFu) << 32;
+  d |= 1ull << 46;
   return d;
 }
 // Instruction descriptor, kind::f16: FP32 accumulate (bits 4-5 = 1), A and B

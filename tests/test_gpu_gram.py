@@ -76,3 +76,32 @@ def test_gram_unsupported_outside_mixed_precision():
         with pytest.raises(E.ElmfbError) as ei:
             s.compute_gram()
         assert ei.value.code == E.ERR_UNSUPPORTED
+
+
+# K below one MMA's granularity, ragged against 4, 8 and 16, and the largest; the
+# level-1 subdomain's rows span several tasks, a (1,)-level problem is one pair
+@pytest.mark.parametrize("levels,K,side", [((1,), 1, 9), ((1, 3), 17, 30), ((1, 2, 4), 100, 50),
+                                           ((5,), 36, 41), ((1, 2), 128, 33)])
+def test_gram_blocks_of_cut_pairs(levels, K, side):
+    """Every block, asked for in either order and into host or device memory,
+    with a pair that shares no rows, against BF16-rounded products in FP64
+    (bound of the module's first reference)."""
+    torch = pytest.importorskip("torch")
+    P = WL.poisson2d(levels=levels, features=K, n_side=side, n_boundary_side=side)
+    M = OS.assemble(P, fmt="dense")["M"]
+    Mb, A, nsub = _bf16(M), np.abs(M), P.n_subdomains
+    pairs = [(i, j) if (i + j) % 2 else (j, i) for i in range(nsub) for j in range(i, nsub)]
+    with E.Solver.from_problem(P, precision=E.MIXED) as s:
+        s.assemble_problem(P)
+        s.compute_gram()
+        got = s.gram_blocks(pairs)
+        p = np.array(pairs, dtype=np.int32)
+        dev = torch.empty((len(p), K, K), dtype=torch.float64, device="cuda")
+        assert E.lib().elmfb_get_gram(s.h, len(p), p.ctypes.data, dev.data_ptr()) == E.OK
+        s.compute_gram()   # the plan is kept, the blocks are the same
+        again = s.gram_blocks(pairs)
+    assert np.array_equal(dev.cpu().numpy(), got) and np.array_equal(again, got)
+    for q, (i, j) in enumerate(pairs):
+        bi, bj = slice(i * K, (i + 1) * K), slice(j * K, (j + 1) * K)
+        assert np.all(np.abs(got[q] - Mb[:, bi].T @ Mb[:, bj]) <=
+                      2.0 ** -9 * (A[:, bi].T @ A[:, bj]))
