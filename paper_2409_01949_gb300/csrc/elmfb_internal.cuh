@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <cstring>
 #include <functional>
 #include <string>
 #include <vector>
@@ -43,17 +45,19 @@ struct DevBuf {
   void* p = nullptr;
   size_t bytes = 0;
   cudaStream_t s = nullptr;
+  bool own = true;   // false: a part of another buffer (Upload)
   DevBuf() = default;
   DevBuf(const DevBuf&) = delete;
   DevBuf& operator=(const DevBuf&) = delete;
   ~DevBuf() { release(); }
   void release() {
-    if (p) cudaFreeAsync(p, s);
+    if (p && own) cudaFreeAsync(p, s);
     p = nullptr;
     bytes = 0;
+    own = true;
   }
   void alloc(size_t n, cudaStream_t stream) {
-    if (n <= bytes && p) return;
+    if (n <= bytes && p && own) return;
     release();
     s = stream;
     if (n == 0) return;
@@ -67,6 +71,36 @@ struct DevBuf {
 // rows 16 q .. 16 q + 15, all of one cell) are one block, element (feature k, row
 // r) at byte (r / 8) (block / 2) + (k / 8) 128 + (k % 8) 16 + (r % 8) 2.
 __host__ __device__ constexpr int gram_block_bytes(int K) { return ((K + 7) & ~7) * 32; }
+
+// Several host arrays uploaded as one copy into one buffer, each buffer added
+// becoming a part of it: a copy of a small pageable array costs 5 us of host time
+// whatever its size.  The parts are valid until the owner is sent or released again.
+struct Upload {
+  struct Part {
+    DevBuf* to;
+    size_t at, bytes;
+  };
+  std::vector<char> host;
+  std::vector<Part> parts;
+  template <class T>
+  void add(DevBuf& to, const T* src, size_t n) {
+    const size_t at = (host.size() + 15) & ~size_t(15), bytes = n * sizeof(T);
+    host.resize(at + std::max<size_t>(bytes, 16));
+    if (bytes) std::memcpy(host.data() + at, src, bytes);
+    parts.push_back({&to, at, bytes});
+  }
+  void send(DevBuf& owner, cudaStream_t stream) {
+    owner.alloc(host.size(), stream);
+    CUDA_CHECK(cudaMemcpyAsync(owner.p, host.data(), host.size(), cudaMemcpyHostToDevice, stream));
+    for (const Part& q : parts) {
+      q.to->release();
+      q.to->p = static_cast<char*>(owner.p) + q.at;
+      q.to->bytes = q.bytes;
+      q.to->s = stream;
+      q.to->own = false;
+    }
+  }
+};
 
 // Row padding of a cell of the common refinement and the row-class limit.
 constexpr int kCellPad = 16;            // cell row groups are padded to this multiple
@@ -180,6 +214,7 @@ struct elmfb_ctx {
   int64_t n_gram_pairs = 0;
   double gram_flops = 0.0;
 
+  DevBuf d_layout;      // owner of the layout tables below (cls .. entry_base)
   DevBuf d_pts_user, d_rhs_user, d_cls_user;  // user order
   DevBuf d_cls;                                 // [kMaxClasses] RowClass table
   DevBuf d_row_cell, d_cell_count, d_cell_pstart;
@@ -300,7 +335,8 @@ struct __align__(8) df2 {
 };
 
 struct FusedPlan {
-  DevBuf units, fo, fe, part;
+  DevBuf lists;         // owner of units, fe, pch, pco
+  DevBuf units, fe, part;
   DevBuf tf;            // FP32 copy of t for FP32 panels
   DevBuf pch, pco, csum;   // per-panel slices of the partial list and their sums
   int n_pchunks = 0;

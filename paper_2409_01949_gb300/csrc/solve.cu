@@ -2374,18 +2374,6 @@ struct SolveLayout {
 
 // Heuristic rows per fused-pass work unit (see build_fused_plan).
 int64_t fused_unit_target(const elmfb_ctx* h) {
-  const double row_bytes =
-      (double)h->NPR / (double)std::max<int64_t>(h->NR, 1) * h->K * (double)h->panel_elem();
-  const int64_t by_bytes = (int64_t)((2.0 * 1024 * 1024) / std::max(row_bytes, 1.0));
-  return std::min<int64_t>(
-      kMaxUnitRows, std::max<int64_t>(8, std::max(h->NR / 608, by_bytes) & ~int64_t(7)));
-}
-
-bool build_fused_plan(elmfb_ctx* h, FusedPlan& fp, int unit_rows) {
-  const int K = h->K;
-  if (h->max_cover > 32 || K > 128) return false;
-  cudaStream_t st = h->stream;
-  fp.threads = 32 * std::max(1, h->max_cover);
   // rows per work unit: about NR / 608 (4 waves of one-CTA-per-SM units), but
   // at least the rows of about 2 MB of covering panels, so that a unit's
   // start-up (barrier set-up, the first copies in flight) stays small next to
@@ -2395,10 +2383,19 @@ bool build_fused_plan(elmfb_ctx* h, FusedPlan& fp, int unit_rows) {
   // tuning knob: units change the timing and the grouping of the Mᵀu partial
   // sums, not the order of the terms within a row)
   const double row_bytes =
-      (double)h->NPR / (double)std::max<int64_t>(h->NR, 1) * K * (double)h->panel_elem();
+      (double)h->NPR / (double)std::max<int64_t>(h->NR, 1) * h->K * (double)h->panel_elem();
   const int64_t by_bytes = (int64_t)((2.0 * 1024 * 1024) / std::max(row_bytes, 1.0));
-  int64_t target = std::min<int64_t>(
+  const int64_t target = std::min<int64_t>(
       kMaxUnitRows, std::max<int64_t>(8, std::max(h->NR / 608, by_bytes) & ~int64_t(7)));
+  return target;
+}
+
+bool build_fused_plan(elmfb_ctx* h, FusedPlan& fp, int unit_rows) {
+  const int K = h->K;
+  if (h->max_cover > 32 || K > 128) return false;
+  cudaStream_t st = h->stream;
+  fp.threads = 32 * std::max(1, h->max_cover);
+  int64_t target = fused_unit_target(h);   // rows per work unit
   if (const char* e = getenv("ELMFB_FUSED_UNIT_ROWS")) {
     const long v = atol(e);
     if (v >= 8 && v <= kMaxUnitRows) target = v & ~7L;
@@ -2429,9 +2426,9 @@ bool build_fused_plan(elmfb_ctx* h, FusedPlan& fp, int unit_rows) {
     fe.insert(fe.end(), plist[s2].begin(), plist[s2].end());
   }
   fo[h->n_sub] = (int)fe.size();
-  fp.units.alloc(std::max<size_t>(units.size(), 1) * sizeof(int4), st);
-  fp.fo.alloc(fo.size() * sizeof(int), st);
-  fp.fe.alloc(std::max<size_t>(fe.size(), 1) * sizeof(int), st);
+  Upload lists;
+  lists.add(fp.units, units.data(), units.size());
+  lists.add(fp.fe, fe.data(), fe.size());
   fp.part.alloc(std::max<int64_t>(pbase, 1) * K * sizeof(double), st);
   fp.pairs = !h->fp64();
   // fixed slices of at most kPanelChunk partials per panel: the big panels of
@@ -2447,23 +2444,13 @@ bool build_fused_plan(elmfb_ctx* h, FusedPlan& fp, int unit_rows) {
     }
     pco[h->n_sub] = (int)pch.size();
     fp.n_pchunks = (int)pch.size();
-    fp.pch.alloc(std::max<size_t>(pch.size(), 1) * sizeof(int2), st);
-    fp.pco.alloc(pco.size() * sizeof(int), st);
+    lists.add(fp.pch, pch.data(), pch.size());
+    lists.add(fp.pco, pco.data(), pco.size());
     fp.csum.alloc(std::max<size_t>(pch.size(), 1) * K * sizeof(double), st);
-    if (!pch.empty())
-      CUDA_CHECK(cudaMemcpyAsync(fp.pch.p, pch.data(), pch.size() * sizeof(int2),
-                                 cudaMemcpyHostToDevice, st));
-    CUDA_CHECK(cudaMemcpyAsync(fp.pco.p, pco.data(), pco.size() * sizeof(int),
-                               cudaMemcpyHostToDevice, st));
   }
+  lists.send(fp.lists, st);
   if (fp.pairs)
     fp.tf.alloc(std::max<int64_t>(h->NPhi, 1) * (h->df32() ? sizeof(float2) : sizeof(float)), st);
-  CUDA_CHECK(cudaMemcpyAsync(fp.units.p, units.data(), units.size() * sizeof(int4),
-                             cudaMemcpyHostToDevice, st));
-  CUDA_CHECK(cudaMemcpyAsync(fp.fo.p, fo.data(), fo.size() * sizeof(int), cudaMemcpyHostToDevice,
-                             st));
-  CUDA_CHECK(cudaMemcpyAsync(fp.fe.p, fe.data(), fe.size() * sizeof(int), cudaMemcpyHostToDevice,
-                             st));
   return true;
 }
 
@@ -2993,28 +2980,13 @@ void lsqr(elmfb_ctx* h, const elmfb_solve_opts* o, elmfb_solve_info* info) {
   info->precond_retries = h->bj_retries;
   info->precond_dropped = h->bj_dropped;
 
-  // panel -> entries (cell order)
   const int ne = (int)h->cover_sub.size();
-  std::vector<int> pent_off(h->n_sub + 1, 0), pent(ne);
-  for (int e = 0; e < ne; ++e) pent_off[h->cover_sub[e] + 1]++;
-  for (int s = 0; s < h->n_sub; ++s) pent_off[s + 1] += pent_off[s];
-  {
-    std::vector<int> fill(pent_off.begin(), pent_off.end() - 1);
-    for (int e = 0; e < ne; ++e) pent[fill[h->cover_sub[e]]++] = e;
-  }
-  DevBuf dpo, dpe;
-  dpo.alloc(pent_off.size() * sizeof(int), st);
-  dpe.alloc(std::max(ne, 1) * sizeof(int), st);
-  CUDA_CHECK(cudaMemcpyAsync(dpo.p, pent_off.data(), pent_off.size() * sizeof(int),
-                             cudaMemcpyHostToDevice, st));
-  CUDA_CHECK(cudaMemcpyAsync(dpe.p, pent.data(), ne * sizeof(int), cudaMemcpyHostToDevice, st));
-
+  DevBuf dpo, dpe;   // panel -> entries (cell order); the fused pass needs none
   h->d_u.alloc(h->NR * sizeof(double), st);
   h->d_v.alloc(N * sizeof(double), st);
   h->d_w.alloc(N * sizeof(double), st);
   h->d_x_sol.alloc(N * sizeof(double), st);
   h->d_tmp.alloc(std::max<int64_t>(N, h->NR) * sizeof(double), st);
-  h->d_partial.alloc((int64_t)ne * K * sizeof(double), st);
   // scalar slots, then the Golub-Kahan record (alpha, beta) of steps 0..max_iter
   const int gk_cap = o->max_iter + 1;
   h->d_scal.alloc((2 * kScal + 2 * (size_t)gk_cap) * sizeof(double), st);
@@ -3022,15 +2994,6 @@ void lsqr(elmfb_ctx* h, const elmfb_solve_opts* o, elmfb_solve_info* info) {
   double* gpart = h->d_ptile.as<double>();
   double* vpart = gpart + kGatherBlocks;
   const double panel_bytes = (double)h->NPR * K * sizeof(T);
-  CUDA_CHECK(cudaMemsetAsync(h->d_scal.p, 0, 2 * kScal * sizeof(double), st));
-  {
-    const double cap_d = (double)gk_cap;   // pageable: staged before the call returns
-    CUDA_CHECK(cudaMemcpyAsync(h->d_scal.as<double>() + S_GKCAP, &cap_d, sizeof(double),
-                               cudaMemcpyHostToDevice, st));
-    CUDA_CHECK(cudaMemcpyAsync(h->d_scal.as<double>() + kStage + S_GKCAP, &cap_d, sizeof(double),
-                               cudaMemcpyHostToDevice, st));
-  }
-
   const T* P = (const T*)h->d_panels.p;
   double* scal = h->d_scal.as<double>();
   const double* Xr = h->d_R.as<double>();
@@ -3081,6 +3044,21 @@ void lsqr(elmfb_ctx* h, const elmfb_solve_opts* o, elmfb_solve_info* info) {
   const int tuned_rows = o->autotune && h->max_cover <= 32 && K <= 128
                              ? autotune_unit_rows<T>(h) : 0;
   const bool fused = build_fused_plan(h, fp, tuned_rows);
+  if (!fused) {
+    std::vector<int> pent_off(h->n_sub + 1, 0), pent(ne);
+    for (int e = 0; e < ne; ++e) pent_off[h->cover_sub[e] + 1]++;
+    for (int s = 0; s < h->n_sub; ++s) pent_off[s + 1] += pent_off[s];
+    {
+      std::vector<int> fill(pent_off.begin(), pent_off.end() - 1);
+      for (int e = 0; e < ne; ++e) pent[fill[h->cover_sub[e]]++] = e;
+    }
+    dpo.alloc(pent_off.size() * sizeof(int), st);
+    dpe.alloc(std::max(ne, 1) * sizeof(int), st);
+    CUDA_CHECK(cudaMemcpyAsync(dpo.p, pent_off.data(), pent_off.size() * sizeof(int),
+                               cudaMemcpyHostToDevice, st));
+    CUDA_CHECK(cudaMemcpyAsync(dpe.p, pent.data(), ne * sizeof(int), cudaMemcpyHostToDevice, st));
+    h->d_partial.alloc((int64_t)ne * K * sizeof(double), st);
+  }
   DevBuf& dfpart = fp.part;
   const int n_units = fp.n_units;
   if (fused) {
@@ -3116,11 +3094,16 @@ void lsqr(elmfb_ctx* h, const elmfb_solve_opts* o, elmfb_solve_info* info) {
     CUDA_CHECK(cudaMemsetAsync(h->d_x_sol.p, 0, N * sizeof(double), st));
   }
   const int fmode = xpairs ? 2 : 0;              // the loop's fused-pass mode
-  if (xpairs) {   // the stopping tests run on the device too (lsqr_recurrence)
-    const double sp[4] = {1.0, o->ntol, o->btol, o->atol};   // S_STOP_ON .. S_ATOL
-    CUDA_CHECK(cudaMemcpyAsync(scal + S_STOP_ON, sp, sizeof(sp), cudaMemcpyHostToDevice, st));
-    CUDA_CHECK(cudaMemcpyAsync(scal + kStage + S_STOP_ON, sp, sizeof(sp), cudaMemcpyHostToDevice,
-                               st));
+  {   // the scalars' start, committed and staged, in one copy
+    double init[2 * kScal] = {};
+    for (int at : {0, kStage}) {
+      init[at + S_GKCAP] = (double)gk_cap;
+      if (xpairs) {   // the stopping tests run on the device too (lsqr_recurrence)
+        const double sp[4] = {1.0, o->ntol, o->btol, o->atol};   // S_STOP_ON .. S_ATOL
+        for (int i = 0; i < 4; ++i) init[at + S_STOP_ON + i] = sp[i];
+      }
+    }
+    CUDA_CHECK(cudaMemcpyAsync(scal, init, sizeof(init), cudaMemcpyHostToDevice, st));
   }
   const int tail_launches = xpairs ? 1 : 2;      // besides the slice sums (counted by themselves)
   auto fused_tail = [&](int init) {

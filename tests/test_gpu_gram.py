@@ -105,3 +105,23 @@ def test_gram_blocks_of_cut_pairs(levels, K, side):
         bi, bj = slice(i * K, (i + 1) * K), slice(j * K, (j + 1) * K)
         assert np.all(np.abs(got[q] - Mb[:, bi].T @ Mb[:, bj]) <=
                       2.0 ** -9 * (A[:, bi].T @ A[:, bj]))
+
+
+@pytest.mark.parametrize("make", [
+    lambda: WL.poisson1d(levels=(1, 3, 5), features=4, n_interior=90),
+    lambda: WL.poisson1d(levels=(7,), features=4, n_interior=5, delta=2.9),       # empty cells
+    lambda: WL.poisson2d(levels=(1, 2, 4, 8), features=4, n_side=40),
+    lambda: WL.poisson2d(levels=(3, 5), features=4, n_side=24, delta=1.4),
+    lambda: WL.poisson2d(levels=(2, 6), features=4, n_side=5, delta=2.9),         # empty cells
+    lambda: WL.helmholtz_lshape(levels=(1, 8), features=4, n_grid=20),            # discarded subdomains
+    lambda: WL.laplace_multiscale(levels=(1, 4, 6), features=4, n_grid=30, placement="endpoint"),
+])
+def test_pair_count_before_and_after_the_gram_blocks(make):
+    """sizes() counts the pairs of subdomains that share a cell with points
+    without forming them; the blocks' own list has the same number."""
+    P = make()
+    with E.Solver.from_problem(P, precision=E.MIXED) as s:
+        s.assemble_problem(P)
+        n = s.sizes().n_gram_pairs
+        s.compute_gram()
+        assert s.sizes().n_gram_pairs == n
