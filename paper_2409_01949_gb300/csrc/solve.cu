@@ -2387,7 +2387,17 @@ int64_t fused_unit_target(const elmfb_ctx* h) {
   const int64_t by_bytes = (int64_t)((2.0 * 1024 * 1024) / std::max(row_bytes, 1.0));
   const int64_t target = std::min<int64_t>(
       kMaxUnitRows, std::max<int64_t>(8, std::max(h->NR / 608, by_bytes) & ~int64_t(7)));
-  return target;
+  // A small FP64-accurate problem whose cells would leave most SMs without a
+  // unit: about one unit per SM instead (1-D Poisson, 33 cells of 64 rows: 132
+  // units of 16 rows; a solve of four steps 449 -> 292 us).  FP32 panels keep
+  // their grouping: their iterates carry the panels' rounding, and another
+  // grouping of the partial sums moves them by as much.
+  if (h->panel_elem() != 8) return target;
+  int64_t units = 0;
+  for (int c = 0; c < h->n_cells; ++c)
+    units += ceil_div(h->cell_pstart[c + 1] - h->cell_pstart[c], target);
+  if (2 * units >= 152) return target;
+  return std::min(target, (ceil_div(h->NR, 152) + 7) & ~int64_t(7));
 }
 
 bool build_fused_plan(elmfb_ctx* h, FusedPlan& fp, int unit_rows) {
