@@ -17,10 +17,10 @@
 //
 // Layout: A is column-major FP64 [ld x (n+1)], ld >= m = the padded sorted
 // rows (padding rows are zero rows and change nothing), column n = h.  One
-// step is two kernels: k_qr_house (one block: pivot swap, reflector) and
-// k_qr_apply (a warp per column: v^T A_j, the update, the new norm, and the
-// arg-max of the norms for the next step, finished by the last block).  The
-// update is FP64-bound: three FP64 FMAs per trailing entry and step.
+// step is one kernel, k_qr_apply: a warp per column forms v^T A_j, the update and
+// the new norm; the last block to finish takes the arg-max of the norms, swaps
+// the next pivot into place and forms its reflector.  The update is FP64-bound:
+// three FP64 FMAs per trailing entry and step.
 #include <algorithm>
 #include <cmath>
 
@@ -29,7 +29,8 @@
 namespace {
 
 constexpr int kApplyThreads = 256;   // 8 warps, a warp per column
-constexpr int kHouseThreads = 1024;
+constexpr int kHouseVirtual = 1024;  // partial sums of a reflector's norm
+constexpr int kRegRows = 64;         // rows a lane may hold of its column (2048 rows)
 constexpr int kQrBatch = 32;         // steps launched between host checks of the stop flag
 
 struct QrState {
@@ -115,8 +116,9 @@ __global__ void k_qr_copy_h(const double* __restrict__ hv, int64_t m, double* __
 
 // The block's best (norm, column) into part[blockIdx]; the last block to
 // finish reduces all partials (the order does not matter: "better" is a total
-// order) into the state.  `lo` is the first candidate column.
-__device__ void argmax_finish(double bv, int bi, double* __restrict__ part_v,
+// order) into the state and returns true, with every block's writes visible
+// (read them past L1).  `lo` is the first candidate column.
+__device__ bool argmax_finish(double bv, int bi, double* __restrict__ part_v,
                               int* __restrict__ part_i, unsigned int* __restrict__ counter,
                               QrState* st, int lo) {
   __shared__ double sv[32];
@@ -142,10 +144,12 @@ __device__ void argmax_finish(double bv, int bi, double* __restrict__ part_v,
     last = atomicAdd(counter, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  if (!last) return;
+  if (!last) return false;
+  __threadfence();
   if (wid == 0) {
     double v = -1.0;
     int i = -1;
+#pragma unroll 4
     for (int b = lane; b < (int)gridDim.x; b += 32) {
       const double pv = __ldcg(part_v + b);
       const int pi = __ldcg(part_i + b);
@@ -169,13 +173,115 @@ __device__ void argmax_finish(double bv, int bi, double* __restrict__ part_v,
       *counter = 0u;
     }
   }
+  __syncthreads();
+  return true;
+}
+
+// Pivot swap and the Householder reflector of column k, by the last block of the
+// kernel that finished step k - 1 (kApplyThreads threads; the norm is summed as 1024
+// strided partial sums, 32 at a time, whatever the block's size).
+__device__ void house_step(double* __restrict__ A, int64_t ld, int64_t m, int k,
+                           double* __restrict__ cn, int* __restrict__ perm,
+                           double* __restrict__ vbuf, QrState* __restrict__ st, double rcond) {
+  __shared__ double part[kHouseVirtual / 32];
+  __shared__ int s_go, s_j;
+  if (threadIdx.x == 0) {
+    int go = !__ldcg(&st->stop);
+    if (go) {
+      const int j = __ldcg(&st->piv);
+      const double cj = __ldcg(&st->cmax);
+      if (k == 0) st->r11 = sqrt(cj);
+      if (__ldcg(&st->bad) != 0.0 || !(cj > 0.0) || sqrt(cj) <= rcond * __ldcg(&st->r11)) {
+        st->stop = 1;
+        st->rank = k;
+        go = 0;
+      } else {
+        s_j = j;
+        if (j != k) {
+          cn[j] = __ldcg(cn + k);
+          const int t = perm[j];
+          perm[j] = perm[k];
+          perm[k] = t;
+        }
+      }
+    }
+    s_go = go;
+  }
+  __syncthreads();
+  if (!s_go) return;
+  const int j = s_j;
+  double* ck = A + (int64_t)k * ld;
+  double* cj = A + (int64_t)j * ld;
+  const int lane = threadIdx.x & 31;
+  // rows above k of both columns are final rows of R: swapped as they are
+  if (j != k)
+#pragma unroll 4
+    for (int64_t i = threadIdx.x; i < k; i += blockDim.x) {
+      const double t = __ldcg(ck + i), u = __ldcg(cj + i);
+      ck[i] = u;
+      cj[i] = t;
+    }
+  // row k by one thread, the rest in the order of the partial sums
+  __shared__ double s_alpha;
+  if (threadIdx.x == 0) {
+    const double t = __ldcg(ck + k), x = __ldcg(cj + k);
+    if (j != k) cj[k] = t;
+    s_alpha = j != k ? x : t;
+  }
+  // partial sum v = thread + 256 q takes rows k + 1 + v + 1024 p in order; the
+  // loads of two p are in flight together
+  constexpr int kQ = kHouseVirtual / kApplyThreads;
+  double s1[kQ] = {};
+  for (int64_t base = k + 1 + threadIdx.x; base < m; base += 2 * kHouseVirtual) {
+    double x[2][kQ], y[2][kQ];
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+      for (int q = 0; q < kQ; ++q) {
+        const int64_t i = base + p * kHouseVirtual + q * kApplyThreads;
+        x[p][q] = i < m ? __ldcg(cj + i) : 0.0;
+        y[p][q] = i < m ? __ldcg(ck + i) : 0.0;
+      }
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+      for (int q = 0; q < kQ; ++q) {
+        const int64_t i = base + p * kHouseVirtual + q * kApplyThreads;
+        if (i >= m) continue;
+        if (j != k) {
+          cj[i] = y[p][q];
+          ck[i] = x[p][q];
+        }
+        s1[q] = fma(x[p][q], x[p][q], s1[q]);
+        vbuf[i] = x[p][q];
+      }
+  }
+#pragma unroll
+  for (int q = 0; q < kQ; ++q) {
+    const double w = warp_sum_d(s1[q]);
+    if (lane == 0) part[(threadIdx.x + q * kApplyThreads) >> 5] = w;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const double s1 = warp_sum_d(part[lane]);
+    if (lane == 0) {
+      const double alpha = s_alpha;
+      const double beta = -copysign(sqrt(fma(alpha, alpha, s1)), alpha);
+      const double v0 = alpha - beta;
+      vbuf[k] = v0;
+      ck[k] = beta;
+      st->c = 2.0 / fma(v0, v0, s1);
+      st->rank = k + 1;
+      if (!(beta == beta) || isinf(beta)) st->bad = 1.0;
+    }
+  }
 }
 
 // squared column norms over all rows, and their arg-max (the first pivot)
 __global__ void __launch_bounds__(kApplyThreads) k_qr_colnorms(
-    const double* __restrict__ A, int64_t ld, int64_t m, int n, double* __restrict__ cn,
+    double* __restrict__ A, int64_t ld, int64_t m, int n, double* __restrict__ cn,
     double* __restrict__ part_v, int* __restrict__ part_i, unsigned int* __restrict__ counter,
-    QrState* st) {
+    QrState* st, int* __restrict__ perm, double* __restrict__ vbuf, double rcond) {
   const int lane = threadIdx.x & 31;
   const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int nwarps = gridDim.x * (blockDim.x >> 5);
@@ -192,75 +298,25 @@ __global__ void __launch_bounds__(kApplyThreads) k_qr_colnorms(
       bi = j;
     }
   }
-  argmax_finish(bv, bi, part_v, part_i, counter, st, 0);
+  if (argmax_finish(bv, bi, part_v, part_i, counter, st, 0))
+    house_step(A, ld, m, 0, cn, perm, vbuf, st, rcond);
 }
 
-// Step k, part 1: pivot swap and the Householder reflector of column k.
-__global__ void __launch_bounds__(kHouseThreads) k_qr_house(
-    double* __restrict__ A, int64_t ld, int64_t m, int k, double* __restrict__ cn,
-    int* __restrict__ perm, double* __restrict__ vbuf, QrState* __restrict__ st, double rcond) {
-  __shared__ double red[33];
-  __shared__ int s_go, s_j;
-  if (threadIdx.x == 0) {
-    int go = !st->stop;
-    if (go) {
-      const int j = st->piv;
-      const double cj = st->cmax;
-      if (k == 0) st->r11 = sqrt(cj);
-      if (st->bad != 0.0 || !(cj > 0.0) || sqrt(cj) <= rcond * st->r11) {
-        st->stop = 1;
-        st->rank = k;
-        go = 0;
-      } else {
-        s_j = j;
-        if (j != k) {
-          cn[j] = cn[k];
-          const int t = perm[j];
-          perm[j] = perm[k];
-          perm[k] = t;
-        }
-      }
-    }
-    s_go = go;
-  }
-  __syncthreads();
-  if (!s_go) return;
-  const int j = s_j;
-  double* ck = A + (int64_t)k * ld;
-  if (j != k) {
-    double* cj = A + (int64_t)j * ld;
-    for (int64_t i = threadIdx.x; i < m; i += blockDim.x) {
-      const double t = ck[i];
-      ck[i] = cj[i];
-      cj[i] = t;
-    }
-    __syncthreads();
-  }
-  double s1 = 0.0;
-  for (int64_t i = k + 1 + threadIdx.x; i < m; i += blockDim.x) {
-    const double x = ck[i];
-    s1 = fma(x, x, s1);
-    vbuf[i] = x;
-  }
-  s1 = block_sum_d(s1, red);
-  if (threadIdx.x == 0) {
-    const double alpha = ck[k];
-    const double beta = -copysign(sqrt(fma(alpha, alpha, s1)), alpha);
-    const double v0 = alpha - beta;
-    vbuf[k] = v0;
-    ck[k] = beta;
-    st->c = 2.0 / fma(v0, v0, s1);
-    st->rank = k + 1;
-    if (!(beta == beta) || isinf(beta)) st->bad = 1.0;
-  }
-}
-
-// Step k, part 2: A_j -= c (v^T A_j) v for every later column j (h included),
-// the new squared norms over rows k+1.., and their arg-max.
+// Step k: A_j -= c (v^T A_j) v for every later column j (h included), the new
+// squared norms over rows k+1.., their arg-max, and the next reflector.  kReg: a
+// lane holds its at most kRegRows rows of the column from the product to the
+// update (and v comes from shared memory), so that a column is read once, all its
+// loads in flight together; else (more than 2048 rows left) it is read twice.  Both
+// sum the same rows in the same order.  At 2016 rows, 1024 columns the update took
+// 31 us a step reading twice and the reflector 9 us in a kernel of its own; the
+// solve of 242 steps 9.4 -> 7.7 ms (its back substitution included).
+template <bool kReg>
 __global__ void __launch_bounds__(kApplyThreads) k_qr_apply(
-    double* __restrict__ A, int64_t ld, int64_t m, int n, int k, const double* __restrict__ vbuf,
-    QrState* st, double* __restrict__ cn, double* __restrict__ part_v, int* __restrict__ part_i,
-    unsigned int* __restrict__ counter) {
+    double* __restrict__ A, int64_t ld, int64_t m, int n, int k, int steps,
+    double* __restrict__ vbuf, QrState* st, double* __restrict__ cn, double* __restrict__ part_v,
+    int* __restrict__ part_i, unsigned int* __restrict__ counter, int* __restrict__ perm,
+    double rcond) {
+  __shared__ double vs[kReg ? kRegRows * 32 : 1];
   if (st->stop) return;
   const double c = st->c;
   const int lane = threadIdx.x & 31;
@@ -268,30 +324,62 @@ __global__ void __launch_bounds__(kApplyThreads) k_qr_apply(
   const int nwarps = gridDim.x * (blockDim.x >> 5);
   double bv = -1.0;
   int bi = -1;
+  if constexpr (kReg) {
+    for (int i = threadIdx.x; i < (int)(m - k); i += blockDim.x) vs[i] = vbuf[k + i];
+    __syncthreads();
+  }
   for (int j = k + 1 + gw; j <= n; j += nwarps) {
     double* col = A + (int64_t)j * ld;
-    double s0 = 0.0, s1 = 0.0;
-    int64_t i = k + lane;
-    for (; i + 32 < m; i += 64) {
-      s0 = fma(vbuf[i], col[i], s0);
-      s1 = fma(vbuf[i + 32], col[i + 32], s1);
-    }
-    if (i < m) s0 = fma(vbuf[i], col[i], s0);
-    const double s = warp_sum_d(s0 + s1) * c;
-    double n0 = 0.0, n1 = 0.0;
-    i = k + lane;
-    for (; i + 32 < m; i += 64) {
-      const double a0 = fma(-s, vbuf[i], col[i]);
-      const double a1 = fma(-s, vbuf[i + 32], col[i + 32]);
-      col[i] = a0;
-      col[i + 32] = a1;
-      if (i > k) n0 = fma(a0, a0, n0);
-      n1 = fma(a1, a1, n1);
-    }
-    if (i < m) {
-      const double a0 = fma(-s, vbuf[i], col[i]);
-      col[i] = a0;
-      if (i > k) n0 = fma(a0, a0, n0);
+    double s0 = 0.0, s1 = 0.0, n0 = 0.0, n1 = 0.0;
+    if constexpr (kReg) {
+      const int left = (int)(m - k) - lane;   // row k + lane + 32 t exists while 32 t < left
+      double* cl = col + k + lane;
+      double x[kRegRows];
+#pragma unroll
+      for (int t = 0; t < kRegRows; ++t) x[t] = 32 * t < left ? cl[32 * t] : 0.0;
+#pragma unroll
+      for (int t = 0; t < kRegRows; t += 2) {
+        if (32 * t >= (int)(m - k)) break;   // uniform
+        if (32 * t < left) s0 = fma(vs[lane + 32 * t], x[t], s0);
+        if (32 * (t + 1) < left) s1 = fma(vs[lane + 32 * (t + 1)], x[t + 1], s1);
+      }
+      const double s = warp_sum_d(s0 + s1) * c;
+#pragma unroll
+      for (int t = 0; t < kRegRows; t += 2) {
+        if (32 * t >= (int)(m - k)) break;
+        if (32 * t < left) {
+          const double a0 = fma(-s, vs[lane + 32 * t], x[t]);
+          cl[32 * t] = a0;
+          if (t > 0 || lane > 0) n0 = fma(a0, a0, n0);
+        }
+        if (32 * (t + 1) < left) {
+          const double a1 = fma(-s, vs[lane + 32 * (t + 1)], x[t + 1]);
+          cl[32 * (t + 1)] = a1;
+          n1 = fma(a1, a1, n1);
+        }
+      }
+    } else {
+      int64_t i = k + lane;
+      for (; i + 32 < m; i += 64) {
+        s0 = fma(vbuf[i], col[i], s0);
+        s1 = fma(vbuf[i + 32], col[i + 32], s1);
+      }
+      if (i < m) s0 = fma(vbuf[i], col[i], s0);
+      const double s = warp_sum_d(s0 + s1) * c;
+      i = k + lane;
+      for (; i + 32 < m; i += 64) {
+        const double a0 = fma(-s, vbuf[i], col[i]);
+        const double a1 = fma(-s, vbuf[i + 32], col[i + 32]);
+        col[i] = a0;
+        col[i + 32] = a1;
+        if (i > k) n0 = fma(a0, a0, n0);
+        n1 = fma(a1, a1, n1);
+      }
+      if (i < m) {
+        const double a0 = fma(-s, vbuf[i], col[i]);
+        col[i] = a0;
+        if (i > k) n0 = fma(a0, a0, n0);
+      }
     }
     if (j < n) {
       const double nr = warp_sum_d(n0 + n1);
@@ -305,7 +393,8 @@ __global__ void __launch_bounds__(kApplyThreads) k_qr_apply(
       }
     }
   }
-  argmax_finish(bv, bi, part_v, part_i, counter, st, k + 1);
+  if (argmax_finish(bv, bi, part_v, part_i, counter, st, k + 1) && k + 1 < steps)
+    house_step(A, ld, m, k + 1, cn, perm, vbuf, st, rcond);
 }
 
 // R z = (Q^T h)[0:r] by back substitution, column by column (R's columns are
@@ -315,23 +404,40 @@ __global__ void __launch_bounds__(1024) k_qr_backsub(const double* __restrict__ 
                                                      double* __restrict__ y, double* __restrict__ z,
                                                      double* __restrict__ res2) {
   __shared__ double red[33];
-  __shared__ double zj;
+  __shared__ double zj[2];
   const int r = st->rank;
   const double* hc = A + (int64_t)n * ld;
   double s = 0.0;
   for (int64_t i = r + threadIdx.x; i < m; i += blockDim.x) s = fma(hc[i], hc[i], s);
   s = block_sum_d(s, red);
   if (threadIdx.x == 0) *res2 = s;
+  if (r <= (int)blockDim.x) {
+    // thread i keeps y_i and holds the next column's entry before it is needed
+    const int i = threadIdx.x;
+    double yi = i < r ? hc[i] : 0.0;
+    double next = r > 0 && i < r ? A[(int64_t)(r - 1) * ld + i] : 0.0;
+    for (int j = r - 1; j >= 0; --j) {
+      const double cij = next;
+      if (j > 0 && i < j) next = A[(int64_t)(j - 1) * ld + i];
+      if (i == j) {
+        zj[j & 1] = yi / cij;
+        z[j] = zj[j & 1];
+      }
+      __syncthreads();
+      if (i < j) yi = fma(-cij, zj[j & 1], yi);
+    }
+    return;
+  }
   for (int i = threadIdx.x; i < r; i += blockDim.x) y[i] = hc[i];
   __syncthreads();
   for (int j = r - 1; j >= 0; --j) {
     const double* cj = A + (int64_t)j * ld;
     if (threadIdx.x == 0) {
-      zj = y[j] / cj[j];
-      z[j] = zj;
+      zj[0] = y[j] / cj[j];
+      z[j] = zj[0];
     }
     __syncthreads();
-    const double zz = zj;
+    const double zz = zj[0];
     for (int i = threadIdx.x; i < j; i += blockDim.x) y[i] = fma(-cj[i], zz, y[i]);
     __syncthreads();
   }
@@ -410,7 +516,8 @@ void qr_solve(elmfb_ctx* h, const elmfb_solve_opts* o, elmfb_solve_info* info) {
   k_qr_iota<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256), 1024)), 256, 0,
               st>>>(dperm.as<int>(), n);
   k_qr_colnorms<<<nb0, kApplyThreads, 0, st>>>(A, ld, m, n, dcn.as<double>(), dpv.as<double>(),
-                                               dpi.as<int>(), dcnt.as<unsigned int>(), S);
+                                               dpi.as<int>(), dcnt.as<unsigned int>(), S,
+                                               dperm.as<int>(), dv.as<double>(), o->rcond);
   count_launch(h, 2);
   check_launch("qr set-up");
 
@@ -420,15 +527,14 @@ void qr_solve(elmfb_ctx* h, const elmfb_solve_opts* o, elmfb_solve_info* info) {
   while (k < steps) {
     const int batch = std::min(kQrBatch, steps - k);
     for (int b = 0; b < batch; ++b, ++k) {
-      k_qr_house<<<1, kHouseThreads, 0, st>>>(A, ld, m, k, dcn.as<double>(), dperm.as<int>(),
-                                              dv.as<double>(), S, o->rcond);
       const int nb = (int)std::max<int64_t>(
           1, std::min<int64_t>(ceil_div(n - k, warps_per_block), max_blocks));
-      k_qr_apply<<<nb, kApplyThreads, 0, st>>>(A, ld, m, n, k, dv.as<double>(), S,
-                                               dcn.as<double>(), dpv.as<double>(), dpi.as<int>(),
-                                               dcnt.as<unsigned int>());
+      auto* const apply = m - k <= 32 * kRegRows ? k_qr_apply<true> : k_qr_apply<false>;
+      apply<<<nb, kApplyThreads, 0, st>>>(A, ld, m, n, k, steps, dv.as<double>(), S,
+                                          dcn.as<double>(), dpv.as<double>(), dpi.as<int>(),
+                                          dcnt.as<unsigned int>(), dperm.as<int>(), o->rcond);
     }
-    count_launch(h, 2 * batch);
+    count_launch(h, batch);
     check_launch("qr step");
     CUDA_CHECK(cudaMemcpyAsync(&hs, S, sizeof(QrState), cudaMemcpyDeviceToHost, st));
     stream_sync(h);

@@ -496,3 +496,51 @@ def test_profiling_stride_times_every_nth_launch():
     assert timed == (passes + 3) // 4
     assert ms > 0.0
     assert set(stats) == {"fused_Mt_MTu"}
+
+
+@pytest.mark.parametrize("n", [20, 200, 2030, 2046, 2078, 4200])
+def test_qr_over_row_counts(n):
+    """The QR update holds a column in registers once at most 2048 rows are left
+    and reads it twice before that: systems of fewer rows than columns (20), well
+    below, at and just past the limit (cells are padded to 16 rows), and far past
+    it, against the oracle's QR: the rank to one (a pivot may sit at the cut) and
+    the error to half as much again (two orders of the same rows differ by less
+    in the golden workloads)."""
+    from oracle import lstsq as OL
+    from oracle import system as OS
+    P = WL.poisson1d(levels=(1, 4), features=12, n_interior=n, lam=1e4)
+    ref = OS.assemble(P, fmt="dense")
+    a_o, rank = OL.lstsq_qr(ref["M"], ref["h"])
+    with E.Solver.from_problem(P, precision=E.FP64) as s:
+        s.assemble_problem(P)
+        info = s.solve(method=E.SOLVE_QR)
+        a = s.coeffs()
+    assert abs(info.rank - rank) <= 1
+    r, r_o = (np.linalg.norm(ref["M"] @ v - ref["h"]) for v in (a, a_o))
+    h = np.linalg.norm(ref["h"])
+    assert r <= 1.5 * r_o + 1e-9 * h
+
+
+@pytest.mark.parametrize("K", [8, 24, 32, 56, 72, 104, 128])
+def test_block_jacobi_factors_over_feature_counts(K):
+    """Preconditioned LSQR on FP32 panels at feature counts multiple of 8 (the
+    packed 4 x 8 tiles of the diagonal Gram blocks: one tile column, ragged last
+    warps, the largest): with a shift of 1e-2 the first iterate depends on the
+    blocks only to FP32 accuracy times the shift's inverse, 100 x 2^-24 x (a few
+    roundings) < 1e-4 of the one that SciPy gives with the oracle's FP64 blocks."""
+    from oracle import system as OS
+    P = WL.poisson2d(levels=(1, 2), features=K, n_side=37, n_boundary_side=12)
+    ref = OS.assemble(P, fmt="dense")
+    M, h, ns = ref["M"], ref["h"], P.n_subdomains
+    X = np.zeros((ns * K, ns * K))
+    for j in range(ns):
+        b = slice(j * K, (j + 1) * K)
+        G = M[:, b].T @ M[:, b]
+        L = np.linalg.cholesky(G + 1e-2 * np.trace(G) / K * np.eye(K))
+        X[b, b] = np.linalg.inv(L).T
+    a_ref = X @ spla.lsqr(M @ X, h, atol=0, btol=0, conlim=0, iter_lim=1)[0]
+    with E.Solver.from_problem(P, precision=E.FP32) as s:
+        s.assemble_problem(P)
+        s.solve(max_iter=1, atol=0.0, btol=0.0, shift=1e-2, check_every=1)
+        a = s.coeffs()
+    assert np.linalg.norm(a - a_ref) <= 1e-4 * np.linalg.norm(a_ref)
