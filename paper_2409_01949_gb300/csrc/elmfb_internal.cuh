@@ -72,29 +72,44 @@ struct DevBuf {
 // r) at byte (r / 8) (block / 2) + (k / 8) 128 + (k % 8) 16 + (r % 8) 2.
 __host__ __device__ constexpr int gram_block_bytes(int K) { return ((K + 7) & ~7) * 32; }
 
-// Several host arrays uploaded as one copy into one buffer, each buffer added
-// becoming a part of it: a copy of a small pageable array costs 5 us of host time
-// whatever its size.  The parts are valid until the owner is sent or released again.
+// Several host arrays uploaded into one buffer, each buffer added becoming a part
+// of it: small ones (a copy of a small pageable array costs 5 us of host time
+// whatever its size) packed into one copy, large ones from where they are.  The
+// arrays must live until send(); the parts are valid until the owner is sent or
+// released again.
 struct Upload {
+  static constexpr size_t kLarge = 64 * 1024;
   struct Part {
     DevBuf* to;
+    const void* src;
     size_t at, bytes;
   };
-  std::vector<char> host;
   std::vector<Part> parts;
   template <class T>
   void add(DevBuf& to, const T* src, size_t n) {
-    const size_t at = (host.size() + 15) & ~size_t(15), bytes = n * sizeof(T);
-    host.resize(at + std::max<size_t>(bytes, 16));
-    if (bytes) std::memcpy(host.data() + at, src, bytes);
-    parts.push_back({&to, at, bytes});
+    parts.push_back({&to, src, 0, n * sizeof(T)});
   }
   void send(DevBuf& owner, cudaStream_t stream) {
-    owner.alloc(host.size(), stream);
-    CUDA_CHECK(cudaMemcpyAsync(owner.p, host.data(), host.size(), cudaMemcpyHostToDevice, stream));
+    size_t small = 0, total = 0;
+    auto room = [](const Part& q) { return (std::max<size_t>(q.bytes, 16) + 15) & ~size_t(15); };
+    for (Part& q : parts)
+      if (q.bytes < kLarge) q.at = small, small += room(q);
+    total = small;
+    for (Part& q : parts)
+      if (q.bytes >= kLarge) q.at = total, total += room(q);
+    std::vector<char> host(small);
+    owner.alloc(total, stream);
+    char* const base = static_cast<char*>(owner.p);
+    for (const Part& q : parts)
+      if (q.bytes >= kLarge)
+        CUDA_CHECK(cudaMemcpyAsync(base + q.at, q.src, q.bytes, cudaMemcpyHostToDevice, stream));
+      else if (q.bytes)
+        std::memcpy(host.data() + q.at, q.src, q.bytes);
+    if (small)
+      CUDA_CHECK(cudaMemcpyAsync(base, host.data(), small, cudaMemcpyHostToDevice, stream));
     for (const Part& q : parts) {
       q.to->release();
-      q.to->p = static_cast<char*>(owner.p) + q.at;
+      q.to->p = base + q.at;
       q.to->bytes = q.bytes;
       q.to->s = stream;
       q.to->own = false;

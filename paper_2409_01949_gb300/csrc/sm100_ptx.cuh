@@ -1,5 +1,5 @@
 // Inline-PTX helpers for the Blackwell (sm_100 family, here sm_103a) async
-// machinery used by the tensor-core kernels: mbarriers, bulk copies,
+// machinery used by the tensor-core kernels: mbarriers, TMA copies,
 // TMEM allocation, tcgen05.mma / commit / ld.  Every wait is bounded: after
 // kSpinLimit polls it gives up and reports failure to the caller.
 #pragma once
@@ -54,6 +54,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
 }
 
 // ---------------------------------------------------------------- TMA
+__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int32_t x,
+                                            int32_t y, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
+      : "memory");
+}
 // 1-D bulk copy global -> shared, completing `bytes` on the mbarrier
 // (addresses 16-byte aligned, size a multiple of 16)
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes,

@@ -29,6 +29,7 @@
 #include <cmath>
 
 #include <cooperative_groups.h>
+#include <cudaTypedefs.h>
 #include <cstdlib>
 #include <map>
 #include <mutex>
@@ -479,6 +480,193 @@ __global__ void __launch_bounds__(544) k_gram_diag_pipe(const T* __restrict__ pa
         const int idx = i * K - i * (i - 1) / 2 + (j - i);
         out[idx] = (double)hi[a][b] - (double)lo[a][b];
       }
+    }
+}
+
+// Two FP32 values in a 64-bit register: sm_103a's packed arithmetic rounds each
+// half as the scalar instruction does.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// a - b (b times -1 is exact)
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+  return fma2(b, 0xbf800000bf800000ull, a);
+}
+
+// k_gram_diag_pipe for FP32 panels with K a multiple of 8, the same sums in the
+// same order (16-row FP32 sums by fused multiply-adds, compensated across): a
+// thread holds a 4 x 8 tile in packed pairs, a producer warp of its own runs the
+// ring, and each consumer warp moves on as soon as its rows are in, releasing a
+// stage by its own arrival.  With one refill per block barrier the barrier was
+// the first stall (57% issue-active, FMA pipe 39%), and 4 x 4 tiles of scalar FMAs
+// read 8 values from shared memory per 16 products; this form reads 12 per 32 and
+// issues half the arithmetic instructions.  A step's 16 rows are one TMA box: the
+// rows of a cell with m covering panels are m K elements apart, so the whole panel
+// array is described once per m as a matrix of rows m K wide, and a step starts at
+// (row % m) K of row / m (0.5 ms less than 16 bulk copies of 256 bytes a step on
+// the large 2-D workload).  Block-Jacobi LSQR of 20 steps at 400^2, K = 128: 8.25 ->
+// 7.91 ms, all of it these blocks (1.96 -> 1.6 ms); at K = 64 (72 of 96 lanes hold a
+// tile) the two forms take the same time.
+constexpr int kDiagRing = 8;
+constexpr int kDiagMaps = 32;   // covering panels of a cell, at most
+struct DiagMaps {
+  CUtensorMap of[kDiagMaps];    // of[m - 1]
+};
+
+__global__ void __launch_bounds__(320) k_gram_diag_fp32(const __grid_constant__ DiagMaps maps,
+                                                        int K, const int4* __restrict__ chunks,
+                                                        const int2* __restrict__ steps,
+                                                        const int64_t* __restrict__ entry_base,
+                                                        const int* __restrict__ entry_cell,
+                                                        const int* __restrict__ cover_off,
+                                                        double* __restrict__ partial,
+                                                        int* __restrict__ flags) {
+  extern __shared__ __align__(128) unsigned char smraw[];
+  float* ring = reinterpret_cast<float*>(smraw);   // [kDiagRing][16][K]
+  __shared__ __align__(8) uint64_t full[kDiagRing], empty[kDiagRing];
+  const int4 ch = chunks[blockIdx.x];   // (panel, first step, steps, -)
+  const int nsteps = ch.z;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int consumers = (blockDim.x >> 5) - 1;   // the last warp produces
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < kDiagRing; ++q) {
+      sm100::mbar_init(&full[q], 1);
+      sm100::mbar_init(&empty[q], (uint32_t)consumers);
+    }
+    sm100::fence_mbar_init();
+  }
+  __syncthreads();
+  bool ok = true;
+  if (warp == consumers) {
+    const uint32_t step_bytes = (uint32_t)(16 * K * sizeof(float));
+    int st = 0, ph = 1;
+    for (int q0 = 0; q0 < nsteps; q0 += 32) {
+      // 32 steps looked up at once, one a lane
+      int mine_m = 1, mine_x = 0, mine_y = 0;
+      if (q0 + lane < nsteps) {
+        const DiagStepRows sr =
+            diag_step(steps, entry_base, entry_cell, cover_off, ch.y + q0 + lane, K);
+        mine_m = (int)(sr.mK / K);
+        mine_y = (int)(sr.row0 / mine_m);
+        mine_x = (int)(sr.row0 - (int64_t)mine_y * mine_m) * K;
+      }
+      const int n = min(32, nsteps - q0);
+      for (int q = 0; q < n; ++q) {
+        const int m = __shfl_sync(0xffffffffu, mine_m, q);
+        const int x = __shfl_sync(0xffffffffu, mine_x, q);
+        const int y = __shfl_sync(0xffffffffu, mine_y, q);
+        if (!sm100::mbar_wait(&empty[st], ph, ok ? sm100::kSpinLimit : 4u)) ok = false;
+        if (lane == 0) {
+          sm100::fence_proxy_async_smem();
+          sm100::mbar_arrive_expect_tx(&full[st], step_bytes);
+          sm100::tma_load_2d(ring + (int64_t)st * 16 * K, &maps.of[m - 1], x, y, &full[st]);
+        }
+        __syncwarp();
+        if (++st == kDiagRing) {
+          st = 0;
+          ph ^= 1;
+        }
+      }
+    }
+    if (!ok && lane == 0) atomicOr(&flags[3], 1);
+    return;
+  }
+  // tile (ti, tj): rows 4 ti .. + 3, columns 8 tj .. + 7 of the upper triangle
+  const int nr = K / 4, ncol = K / 8;
+  int ti = -1, tj = 0;
+  {
+    int rem = threadIdx.x;
+    for (int a = 0; a < nr; ++a) {
+      const int len = ncol - (a >> 1);
+      if (rem < len) {
+        ti = a;
+        tj = (a >> 1) + rem;
+        break;
+      }
+      rem -= len;
+    }
+  }
+  // the tile's two column quads in an order that spreads 8 neighbouring lanes'
+  // 16-byte reads over all banks
+  const int swap = ((tj >> 2) ^ tj) & 1;
+  const int c0 = 8 * tj + 4 * swap, c1 = 8 * tj + 4 * (1 - swap);
+  uint64_t hi[4][4], lo[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) hi[a][b] = lo[a][b] = 0;
+  int st = 0, ph = 0;
+  for (int q = 0; q < nsteps; ++q) {
+    if (!sm100::mbar_wait(&full[st], ph, ok ? sm100::kSpinLimit : 4u)) ok = false;
+    if (ti >= 0) {
+      const float* sm = ring + (int64_t)st * 16 * K;
+      uint64_t acc[4][4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = 0;
+#pragma unroll 4
+      for (int r = 0; r < 16; ++r) {
+        const float4 x = *reinterpret_cast<const float4*>(sm + r * K + 4 * ti);
+        const ulonglong2 y0 = *reinterpret_cast<const ulonglong2*>(sm + r * K + c0);
+        const ulonglong2 y1 = *reinterpret_cast<const ulonglong2*>(sm + r * K + c1);
+        const uint64_t xx[4] = {pack2(x.x, x.x), pack2(x.y, x.y), pack2(x.z, x.z),
+                                pack2(x.w, x.w)};
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          acc[a][0] = fma2(xx[a], y0.x, acc[a][0]);
+          acc[a][1] = fma2(xx[a], y0.y, acc[a][1]);
+          acc[a][2] = fma2(xx[a], y1.x, acc[a][2]);
+          acc[a][3] = fma2(xx[a], y1.y, acc[a][3]);
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const uint64_t yv = sub2(acc[a][b], lo[a][b]);
+          const uint64_t tv = add2(hi[a][b], yv);
+          lo[a][b] = sub2(sub2(tv, hi[a][b]), yv);
+          hi[a][b] = tv;
+        }
+    }
+    __syncwarp();
+    if (lane == 0) sm100::mbar_arrive(&empty[st]);
+    if (++st == kDiagRing) {
+      st = 0;
+      ph ^= 1;
+    }
+  }
+  if (!ok && lane == 0) atomicOr(&flags[3], 1);
+  if (ti < 0) return;
+  const int KT = K * (K + 1) / 2;
+  double* out = partial + (int64_t)blockIdx.x * KT;
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      const int i = 4 * ti + a, j = (b < 4 ? c0 : c1 - 4) + b;
+      const float2 h2 = unpack2(hi[a][b >> 1]), l2 = unpack2(lo[a][b >> 1]);
+      if (j >= i)
+        out[i * K - i * (i - 1) / 2 + (j - i)] =
+            (b & 1) ? (double)h2.y - (double)l2.y : (double)h2.x - (double)l2.x;
     }
 }
 
@@ -2456,9 +2644,9 @@ bool build_fused_plan(elmfb_ctx* h, FusedPlan& fp, int unit_rows) {
     fp.n_pchunks = (int)pch.size();
     lists.add(fp.pch, pch.data(), pch.size());
     lists.add(fp.pco, pco.data(), pco.size());
+    lists.send(fp.lists, st);
     fp.csum.alloc(std::max<size_t>(pch.size(), 1) * K * sizeof(double), st);
   }
-  lists.send(fp.lists, st);
   if (fp.pairs)
     fp.tf.alloc(std::max<int64_t>(h->NPhi, 1) * (h->df32() ? sizeof(float2) : sizeof(float)), st);
   return true;
@@ -2636,6 +2824,44 @@ void launch_fused(elmfb_ctx* h, FusedPlan& fp, const double* t64, int mode, doub
 // partials (K(K+1)/2 doubles per chunk) small next to the panel reads
 constexpr int kDiagChunk = 2048;
 
+// cuTensorMapEncodeTiled from the driver, resolved at run time through the
+// runtime's entry-point query (the library does not link libcuda directly).
+static PFN_cuTensorMapEncodeTiled_v12000 encode_tiled() {
+  // thread-safe one-time lookup (function-local static initialisation)
+  static PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
+                                         &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      return nullptr;
+    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+  }();
+  if (!fn) ELMFB_THROW(ELMFB_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
+  return fn;
+}
+
+// The FP32 panels as a matrix of rows m K wide, boxes of 16 rows x K, for every
+// number m of covering panels that a cell with rows has.
+static void encode_diag_maps(elmfb_ctx* h, DiagMaps& maps) {
+  std::memset(&maps, 0, sizeof(maps));
+  bool have[kDiagMaps + 1] = {};
+  for (int c = 0; c < h->n_cells; ++c)
+    if (h->cell_count[c] > 0) have[h->cover_off[c + 1] - h->cover_off[c]] = true;
+  for (int m = 1; m <= kDiagMaps; ++m) {
+    if (!have[m]) continue;
+    const cuuint64_t dim[2] = {(cuuint64_t)m * h->K, (cuuint64_t)ceil_div(h->NPR, m)};
+    const cuuint64_t stride[1] = {dim[0] * sizeof(float)};
+    const cuuint32_t box[2] = {(cuuint32_t)h->K, 16}, step[2] = {1, 1};
+    const CUresult r = encode_tiled()(
+        &maps.of[m - 1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->d_panels.p, dim, stride, box, step,
+        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS)
+      ELMFB_THROW(ELMFB_ERR_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r));
+  }
+}
+
 template <class T>
 void block_jacobi_setup(elmfb_ctx* h, double shift, bool identity, double abs_shift,
                         double drop) {
@@ -2703,6 +2929,18 @@ void block_jacobi_setup(elmfb_ctx* h, double shift, bool identity, double abs_sh
           h->d_panels.as<float2>(), K, dch.as<int4>(), dsteps.as<int2>(),
           h->d_entry_base.as<int64_t>(), h->d_entry_cell.as<int>(), h->d_cover_off.as<int>(),
           h->d_gpart.as<double>(), h->d_flags.as<int>());
+    } else if (std::is_same<T, float>::value && K % 8 == 0 && h->max_cover <= kDiagMaps) {
+      int tiles = 0;
+      for (int a = 0; a < K / 4; ++a) tiles += K / 8 - a / 2;
+      const size_t psmem = (size_t)kDiagRing * 16 * K * sizeof(float);
+      ensure_dyn_smem((const void*)k_gram_diag_fp32, psmem);
+      DiagMaps maps;
+      encode_diag_maps(h, maps);
+      k_gram_diag_fp32<<<(unsigned)chunks.size(), (unsigned)(ceil_div(tiles, 32) * 32 + 32), psmem,
+                         st>>>(
+          maps, K, dch.as<int4>(), dsteps.as<int2>(), h->d_entry_base.as<int64_t>(),
+          h->d_entry_cell.as<int>(), h->d_cover_off.as<int>(), h->d_gpart.as<double>(),
+          h->d_flags.as<int>());
     } else if (K % 4 == 0 && (K * sizeof(T)) % 16 == 0) {
       const size_t psmem = (size_t)kDiagStages * 16 * K * sizeof(T);
       ensure_dyn_smem((const void*)k_gram_diag_pipe<T>, psmem);
