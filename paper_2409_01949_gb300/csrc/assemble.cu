@@ -807,14 +807,14 @@ __global__ void __launch_bounds__(64, 8) k_assemble_fx(
           const int64_t phi = fx::tanh61(arg, 54 - wexp, tab, rows);
           const fx::Val p = fx::split(phi << 1);   // units of 2^-62
           // B and C, then D = B - phi C (2^(er - 59))
-          int64_t xb = (int64_t)rb.x * w0[i].lo + ((int64_t)rb.y * w0[i].hi + (1 << 30));
-          int64_t xc = (int64_t)rg.x * q0[i].lo + ((int64_t)rg.y * q0[i].hi + (1 << 30));
-          int64_t B = (int64_t)rb.x * w0[i].hi, C = (int64_t)rg.x * q0[i].hi;
+          int64_t xb = fx::mad(rb.x, w0[i].lo, fx::mad(rb.y, w0[i].hi, 1 << 30));
+          int64_t xc = fx::mad(rg.x, q0[i].lo, fx::mad(rg.y, q0[i].hi, 1 << 30));
+          int64_t B = fx::mad(rb.x, w0[i].hi, 0), C = fx::mad(rg.x, q0[i].hi, 0);
           if (kTwo) {
-            xb += (int64_t)rb.z * w1[i].lo + (int64_t)rb.w * w1[i].hi;
-            xc += (int64_t)rg.z * q1[i].lo + (int64_t)rg.w * q1[i].hi;
-            B += (int64_t)rb.z * w1[i].hi;
-            C += (int64_t)rg.z * q1[i].hi;
+            xb = fx::mad(rb.z, w1[i].lo, fx::mad(rb.w, w1[i].hi, xb));
+            xc = fx::mad(rg.z, q1[i].lo, fx::mad(rg.w, q1[i].hi, xc));
+            B = fx::mad(rb.z, w1[i].hi, B);
+            C = fx::mad(rg.z, q1[i].hi, C);
           }
           B += xb >> 31;
           C += xc >> 31;

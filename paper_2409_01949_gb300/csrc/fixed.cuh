@@ -31,14 +31,25 @@ struct Val {
   int hi, lo;
 };
 
+// a b + c of 32-bit factors, one instruction on the device
+FX_FN int64_t mad(int a, int b, int64_t c) {
+#if defined(__CUDA_ARCH__)
+  int64_t d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+#else
+  return (int64_t)a * b + c;
+#endif
+}
+
 FX_FN Val split(int64_t v) { return {(int)(v >> 31), (int)(v & 0x7fffffff)}; }
 
 // c + a b / 2^62, to the nearest unit (but for the lo x lo product): rounding
 // down would put half a unit of the same sign on every one of the thousands of
 // terms of a sum
 FX_FN int64_t mul_add(Val a, Val b, int64_t c) {
-  const int64_t cross = (int64_t)a.hi * b.lo + ((int64_t)a.lo * b.hi + (1 << 30));
-  return (int64_t)a.hi * b.hi + c + (cross >> 31);
+  const int64_t cross = mad(a.hi, b.lo, mad(a.lo, b.hi, 1 << 30));
+  return mad(a.hi, b.hi, c) + (cross >> 31);
 }
 
 // The weight scale a as a power of two: weights and biases are at most
@@ -58,11 +69,11 @@ FX_FN int weight_exp(double a) {
 // x in units of 2^-61 and b in units of 2^(wexp - 60); s has b's unit and at
 // most three terms, so it stays below 2^62.
 FX_FN int64_t argument(Val w0, Val x0, Val w1, Val x1, int64_t b, bool two) {
-  int64_t cross = (int64_t)w0.hi * x0.lo + ((int64_t)w0.lo * x0.hi + (1 << 30));
-  int64_t s = (int64_t)w0.hi * x0.hi + b;
+  int64_t cross = mad(w0.hi, x0.lo, mad(w0.lo, x0.hi, 1 << 30));
+  int64_t s = mad(w0.hi, x0.hi, b);
   if (two) {
-    cross += (int64_t)w1.hi * x1.lo + (int64_t)w1.lo * x1.hi;
-    s += (int64_t)w1.hi * x1.hi;
+    cross = mad(w1.hi, x1.lo, mad(w1.lo, x1.hi, cross));
+    s = mad(w1.hi, x1.hi, s);
   }
   return s + (cross >> 31);
 }
@@ -72,10 +83,16 @@ FX_FN int64_t argument(Val w0, Val x0, Val w1, Val x1, int64_t b, bool two) {
 // (tanh_table.py), the last of them for everything past the others.
 FX_FN int64_t tanh61(int64_t s, int shift, const int4* tab, int rows) {
   const uint64_t m = (uint64_t)(s < 0 ? -s : s);
-  const uint64_t j64 = m >> shift;
-  const int j = j64 < (uint64_t)rows ? (int)j64 : rows - 1;
-  // the place in the interval as r in [-1, 1), units of 2^-62
-  const Val r = split((int64_t)((m << (64 - shift)) >> 1) - ((int64_t)1 << 62));
+  // |s| < 2^62 and 38 <= shift <= 58: the interval is in the upper word
+  const uint32_t mh = (uint32_t)(m >> 32), ml = (uint32_t)m;
+  const uint32_t ju = mh >> (shift - 32);
+  const int j = ju < (uint32_t)rows ? (int)ju : rows - 1;
+  // the place in the interval as r in [-1, 1), units of 2^-62: the bits below
+  // `shift`, from bit 62 down, less 2^62
+  const int up = 63 - shift;
+  const uint32_t vl = ml << up;
+  const uint32_t vh = (((mh << up) | (ml >> (32 - up))) & 0x7fffffffu) - 0x40000000u;
+  const Val r = {(int)((vh << 1) | (vl >> 31)), (int)(vl & 0x7fffffffu)};
   const int4 a = tab[3 * j], b = tab[3 * j + 1], d = tab[3 * j + 2];
   auto word = [](int lo, int hi) { return (int64_t)(((uint64_t)(uint32_t)hi << 32) | (uint32_t)lo); };
   // c4 and up fit 32 bits, and the high half of r is enough for them
