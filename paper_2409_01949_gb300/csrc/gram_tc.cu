@@ -13,8 +13,8 @@
 // mixed precision, laid out as the tensor cores read it: per 16 panel rows one
 // block of 8 x 8 core matrices (8 features x 8 rows, 128 contiguous bytes),
 // features fastest, then the two row halves.  For one pair, A = P_i^T (features x
-// rows) and B = P_j^T are both K-major along the contraction; a box of up to 64
-// rows is one contiguous bulk copy into a shared-memory ring, and each of its 16-row
+// rows) and B = P_j^T are both K-major along the contraction; a box of up to 128
+// rows (256 at K <= 32) is one contiguous bulk copy into a shared-memory ring, and each of its 16-row
 // blocks one MMA step without swizzle.  One thread issues tcgen05.mma (M = 128,
 // N = K rounded up to 16) into a TMEM accumulator, releasing each stage with
 // tcgen05.commit.  Feature rows of a tile past K hold whatever the ring holds:
@@ -32,10 +32,9 @@
 // work so far, so that all CTAs are in the same place at the same time and the
 // panels stay in L2: with one CTA per pair, pair after pair, the coarse panels'
 // pairs each streamed the whole domain, and the level-1 pair alone was 2525 boxes
-// of one CTA.  400^2 points, levels 1..16, K = 128 (6297 pairs): 1.64 -> 0.85 ms,
-// 330 -> 640 TFLOP/s; the tiles arrive at 10 TB/s from L2, which bounds it (half
-// the ring costs 4%, so it is not latency): fewer tile reads per block would need
-// several pairs per accumulator set.
+// of one CTA.  400^2 points, levels 1..16, K = 128 (6297 pairs): 1.64 -> 0.75 ms,
+// 330 -> 730 TFLOP/s; 2048^2, levels 1..64, K = 64: 49.6 -> 33.4 ms, 170 -> 253
+// TFLOP/s (half of each MMA's rows are past K there).
 //
 // Every mbarrier wait is bounded; a timeout raises flags[2].
 #include <algorithm>
@@ -54,15 +53,22 @@
 
 namespace {
 
-constexpr int kBoxRows = 64;                 // contraction rows per box
+constexpr int kCutRows = 64;                 // tasks are cut at multiples of this many rows
 constexpr int kMaxGramStages = 12;
 constexpr int kGramThreads = 192;            // producer, MMA, four epilogue warps
 constexpr size_t kGramRing = 192 * 1024;
 // ring, 1 KB alignment, and the rest of a 128-row tile past the last stage's K rows
 constexpr size_t kGramSmem = kGramRing + 16 * 1024 + 1024;
 
-// a box of 64 rows of one panel: four blocks
-__host__ __device__ constexpr int gram_tile_bytes(int K) { return 4 * gram_block_bytes(K); }
+// Contraction rows per box.  A box costs the producer and the MMA thread about 700
+// cycles whatever its size (boxes of 64 rows took the same time at K = 64 and K =
+// 128, and half the ring cost 4%), so it is as large as leaves three stages or more
+// of the ring: 64 -> 128 rows took 0.94 -> 0.75 ms at K = 128, 45.6 -> 33.4 ms at K =
+// 64 on the workloads above.
+__host__ __device__ constexpr int gram_box_rows(int K) { return K <= 32 ? 256 : 128; }
+__host__ __device__ constexpr int gram_tile_bytes(int K) {
+  return gram_box_rows(K) / 16 * gram_block_bytes(K);
+}
 
 // tasks: (first run, end run, diagonal, block: >= 0 a block of G, else partial ~block)
 __global__ void __launch_bounds__(kGramThreads, 1)
@@ -77,6 +83,7 @@ __global__ void __launch_bounds__(kGramThreads, 1)
   uint8_t* sm = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int box = gram_box_rows(K);
   const int tile_bytes = gram_tile_bytes(K), block_bytes = gram_block_bytes(K);
   const int t0 = task_off[blockIdx.x], t1 = task_off[blockIdx.x + 1];   // this CTA's tasks
 
@@ -108,13 +115,13 @@ __global__ void __launch_bounds__(kGramThreads, 1)
       for (int r = task.x; r < task.y && ok; ++r) {
         const int4 run = next;
         next = runs[min(r + 1, task.y - 1)];
-        for (int off = 0; off < run.z; off += kBoxRows) {
+        for (int off = 0; off < run.z; off += box) {
           if (!sm100::mbar_wait(&empty[st], ph)) {   // the first round passes at once
             ok = false;
             break;
           }
           uint8_t* a = sm + (size_t)st * 2 * tile_bytes;
-          const uint32_t bytes = (uint32_t)(min(kBoxRows, run.z - off) / 16 * block_bytes);
+          const uint32_t bytes = (uint32_t)(min(box, run.z - off) / 16 * block_bytes);
           sm100::mbar_arrive_expect_tx(&full[st], task.z ? bytes : 2 * bytes);
           sm100::bulk_load(a, pt + (int64_t)((run.x + off) >> 4) * block_bytes, bytes, &full[st]);
           if (!task.z)
@@ -150,7 +157,7 @@ __global__ void __launch_bounds__(kGramThreads, 1)
       for (int r = task.x; r < task.y && ok; ++r) {
         const int len = next;
         next = runs[min(r + 1, task.y - 1)].z;
-        for (int off = 0; off < len; off += kBoxRows) {
+        for (int off = 0; off < len; off += box) {
           if (!sm100::mbar_wait(&full[st], ph)) {
             ok = false;
             break;
@@ -161,7 +168,7 @@ __global__ void __launch_bounds__(kGramThreads, 1)
           const uint64_t ad = sm100::sdesc_k_plain(sm100::smem_u32(a), lead, 128);
           const uint64_t bd =
               sm100::sdesc_k_plain(sm100::smem_u32(task.z ? a : a + tile_bytes), lead, 128);
-          const int ksteps = min(kBoxRows, len - off) / 16;
+          const int ksteps = min(box, len - off) / 16;
           for (int ks = 0; ks < ksteps; ++ks) {
             const uint64_t step = (uint64_t)(ks * (block_bytes >> 4));
             sm100::mma_bf16(acc_at, ad + step, bd + step, idesc, acc);
@@ -306,10 +313,10 @@ void gram_build_pairs(elmfb_ctx* h) {
   std::iota(order.begin(), order.end(), 0);
   std::sort(order.begin(), order.end(), [&](int x, int y) { return keys[x] < keys[y]; });
   h->gram_pair_ij.clear();
-  // Rows per task: at most 4096 (64 boxes; at K = 128 a partial block is then 3%
+  // Rows per task: at most 4096 (32 boxes; at K = 128 a partial block is then 3%
   // of the operands read for it), fewer where that leaves under 16 tasks a CTA.
   const int64_t cap = std::min<int64_t>(
-      4096, std::max<int64_t>(256, total / (152 * 16) / kBoxRows * kBoxRows));
+      4096, std::max<int64_t>(256, total / (152 * 16) / kCutRows * kCutRows));
   struct Task {
     int4 t;
     int at;
@@ -331,14 +338,14 @@ void gram_build_pairs(elmfb_ctx* h) {
           tasks.push_back({make_int4((int)runs.size(), 0, diag, 0), r.at, 0});
           rows = 0;
         }
-        // a cut inside a run stays on a box
+        // cuts inside a run at multiples of kCutRows
         const int room = (int)(cap - rows);
         const int take = r.len - off <= room ? r.len - off
-                                             : std::max(room / kBoxRows * kBoxRows, kBoxRows);
+                                             : std::max(room / kCutRows * kCutRows, kCutRows);
         const int len = std::min(take, r.len - off);
         runs.push_back(make_int4(r.a + off, r.b + off, len, 0));
         tasks.back().t.y = (int)runs.size();
-        tasks.back().boxes += (int)ceil_div(len, kBoxRows) * (2 - diag);
+        tasks.back().boxes += (int)ceil_div(len, gram_box_rows(h->K)) * (2 - diag);
         off += len;
         rows += len;
       }
