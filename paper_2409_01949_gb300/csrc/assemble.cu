@@ -571,8 +571,10 @@ __device__ __noinline__ double entry64(double w0, double w1, double b, double x0
 // cycles of a sub-partition for a warp's 32 entries); this one by integer issue
 // (ncu: 50% issue-active, the multiply-add pipe 51%), with phase 1's FP64 work
 // beside it.  400^2 points, levels 1..16, K = 128: assembly and one LSQR step
-// 29.5 -> 10.1 ms; the oscillator (20000 points, levels 1..64, K = 96, pairs),
-// four LSQR steps: 4.18 -> 1.63 ms.  Entries against a 113-bit evaluation: 1.5e-16
+// 29.5 -> 10.1 ms with this kernel, 7.1 ms with the host work around it cut and
+// the products as single multiply-adds (that last step 8.4 -> 7.1 ms); the
+// oscillator (20000 points, levels 1..64, K = 96, pairs), four LSQR steps: 4.18
+// -> 1.63 ms, then 1.36 ms.  Entries against a 113-bit evaluation: 1.5e-16
 // -> 0.9e-16 of the system's norm in FP64, the pairs' 48 bits as before.
 //
 // 1-D window factor f = 4 c^4 with (s, c) = sincos(pi x / 2), x = dx / sigma, its
