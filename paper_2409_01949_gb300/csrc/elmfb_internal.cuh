@@ -259,8 +259,8 @@ struct elmfb_ctx {
   // BF16 panel copy (mixed precision; gram_block_bytes) and Gram blocks
   DevBuf d_pt;
   std::vector<std::pair<int, int>> gram_pair_ij;   // sorted (i <= j)
-  int gram_ctas = 0, gram_multi = 0, gram_parts = 0;
-  DevBuf d_gram_tasks, d_gram_task_off, d_gram_runs, d_gram_multi, d_gram;   // d_gram: [pair][K][K] FP32
+  int gram_ctas = 0;
+  DevBuf d_gram_tasks, d_gram_task_off, d_gram_runs, d_gram;   // d_gram: [pair][K][K] FP32
   bool have_gram = false;
 
   // learned preconditioner: subdomain graph, weights, Adam moments, work buffers

@@ -53,7 +53,6 @@
 
 namespace {
 
-constexpr int kCutRows = 64;                 // tasks are cut at multiples of this many rows
 constexpr int kMaxGramStages = 12;
 constexpr int kGramThreads = 192;            // producer, MMA, four epilogue warps
 constexpr size_t kGramRing = 192 * 1024;
@@ -70,11 +69,11 @@ __host__ __device__ constexpr int gram_tile_bytes(int K) {
   return gram_box_rows(K) / 16 * gram_block_bytes(K);
 }
 
-// tasks: (first run, end run, diagonal, block: >= 0 a block of G, else partial ~block)
+// tasks: (first run, end run, 2 boxes + diagonal, block of G)
 __global__ void __launch_bounds__(kGramThreads, 1)
     k_gram_tc(const uint8_t* __restrict__ pt, const int4* __restrict__ tasks,
               const int* __restrict__ task_off, const int4* __restrict__ runs, int K, int N, int S,
-              float* __restrict__ G, float* __restrict__ part, int* __restrict__ flags) {
+              float* __restrict__ G, int* __restrict__ flags) {
   extern __shared__ uint8_t smraw[];
   __shared__ __align__(8) uint64_t full[kMaxGramStages];
   __shared__ __align__(8) uint64_t empty[kMaxGramStages];
@@ -111,6 +110,7 @@ __global__ void __launch_bounds__(kGramThreads, 1)
     int st = 0, ph = 1, issued = 0;
     for (int t = t0; t < t1 && ok; ++t) {
       const int4 task = tasks[t];
+      const bool diag = task.z & 1;
       int4 next = runs[task.x];   // one record ahead, so that its load is not waited for
       for (int r = task.x; r < task.y && ok; ++r) {
         const int4 run = next;
@@ -122,9 +122,9 @@ __global__ void __launch_bounds__(kGramThreads, 1)
           }
           uint8_t* a = sm + (size_t)st * 2 * tile_bytes;
           const uint32_t bytes = (uint32_t)(min(box, run.z - off) / 16 * block_bytes);
-          sm100::mbar_arrive_expect_tx(&full[st], task.z ? bytes : 2 * bytes);
+          sm100::mbar_arrive_expect_tx(&full[st], diag ? bytes : 2 * bytes);
           sm100::bulk_load(a, pt + (int64_t)((run.x + off) >> 4) * block_bytes, bytes, &full[st]);
-          if (!task.z)
+          if (!diag)
             sm100::bulk_load(a + tile_bytes, pt + (int64_t)((run.y + off) >> 4) * block_bytes,
                              bytes, &full[st]);
           ++issued;
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kGramThreads, 1)
           const uint32_t lead = (uint32_t)block_bytes / 2;   // between the row halves
           const uint64_t ad = sm100::sdesc_k_plain(sm100::smem_u32(a), lead, 128);
           const uint64_t bd =
-              sm100::sdesc_k_plain(sm100::smem_u32(task.z ? a : a + tile_bytes), lead, 128);
+              sm100::sdesc_k_plain(sm100::smem_u32(task.z & 1 ? a : a + tile_bytes), lead, 128);
           const int ksteps = min(box, len - off) / 16;
           for (int ks = 0; ks < ksteps; ++ks) {
             const uint64_t step = (uint64_t)(ks * (block_bytes >> 4));
@@ -191,14 +191,16 @@ __global__ void __launch_bounds__(kGramThreads, 1)
     const bool vec = K % 4 == 0;
     int q = 0;
     for (int t = t0; t < t1 && ok; ++t, ++q) {
-      const int block = tasks[t].w, buf = q & 1;
-      if (!sm100::mbar_wait(&acc_full[buf], (q >> 1) & 1)) {
+      const int buf = q & 1;
+      const int4 task = tasks[t];
+      // a pair is one chain: the wait grows with its boxes (each within the limits above)
+      const uint32_t limit = sm100::kSpinLimit + 256u * (uint32_t)(task.z >> 1);
+      if (!sm100::mbar_wait(&acc_full[buf], (q >> 1) & 1, limit)) {
         ok = false;
         break;
       }
       sm100::tc_fence_after();
-      float* out = (block >= 0 ? G + (int64_t)block * K * K : part + (int64_t)~block * K * K) +
-                   (int64_t)m * K;
+      float* out = G + (int64_t)task.w * K * K + (int64_t)m * K;
       if (32 * quad < K) {
         for (int c0 = 0; c0 < N; c0 += 16) {
           uint32_t v[16];
@@ -235,21 +237,6 @@ __global__ void __launch_bounds__(kGramThreads, 1)
   if (warp == 2) sm100::tmem_dealloc(tmem, 256);
 }
 
-// G of the pairs cut into several tasks: (pair, first partial, partials, -), the
-// partial blocks added in order
-__global__ void __launch_bounds__(256) k_gram_sum(const int4* __restrict__ multi, int KK,
-                                                  const float* __restrict__ part,
-                                                  float* __restrict__ G) {
-  const int4 q = multi[blockIdx.x];
-  const int e = blockIdx.y * 256 + threadIdx.x;
-  if (e >= KK) return;
-  const float* p = part + (int64_t)q.y * KK + e;
-  float v = 0.f;
-#pragma unroll 8
-  for (int c = 0; c < q.z; ++c) v += p[(int64_t)c * KK];
-  G[(int64_t)q.x * KK + e] = v;
-}
-
 // out[n] = Gram block (which[n].x: its index, < 0 a zero block; which[n].y: transposed)
 __global__ void __launch_bounds__(256) k_gram_blocks(const int2* __restrict__ which, int K,
                                                      const float* __restrict__ G,
@@ -264,31 +251,20 @@ __global__ void __launch_bounds__(256) k_gram_blocks(const int2* __restrict__ wh
 
 }  // namespace
 
-// Pairs (i <= j) with shared rows, their tasks and the runs of each (host),
-// for the assembled system.
+// Pairs (i <= j) with shared rows, the runs of each and the CTA that takes it
+// (host), for the assembled system.
 void gram_build_pairs(elmfb_ctx* h) {
   struct Run {
-    int a, b, len, at;   // panel rows of i and j; the place of the run's first cell
+    int a, b, len;   // panel rows of i and j
   };
   // pairs numbered as the cells meet them, then sorted by (i, j)
   std::unordered_map<uint64_t, int> number;
   std::vector<uint64_t> keys;
   std::vector<std::vector<Run>> runs_of;
+  std::vector<int> first_cell;
   number.reserve(16 * (size_t)h->n_sub);
-  int64_t total = 0;
-  // the cells in square blocks of about 32 MB of panels
-  const double cell_mb = (double)h->NPR * gram_block_bytes(h->K) / 16 / std::max(h->n_cells, 1) / 1e6;
-  const int side = h->dim == 2 ? std::max(1, (int)std::sqrt(32.0 / std::max(cell_mb, 1e-6)))
-                               : std::max(h->nc[0], 1);
-  std::vector<int> visit;
-  visit.reserve(h->n_cells);
-  for (int by = 0; by < h->nc[1]; by += side)
-    for (int bx = 0; bx < h->nc[0]; bx += side)
-      for (int y = by; y < std::min(by + side, h->nc[1]); ++y)
-        for (int x = bx; x < std::min(bx + side, h->nc[0]); ++x)
-          if (h->cell_count[y * h->nc[0] + x] > 0) visit.push_back(y * h->nc[0] + x);
-  for (int at = 0; at < (int)visit.size(); ++at) {
-    const int c = visit[at];
+  for (int c = 0; c < h->n_cells; ++c) {
+    if (h->cell_count[c] == 0) continue;
     const int pad = h->cell_pstart[c + 1] - h->cell_pstart[c];
     for (int e1 = h->cover_off[c]; e1 < h->cover_off[c + 1]; ++e1)
       for (int e2 = e1; e2 < h->cover_off[c + 1]; ++e2) {
@@ -300,67 +276,52 @@ void gram_build_pairs(elmfb_ctx* h) {
         if (fresh) {
           keys.push_back(key);
           runs_of.emplace_back();
+          first_cell.push_back(c);
         }
         auto& v = runs_of[it->second];
         if (!v.empty() && v.back().a + v.back().len == a && v.back().b + v.back().len == b)
           v.back().len += pad;
         else
-          v.push_back({a, b, pad, at});
-        total += pad;
+          v.push_back({a, b, pad});
       }
   }
   std::vector<int> order(keys.size());
   std::iota(order.begin(), order.end(), 0);
   std::sort(order.begin(), order.end(), [&](int x, int y) { return keys[x] < keys[y]; });
   h->gram_pair_ij.clear();
-  // Rows per task: at most 4096 (32 boxes; at K = 128 a partial block is then 3%
-  // of the operands read for it), fewer where that leaves under 16 tasks a CTA.
-  const int64_t cap = std::min<int64_t>(
-      4096, std::max<int64_t>(256, total / (152 * 16) / kCutRows * kCutRows));
   struct Task {
     int4 t;
-    int at;
-    int boxes;   // tiles read
+    int at;      // the pair's first cell
+    int tiles;   // tiles read
   };
   std::vector<Task> tasks;
-  std::vector<int4> runs, multi;
-  int n_part = 0;
+  std::vector<int4> runs;
+  int64_t total = 0;
   for (size_t p = 0; p < order.size(); ++p) {
     const uint64_t key = keys[order[p]];
     h->gram_pair_ij.push_back({(int)(key >> 32), (int)(uint32_t)key});
-    const auto& v = runs_of[order[p]];
     const int diag = (key >> 32) == (uint32_t)key;
-    const size_t t0 = tasks.size();
-    int64_t rows = cap;   // open a task at the first run
-    for (const Run& r : v)
-      for (int off = 0; off < r.len;) {
-        if (rows >= cap) {
-          tasks.push_back({make_int4((int)runs.size(), 0, diag, 0), r.at, 0});
-          rows = 0;
-        }
-        // cuts inside a run at multiples of kCutRows
-        const int room = (int)(cap - rows);
-        const int take = r.len - off <= room ? r.len - off
-                                             : std::max(room / kCutRows * kCutRows, kCutRows);
-        const int len = std::min(take, r.len - off);
-        runs.push_back(make_int4(r.a + off, r.b + off, len, 0));
-        tasks.back().t.y = (int)runs.size();
-        tasks.back().boxes += (int)ceil_div(len, gram_box_rows(h->K)) * (2 - diag);
-        off += len;
-        rows += len;
-      }
-    const int n = (int)(tasks.size() - t0);
-    for (int k = 0; k < n; ++k) tasks[t0 + k].t.w = n == 1 ? (int)p : ~(n_part + k);
-    if (n > 1) {
-      multi.push_back(make_int4((int)p, n_part, n, 0));
-      n_part += n;
+    const int r0 = (int)runs.size();
+    int boxes = 0;
+    for (const Run& r : runs_of[order[p]]) {
+      runs.push_back(make_int4(r.a, r.b, r.len, 0));
+      boxes += (int)ceil_div(r.len, gram_box_rows(h->K));
     }
+    tasks.push_back({make_int4(r0, (int)runs.size(), 2 * boxes + diag, (int)p),
+                     first_cell[order[p]], boxes * (2 - diag)});
+    total += tasks.back().tiles;
   }
-  std::stable_sort(tasks.begin(), tasks.end(),
-                   [](const Task& x, const Task& y) { return x.at < y.at; });
   int sms = 0;
   CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
   const int ctas = (int)std::min<size_t>(tasks.size(), sms);
+  // pairs above an eighth of a CTA's share first, the longest before the others;
+  // the rest in the order of their first cell
+  const int64_t large = total / std::max(ctas, 1) / 8;
+  std::stable_sort(tasks.begin(), tasks.end(), [large](const Task& x, const Task& y) {
+    const bool lx = x.tiles > large, ly = y.tiles > large;
+    if (lx != ly) return lx;
+    return lx ? x.tiles > y.tiles : x.at < y.at;
+  });
   std::vector<int> owner(tasks.size()), task_off(ctas + 1, 0);
   {
     typedef std::pair<int64_t, int> Load;   // tiles so far, CTA
@@ -371,7 +332,7 @@ void gram_build_pairs(elmfb_ctx* h) {
       idle.pop();
       owner[k] = l.second;
       task_off[l.second + 1]++;
-      idle.push({l.first + tasks[k].boxes + 8, l.second});   // 8: a task's own cost
+      idle.push({l.first + tasks[k].tiles + 8, l.second});   // 8: a task's own cost
     }
     for (int c = 0; c < ctas; ++c) task_off[c + 1] += task_off[c];
   }
@@ -385,8 +346,6 @@ void gram_build_pairs(elmfb_ctx* h) {
                              cudaMemcpyHostToDevice, h->stream));
   h->gram_ctas = ctas;
   h->n_gram_pairs = (int64_t)order.size();
-  h->gram_multi = (int)multi.size();
-  h->gram_parts = n_part;
   auto up = [&](DevBuf& d, const std::vector<int4>& v) {
     d.alloc(std::max<size_t>(v.size(), 1) * sizeof(int4), h->stream);
     if (!v.empty())
@@ -395,7 +354,6 @@ void gram_build_pairs(elmfb_ctx* h) {
   };
   up(h->d_gram_tasks, flat);
   up(h->d_gram_runs, runs);
-  up(h->d_gram_multi, multi);
 }
 
 void gram_compute(elmfb_ctx* h) {
@@ -407,8 +365,6 @@ void gram_compute(elmfb_ctx* h) {
   const int K = h->K;
   const int N = (K + 15) & ~15;
   h->d_gram.alloc(std::max<int64_t>(h->n_gram_pairs, 1) * K * K * sizeof(float), st);
-  DevBuf dpart;
-  dpart.alloc((size_t)h->gram_parts * K * K * sizeof(float), st);
   ensure_dyn_smem((const void*)k_gram_tc, kGramSmem);
   CUDA_CHECK(cudaMemsetAsync(h->d_flags.p, 0, 16 * sizeof(int), st));
   stage_begin(h, 3);
@@ -418,13 +374,7 @@ void gram_compute(elmfb_ctx* h) {
     const int S = (int)std::min<size_t>(kMaxGramStages, kGramRing / (2 * gram_tile_bytes(K)));
     k_gram_tc<<<(unsigned)h->gram_ctas, kGramThreads, kGramSmem, st>>>(
         h->d_pt.as<uint8_t>(), h->d_gram_tasks.as<int4>(), h->d_gram_task_off.as<int>(),
-        h->d_gram_runs.as<int4>(), K, N, S, h->d_gram.as<float>(), dpart.as<float>(),
-        h->d_flags.as<int>());
-    if (h->gram_multi > 0) {
-      k_gram_sum<<<dim3((unsigned)h->gram_multi, (unsigned)ceil_div(K * K, 256)), 256, 0, st>>>(
-          h->d_gram_multi.as<int4>(), K * K, dpart.as<float>(), h->d_gram.as<float>());
-      count_launch(h);
-    }
+        h->d_gram_runs.as<int4>(), K, N, S, h->d_gram.as<float>(), h->d_flags.as<int>());
   }
   prof_end(h, KID_GRAM_TC);
   check_launch("k_gram_tc");

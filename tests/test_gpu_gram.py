@@ -125,3 +125,46 @@ def test_pair_count_before_and_after_the_gram_blocks(make):
         n = s.sizes().n_gram_pairs
         s.compute_gram()
         assert s.sizes().n_gram_pairs == n
+
+
+def _scattered(n, box, seed):
+    r = np.random.default_rng(seed)
+    lo, hi = np.array(box[0]), np.array(box[1])
+    return lo + (hi - lo) * r.random((n, 2))
+
+
+@pytest.mark.parametrize("K,n", [(32, 40000), (128, 40000)])
+def test_gram_block_depends_on_its_own_rows_only(K, n):
+    """A pair's block is one accumulation over its rows: the blocks of the
+    subdomains left of x = 0.5 have the same bits whether the other half of the
+    domain holds a few points or most of them.  (The second system has four
+    times the interior points, so its rows are scaled by exactly 1/2.)
+
+    They also agree with the FP64 products of the rounded operands -- BF16 of
+    the panels' own FP32 entries -- to FP32 accumulation over steps of 16 rows,
+    each step truncated at 2^-23 of the accumulated magnitude in each of its
+    partial sums (2^-22 a step): a lost row of a pair's thousands would
+    show."""
+    left = _scattered(n, ((0.0, 0.0), (0.45, 1.0)), 1)
+    few = _scattered(n // 8, ((0.75, 0.0), (1.0, 1.0)), 2)
+    many = _scattered(4 * (n + n // 8) - n, ((0.75, 0.0), (1.0, 1.0)), 3)
+    # single level, 4 x 4 subdomains of half-width 1/4: those of columns 0 and 1
+    # end at x = 0.625
+    pairs = [(0, 0), (0, 1), (1, 5), (4, 5), (9, 9), (8, 13)]
+    out, T = [], None
+    for right in (few, many):
+        x = np.concatenate([left, right])
+        with E.Solver(2, (0.0, 0.0), (1.0, 1.0), (4,), 2.0, K, precision=E.MIXED) as s:
+            s.assemble([dict(points=x, rhs=np.zeros(len(x)), c2=(-1.0, -1.0))])
+            s.compute_gram()
+            out.append(s.gram_blocks(pairs))
+            if T is None:
+                T = s.get_rows(np.arange(n))[0]
+    assert np.array_equal(out[0], 4.0 * out[1])
+    B = _bf16(T)
+    for q, (i, j) in enumerate(pairs):
+        bi, bj = B[:, i * K:(i + 1) * K], B[:, j * K:(j + 1) * K]
+        # rows of cells that the supports share, padded to 16 a cell (16 cells at most)
+        steps = np.count_nonzero(np.abs(bi).any(1) & np.abs(bj).any(1)) / 16 + 16
+        mag = np.abs(bi).T @ np.abs(bj)
+        assert np.all(np.abs(out[0][q] - bi.T @ bj) <= steps * 2.0 ** -22 * mag)
