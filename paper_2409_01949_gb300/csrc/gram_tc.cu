@@ -23,18 +23,18 @@
 // pieces 4 MB apart: 4.3 GB of DRAM reads for 0.57 GB of panels at 400^2 points,
 // K = 128, at a third of the DRAM rate.)
 //
-// A pair's rows are cut into tasks of a bounded number of rows, and one persistent
-// CTA per SM walks its list of them: a producer warp, an MMA warp and four
-// epilogue warps, with two accumulators, so that the ring runs on across tasks
-// while the last one's block is stored.  A pair of several tasks sums their blocks
-// in order (k_gram_sum).  Cells are visited in square blocks of 32 MB of panels
-// and tasks dealt in the order of their first cell, each to the CTA with the least
-// work so far, so that all CTAs are in the same place at the same time and the
-// panels stay in L2: with one CTA per pair, pair after pair, the coarse panels'
-// pairs each streamed the whole domain, and the level-1 pair alone was 2525 boxes
-// of one CTA.  400^2 points, levels 1..16, K = 128 (6297 pairs): 1.64 -> 0.75 ms,
-// 330 -> 730 TFLOP/s; 2048^2, levels 1..64, K = 64: 49.6 -> 33.4 ms, 170 -> 253
-// TFLOP/s (half of each MMA's rows are past K there).
+// One persistent CTA per SM walks its list of pairs: a producer warp, an MMA warp
+// and four epilogue warps, with two accumulators, so that the ring runs on across
+// pairs while the last one's block is stored.  A pair is one accumulation chain over
+// its rows in cell order, so that its block depends on its own rows only: the tensor
+// cores truncate each step's sum, and a chain cut by the system's size would move a
+// block by up to 5e-5 of its norm from system to system.  The longest chain (level 1
+// with itself: 1263 boxes of one CTA) takes about as long as all CTAs' shares.
+// Large pairs are dealt first, the rest in the order of their first cell, each to
+// the CTA with the least work so far, so that all CTAs are in the same place at the
+// same time and the panels stay in L2.  400^2 points, levels 1..16, K = 128 (6297
+// pairs), against one CTA per pair, pair after pair: 1.64 -> 0.79 ms, 330 -> 690
+// TFLOP/s.
 //
 // Every mbarrier wait is bounded; a timeout raises flags[2].
 #include <algorithm>
@@ -291,8 +291,8 @@ void gram_build_pairs(elmfb_ctx* h) {
   h->gram_pair_ij.clear();
   struct Task {
     int4 t;
-    int at;      // the pair's first cell
-    int tiles;   // tiles read
+    int at;   // the pair's first cell
+    int boxes;
   };
   std::vector<Task> tasks;
   std::vector<int4> runs;
@@ -308,23 +308,25 @@ void gram_build_pairs(elmfb_ctx* h) {
       boxes += (int)ceil_div(r.len, gram_box_rows(h->K));
     }
     tasks.push_back({make_int4(r0, (int)runs.size(), 2 * boxes + diag, (int)p),
-                     first_cell[order[p]], boxes * (2 - diag)});
-    total += tasks.back().tiles;
+                     first_cell[order[p]], boxes});
+    total += boxes;
   }
   int sms = 0;
   CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
   const int ctas = (int)std::min<size_t>(tasks.size(), sms);
-  // pairs above an eighth of a CTA's share first, the longest before the others;
-  // the rest in the order of their first cell
+  // A box costs its CTA about the same whether one tile or two are read for it, so
+  // boxes are what is shared out (by tiles: 0.99 instead of 0.79 ms).  Pairs above an
+  // eighth of a CTA's share first, the longest before the others (all in spatial
+  // order: 0.97 ms); the rest in the order of their first cell.
   const int64_t large = total / std::max(ctas, 1) / 8;
   std::stable_sort(tasks.begin(), tasks.end(), [large](const Task& x, const Task& y) {
-    const bool lx = x.tiles > large, ly = y.tiles > large;
+    const bool lx = x.boxes > large, ly = y.boxes > large;
     if (lx != ly) return lx;
-    return lx ? x.tiles > y.tiles : x.at < y.at;
+    return lx ? x.boxes > y.boxes : x.at < y.at;
   });
   std::vector<int> owner(tasks.size()), task_off(ctas + 1, 0);
   {
-    typedef std::pair<int64_t, int> Load;   // tiles so far, CTA
+    typedef std::pair<int64_t, int> Load;   // boxes so far, CTA
     std::priority_queue<Load, std::vector<Load>, std::greater<Load>> idle;
     for (int c = 0; c < ctas; ++c) idle.push({0, c});
     for (size_t k = 0; k < tasks.size(); ++k) {
@@ -332,7 +334,7 @@ void gram_build_pairs(elmfb_ctx* h) {
       idle.pop();
       owner[k] = l.second;
       task_off[l.second + 1]++;
-      idle.push({l.first + tasks[k].tiles + 8, l.second});   // 8: a task's own cost
+      idle.push({l.first + tasks[k].boxes + 8, l.second});   // 8: a task's own cost
     }
     for (int c = 0; c < ctas; ++c) task_off[c + 1] += task_off[c];
   }
