@@ -558,24 +558,27 @@ __device__ __noinline__ double entry64(double w0, double w1, double b, double x0
 }
 
 // K1 for FP64 entries and FP32 pairs (kSplit) in fixed point (fixed.cuh): phase
-// 1 as k_assemble, in FP64; phase 2 in integers.  A row's terms share an
-// exponent er, 2^er above the largest of |A|, |beta_i w / sigma_i|, 2 |gamma_i
-// (w / sigma_i)^2| over |w| <= 2^wexp, and become
+// 1 as k_assemble, in FP64; phase 2 in integers:
 //     M = phi A + (1 - phi^2) D = D + phi (A - phi D),  D = B - phi C,
-//     B = sum beta_i u_i,  C = sum 2 gamma_i u_i^2,  u = w / 2^wexp,
-// in units of 2^(er - 59): every term of a row is held to
-// 2^-59 of the row's largest, where FP64 rounds each operation to 2^-53 of its
-// result.  The sum is rounded once, to a double or to an FP32 pair.
+//     B = sum b_i u_i 2^-s_i,  C = sum c_i u_i^2 2^-2 s_i,
+// with w_i / 2^wexp = u_i 2^-s_i, |u_i| in [1/2, 1], and b_i = beta_i 2^wexp /
+// sigma_i, c_i = 2 gamma_i (2^wexp / sigma_i)^2.  A, b_i and c_i of a row are 60-bit
+// mantissas with an exponent each; an entry's five terms are aligned to the largest
+// of them, 2^er, and added in units of 2^(er - 59), so that an entry of a small
+// weight, or of a row without some of the terms, is held as well as any other (with
+// one exponent for a row, entries of w = 2^-6 where one subdomain covers the point
+// had a relative error of 4e-13).  phi is held to 2^-60: features whose weights and
+// bias are all below 2^-5 of the scale, or 2^-6, are evaluated in FP64, which holds
+// their phi to its own last place.  The sum is rounded once, to a double or to an
+// FP32 pair.
 //
 // The FP64 form is bound by the FP64 pipe (47 instructions an entry, 3020
-// cycles of a sub-partition for a warp's 32 entries); this one by integer issue
-// (ncu: 50% issue-active, the multiply-add pipe 51%), with phase 1's FP64 work
-// beside it.  400^2 points, levels 1..16, K = 128: assembly and one LSQR step
-// 29.5 -> 10.1 ms with this kernel, 7.1 ms with the host work around it cut and
-// the products as single multiply-adds (that last step 8.4 -> 7.1 ms); the
-// oscillator (20000 points, levels 1..64, K = 96, pairs), four LSQR steps: 4.18
-// -> 1.63 ms, then 1.36 ms.  Entries against a 113-bit evaluation: 1.5e-16
-// -> 0.9e-16 of the system's norm in FP64, the pairs' 48 bits as before.
+// cycles of a sub-partition for a warp's 32 entries); this one by integer issue,
+// with phase 1's FP64 work beside it.  400^2 points, levels 1..16, K = 128: 23.9 ->
+// 3.7 ms (the exponents of its own for every term are 0.17 ms of it), assembly and
+// one LSQR step 29.5 -> 7.3 ms; the oscillator (20000 points, levels 1..64, K = 96,
+// pairs): 2.59 -> 0.34 ms.  Entries against a 113-bit evaluation: 1.5e-16 -> 0.9e-16
+// of the system's norm in FP64, the pairs' 48 bits as before.
 //
 // 1-D window factor f = 4 c^4 with (s, c) = sincos(pi x / 2), x = dx / sigma, its
 // derivatives (file header), and x in units of 2^-61.  Sine and cosine come
@@ -617,18 +620,19 @@ __device__ __forceinline__ void window_axis(double dx, double sigma, double inv,
   fpp = 4.0 * c2 * (3.0 - 4.0 * c2) * g * g;   // 3 s^2 - c^2, s^2 = 1 - c^2
 }
 
-struct RowTerms {   // one row of phase 2, as four 16-byte words
-  int4 a;    // A59.hi, A59.lo, er (kRow64: in FP64), -
-  int4 b;    // beta'' of axis 0 (hi, lo), axis 1
-  int4 c;    // 2 gamma'' of axis 0, axis 1
-  int4 x;    // scaled coordinates
+struct RowTerms {   // one row of phase 2, as 16-byte words (the last two: two axes only)
+  int4 a;    // A (low, high word), its exponent (kRow64: in FP64), that of b0
+  int4 b;    // b0 and c0 (hi, lo)
+  int4 x;    // scaled coordinates; one axis: x0, the exponent of c0, -
+  int4 c;    // b1 and c1
+  int4 e;    // exponents of c0, b1, c1, -
+  double f[6];   // A, beta of both axes, gamma of both, -: for entries in FP64
 };
 constexpr int kRow64 = INT_MIN;
-
-constexpr int kFxFeatures = 2;   // a lane's features of one pass over a panel's rows
+constexpr int kNoExp = -8000;    // exponent of a zero term
 
 template <bool kSplit, bool kTwo>
-__global__ void __launch_bounds__(64, 8) k_assemble_fx(
+__global__ void __launch_bounds__(128, 4) k_assemble_fx(
     const int4* __restrict__ tiles, int64_t n_tiles, int K, int nl_max,
     const SubGeom* __restrict__ sub, const int* __restrict__ cover_sub,
     const int* __restrict__ entry_cell, const int* __restrict__ cell_count,
@@ -702,6 +706,7 @@ __global__ void __launch_bounds__(64, 8) k_assemble_fx(
   }
   const double wsc = scalbn(1.0, wexp);
   const double w_in = scalbn(1.0, 61 - wexp), b_in = scalbn(1.0, 60 - wexp);
+  const double w_low = fmax(scalbn(1.0, wexp - 5), 0x1p-6);
 
   for (int k = 0; k < nl; ++k) {
     const int e = e0 + k;
@@ -742,143 +747,189 @@ __global__ void __launch_bounds__(64, 8) k_assemble_fx(
     __syncwarp();   // the previous panel's row terms have been read
     {
       const double s0 = is0 * wsc, s1 = is1 * wsc;
-      const double B0 = be0 * s0, B1 = be1 * s1;
-      const double C0 = 2.0 * ga0 * (s0 * s0), C1 = 2.0 * ga1 * (s1 * s1);
-      auto expo = [](double v) { return (__double2hiint(v) >> 20) & 0x7ff; };
-      const int ef = max(max(expo(A), max(expo(B0), expo(B1))), max(expo(C0), expo(C1)));
-      const bool zero = A == 0.0 && B0 == 0.0 && B1 == 0.0 && C0 == 0.0 && C1 == 0.0;
-      const bool fits = zero || (ef > 150 && ef < 1900);
-      const int er = zero ? 0 : ef - 1022;
-      const double q = fits ? scalbn(1.0, 60 - er) : 0.0;
-      auto fixed = [&](double v) { return fx::split(fits ? __double2ll_rn(v * q) : 0ll); };
-      const fx::Val a = fixed(0.5 * A), b0 = fixed(B0), b1 = fixed(B1), c0 = fixed(C0),
-                    c1 = fixed(C1);
-      const fx::Val v0 = fx::split(y0), v1 = fx::split(y1);
-      rowt[lane].a = make_int4(a.hi, a.lo, fits ? er : kRow64, 0);
-      rowt[lane].b = make_int4(b0.hi, b0.lo, b1.hi, b1.lo);
-      rowt[lane].c = make_int4(c0.hi, c0.lo, c1.hi, c1.lo);
-      rowt[lane].x = make_int4(v0.hi, v0.lo, v1.hi, v1.lo);
+      const double v[5] = {A, be0 * s0, 2.0 * ga0 * (s0 * s0), be1 * s1, 2.0 * ga1 * (s1 * s1)};
+      int top = 0;
+      bool zero = true;
+#pragma unroll
+      for (int i = 0; i < 5; ++i) {
+        top = max(top, (__double2hiint(v[i]) >> 20) & 0x7ff);
+        zero = zero && v[i] == 0.0;
+      }
+      // an entry's exponent is at most 48 below its largest term's (|w| >= 2^-24
+      // of the scale), and terms 200 below the row's largest add nothing to it
+      const bool fits = zero || (top > 350 && top < 1900);
+      int64_t m[5];
+      int ex[5];
+#pragma unroll
+      for (int i = 0; i < 5; ++i) {
+        const int ef = (__double2hiint(v[i]) >> 20) & 0x7ff;
+        const int64_t bits = __double_as_longlong(v[i]);
+        const int64_t mag = ((bits & 0xfffffffffffffll) | 0x10000000000000ll) << 7;
+        const bool on = fits && !zero && ef >= top - 200;
+        m[i] = on ? (bits < 0 ? -mag : mag) : 0ll;
+        ex[i] = on ? ef - 1022 : kNoExp;
+      }
+      const fx::Val b0 = fx::split(m[1]), c0 = fx::split(m[2]), v0 = fx::split(y0);
+      rowt[lane].a = make_int4((int)(uint32_t)m[0], (int)(m[0] >> 32), fits ? ex[0] : kRow64, ex[1]);
+      rowt[lane].b = make_int4(b0.hi, b0.lo, c0.hi, c0.lo);
+      rowt[lane].f[0] = A;
+      rowt[lane].f[1] = be0;
+      rowt[lane].f[2] = be1;
+      rowt[lane].f[3] = ga0;
+      rowt[lane].f[4] = ga1;
+      if (kTwo) {
+        const fx::Val b1 = fx::split(m[3]), c1 = fx::split(m[4]), v1 = fx::split(y1);
+        rowt[lane].x = make_int4(v0.hi, v0.lo, v1.hi, v1.lo);
+        rowt[lane].c = make_int4(b1.hi, b1.lo, c1.hi, c1.lo);
+        rowt[lane].e = make_int4(ex[2], ex[3], ex[4], 0);
+      } else {
+        rowt[lane].x = make_int4(v0.hi, v0.lo, ex[2], 0);
+      }
     }
     __syncwarp();
     double* out = panels + entry_base[e] * (int64_t)K + (int64_t)p0 * rstride;
-    // 64 features at a time: two a lane keep the registers for four blocks an SM
-    for (int f0 = 0; f0 < K; f0 += 32 * kFxFeatures) {
-      // this lane's features f0 + lane + 32 i: weights, their squares, bias
-      fx::Val w0[kFxFeatures], w1[kFxFeatures], q0[kFxFeatures], q1[kFxFeatures];
-      int64_t bb[kFxFeatures];
-#pragma unroll
-      for (int i = 0; i < kFxFeatures; ++i) {
-        const int f = f0 + lane + 32 * i;
-        const int64_t q = (int64_t)s * K + f;
-        const bool on = f < K;
-        w0[i] = fx::split(on ? __double2ll_rn(W[q * dim] * w_in) : 0ll);
-        q0[i] = fx::split(fx::mul_add(w0[i], w0[i], 0) << 1);
-        w1[i] = fx::split(on && kTwo ? __double2ll_rn(W[q * dim + 1] * w_in) : 0ll);
-        q1[i] = fx::split(fx::mul_add(w1[i], w1[i], 0) << 1);
-        bb[i] = on ? __double2ll_rn(Bias[q] * b_in) : 0ll;
-      }
+    // 32 features at a time, one a lane (two a lane spill: 3.71 -> 3.81 ms of the 2-D
+    // system above)
+    for (int f0 = 0; f0 < K; f0 += 32) {
+      // this lane's feature: bias, and per axis the weight in the scale's units and
+      // as u 2^-s with |u| in [1/2, 1], and u^2
+      const int f = f0 + lane;
+      const bool on = f < K;
+      const int64_t q = (int64_t)s * K + f;
+      const double wd0 = on ? W[q * dim] : 0.0, wd1 = on && kTwo ? W[q * dim + 1] : 0.0;
+      const double bd = on ? Bias[q] : 0.0;
+      fx::Val w0, w1, u0, u1, q0, q1;
+      int s0, s1;
+      auto weight = [&](double v, fx::Val& w, fx::Val& u, fx::Val& sq, int& sh) {
+        sh = v == 0.0 ? 0 : max(wexp - 1 - ilogb(v), 0);
+        w = fx::split(__double2ll_rn(v * w_in));
+        u = fx::split(__double2ll_rn(scalbn(v * w_in, sh)));
+        sq = fx::split(fx::mul_add(u, u, 0) << 1);
+      };
+      weight(wd0, w0, u0, q0, s0);
+      weight(wd1, w1, u1, q1, s1);
+      const int64_t bb = __double2ll_rn(bd * b_in);
+      const bool low = on && fmax(fmax(fabs(wd0), fabs(wd1)), fabs(bd)) < w_low;
+      // entries in FP64; of a feature below w_low, every lane its own row's
+      auto store64 = [&](double* at, double v) {
+        if (kSplit) {
+          const float hi = __double2float_rn(v);
+          *reinterpret_cast<float2*>(at) = make_float2(hi, __double2float_rn(v - (double)hi));
+          if (panels32) panels32[at - panels] = hi;
+        } else {
+          *at = v;
+        }
+      };
+      auto in64 = [&](int r, int col) {
+        const int64_t qc = (int64_t)s * K + col;
+        const double* rf = rowt[r].f;
+        const int4 rx = rowt[r].x;
+        const double ux0 = ((double)rx.x * 0x1p31 + (double)rx.y) * 0x1p-61;
+        const double ux1 = kTwo ? ((double)rx.z * 0x1p31 + (double)rx.w) * 0x1p-61 : 0.0;
+        store64(out + (int64_t)r * rstride + col,
+                entry64(W[qc * dim], kTwo ? W[qc * dim + 1] : 0.0, Bias[qc], ux0, ux1, is0, is1,
+                        rf[0], rf[1], rf[2], rf[3], rf[4]));
+      };
+      for (unsigned m = __ballot_sync(0xffffffffu, low); m; m &= m - 1)
+        if (lane < nrows) in64(lane, f0 + __ffs(m) - 1);
 
-      // phase 2: row by row, every lane its own features
+      // phase 2: row by row, every lane its own feature
       for (int r = 0; r < nrows; ++r) {
-        const int4 ra = rowt[r].a, rb = rowt[r].b, rg = rowt[r].c, rx = rowt[r].x;
+        const int4 ra = rowt[r].a, rb = rowt[r].b, rx = rowt[r].x;
         double* orow = out + (int64_t)r * rstride;
         if (ra.z == kRow64) {
-          const double uA = __shfl_sync(0xffffffffu, A, r);
-          const double ub0 = __shfl_sync(0xffffffffu, be0, r), ub1 = __shfl_sync(0xffffffffu, be1, r);
-          const double ug0 = __shfl_sync(0xffffffffu, ga0, r), ug1 = __shfl_sync(0xffffffffu, ga1, r);
-          const double ux0 = (double)__shfl_sync(0xffffffffu, y0, r) * 0x1p-61;
-          const double ux1 = (double)__shfl_sync(0xffffffffu, y1, r) * 0x1p-61;
-          for (int f = f0 + lane; f < min(K, f0 + 32 * kFxFeatures); f += 32) {
-            const int64_t q = (int64_t)s * K + f;
-            const double v = entry64(W[q * dim], kTwo ? W[q * dim + 1] : 0.0, Bias[q], ux0, ux1, is0,
-                                     is1, uA, ub0, ub1, ug0, ug1);
-            if (kSplit) {
-              const float hi = __double2float_rn(v);
-              reinterpret_cast<float2*>(orow)[f] = make_float2(hi, __double2float_rn(v - (double)hi));
-              if (panels32) panels32[(orow - panels) + f] = hi;
-            } else {
-              orow[f] = v;
-            }
-          }
+          if (on) in64(r, f);
           continue;
         }
-#pragma unroll
-        for (int i = 0; i < kFxFeatures; ++i) {
-          if (f0 + 32 * i >= K) break;   // warp-uniform
-          const int64_t arg = fx::argument(w0[i], {rx.x, rx.y}, w1[i], {rx.z, rx.w}, bb[i], kTwo);
-          const int64_t phi = fx::tanh61(arg, 54 - wexp, tab, rows);
-          const fx::Val p = fx::split(phi << 1);   // units of 2^-62
-          // B and C, then D = B - phi C (2^(er - 59))
-          int64_t xb = fx::mad(rb.x, w0[i].lo, fx::mad(rb.y, w0[i].hi, 1 << 30));
-          int64_t xc = fx::mad(rg.x, q0[i].lo, fx::mad(rg.y, q0[i].hi, 1 << 30));
-          int64_t B = fx::mad(rb.x, w0[i].hi, 0), C = fx::mad(rg.x, q0[i].hi, 0);
-          if (kTwo) {
-            xb = fx::mad(rb.z, w1[i].lo, fx::mad(rb.w, w1[i].hi, xb));
-            xc = fx::mad(rg.z, q1[i].lo, fx::mad(rg.w, q1[i].hi, xc));
-            B = fx::mad(rb.z, w1[i].hi, B);
-            C = fx::mad(rg.z, q1[i].hi, C);
-          }
-          B += xb >> 31;
-          C += xc >> 31;
-          const int64_t D = B - fx::mul_add(p, fx::split(C), 0);
-          // M = D + phi (A - phi D) (2^(er - 59))
-          const int64_t A59 = ((int64_t)ra.x << 31) + ra.y;
-          const int64_t M =
-              fx::mul_add(p, fx::split(A59 - fx::mul_add(p, fx::split(D), 0)), D);
-          const int f = f0 + lane + 32 * i;
-          if (f >= K) continue;
-          // M 2^(er - 59) as n 2^(ex - 63), n's top bit set
-          const uint64_t m = (uint64_t)(M < 0 ? -M : M);
-          const int lz = __clzll((long long)m);
-          const uint64_t nrm = m << (lz & 63);
-          const int ex = ra.z + 4 - lz;
-          const uint64_t odd = (nrm >> 11) & 1;
-          const uint64_t man = (nrm >> 11) + ((nrm & 0x7ff) + odd > 0x400);   // to nearest even
-          const uint64_t sign = (uint64_t)M & 0x8000000000000000ull;
-          if (kSplit) {
-            float2 hl;
-            if (ex > -72 && ex < 100 && m != 0) {   // both parts in FP32's normal range
-              // the double's top 24 bits to nearest even, and the rest
-              const uint32_t h24 = (uint32_t)(man >> 29), rest = (uint32_t)man & 0x1fffffffu;
-              const uint32_t up = rest + (h24 & 1) > 0x10000000u;
-              const uint32_t sg = (uint32_t)(sign >> 32);
-              hl.x = __uint_as_float((((uint32_t)(ex + 126) << 23) + h24 + up) | sg);
-              const float lo = __int2float_rn((int)rest - (int)(up << 29)) *
-                               __uint_as_float((uint32_t)(ex - 52 + 127) << 23);
-              hl.y = __uint_as_float(__float_as_uint(lo) ^ sg);
-            } else {
-              const double v = m == 0 ? 0.0
-                                      : __longlong_as_double((long long)(
-                                            (((uint64_t)(ex + 1022) << 52) + man) | sign));
-              hl.x = __double2float_rn(v);
-              hl.y = __double2float_rn(v - (double)hl.x);
-            }
-            reinterpret_cast<float2*>(orow)[f] = hl;
-            if (panels32) panels32[(orow - panels) + f] = hl.x;
+        int4 rg, re;
+        if (kTwo) rg = rowt[r].c, re = rowt[r].e;
+        const int64_t arg = fx::argument(w0, {rx.x, rx.y}, w1, {rx.z, rx.w}, bb, kTwo);
+        const int64_t phi = fx::tanh61(arg, 54 - wexp, tab, rows);
+        const fx::Val p = fx::split(phi << 1);   // units of 2^-62
+        // the terms' exponents and the largest of them, er
+        const int eb0 = ra.w - s0, ec0 = (kTwo ? re.x : rx.z) - 2 * s0;
+        const int eb1 = kTwo ? re.y - s1 : 0, ec1 = kTwo ? re.z - 2 * s1 : 0;
+        int er = max(ra.z, max(eb0, ec0));
+        if (kTwo) er = max(er, max(eb1, ec1));
+        // B and C, then D = B - phi C (2^(er - 59))
+        int64_t B = fx::down(fx::mul_add({rb.x, rb.y}, u0, 0), er - eb0);
+        int64_t C = fx::down(fx::mul_add({rb.z, rb.w}, q0, 0), er - ec0);
+        if (kTwo) {
+          B += fx::down(fx::mul_add({rg.x, rg.y}, u1, 0), er - eb1);
+          C += fx::down(fx::mul_add({rg.z, rg.w}, q1, 0), er - ec1);
+        }
+        const int64_t D = B - fx::mul_add(p, fx::split(C), 0);
+        // M = D + phi (A - phi D) (2^(er - 59))
+        const int64_t A59 =
+            fx::down((int64_t)(((uint64_t)(uint32_t)ra.y << 32) | (uint32_t)ra.x), er - ra.z + 1);
+        const int64_t M =
+            fx::mul_add(p, fx::split(A59 - fx::mul_add(p, fx::split(D), 0)), D);
+        if (!on || low) continue;
+        // M 2^(er - 59) as n 2^(ex - 63), n's top bit set
+        const uint64_t m = (uint64_t)(M < 0 ? -M : M);
+        const int lz = __clzll((long long)m);
+        const uint64_t nrm = m << (lz & 63);
+        const int ex = er + 4 - lz;
+        const uint64_t odd = (nrm >> 11) & 1;
+        const uint64_t man = (nrm >> 11) + ((nrm & 0x7ff) + odd > 0x400);   // to nearest even
+        const uint64_t sign = (uint64_t)M & 0x8000000000000000ull;
+        if (kSplit) {
+          float2 hl;
+          if (ex > -72 && ex < 100 && m != 0) {   // both parts in FP32's normal range
+            // the double's top 24 bits to nearest even, and the rest
+            const uint32_t h24 = (uint32_t)(man >> 29), rest = (uint32_t)man & 0x1fffffffu;
+            const uint32_t up = rest + (h24 & 1) > 0x10000000u;
+            const uint32_t sg = (uint32_t)(sign >> 32);
+            hl.x = __uint_as_float((((uint32_t)(ex + 126) << 23) + h24 + up) | sg);
+            const float lo = __int2float_rn((int)rest - (int)(up << 29)) *
+                             __uint_as_float((uint32_t)(ex - 52 + 127) << 23);
+            hl.y = __uint_as_float(__float_as_uint(lo) ^ sg);
           } else {
-            orow[f] = m == 0 ? 0.0
-                             : __longlong_as_double(
-                                   (long long)((((uint64_t)(ex + 1022) << 52) + man) | sign));
+            const double v = m == 0 ? 0.0
+                                    : __longlong_as_double((long long)(
+                                          (((uint64_t)(ex + 1022) << 52) + man) | sign));
+            hl.x = __double2float_rn(v);
+            hl.y = __double2float_rn(v - (double)hl.x);
           }
+          reinterpret_cast<float2*>(orow)[f] = hl;
+          if (panels32) panels32[(orow - panels) + f] = hl.x;
+        } else {
+          orow[f] = m == 0 ? 0.0
+                           : __longlong_as_double(
+                                 (long long)((((uint64_t)(ex + 1022) << 52) + man) | sign));
         }
       }
     }
   }
 }
 
-// FP64-accurate entries in fixed point: weight scales 1/16 .. 1, at which
+// FP64-accurate entries in fixed point: weight scales above 1/16 up to 1, at which
 // arguments stay within +-3 and 1 - phi^2 above 2^-7, so that its 2^-60 absolute
-// error is no larger than FP64's relative one; larger and smaller scales keep
-// the FP64 form.  False: not taken.
+// error is no larger than FP64's relative one, and phi's is below FP64's own error
+// of the argument (root mean square over an entry's terms, against 113 bits: 0.7e-16
+// or less where FP64 has 1.1e-16; 1.6e-16 at a scale of 1/16); larger and smaller
+// scales keep the FP64 form.  False: not taken.
+constexpr int kMinAssembleExp = -3;
 bool launch_assemble_fx(elmfb_ctx* h, bool split, double* panels, float* panels32,
                         const Ansatz& an) {
   const double a = h->cfg.weight_scale;
   const int wexp = a > 0.0 ? fx::weight_exp(a) : 1;
-  if (wexp < fx::kMinExp || wexp > 0) return false;
-  const int rows = fx::tanh_rows(h->dim, wexp), warps = 2;
-  const size_t smem = (size_t)rows * 3 * sizeof(int4) + warps * 32 * sizeof(RowTerms) +
-                      (size_t)warps * h->nl_max * kFacVals * 32 * sizeof(double);
-  if (smem > 220 * 1024) return false;
+  if (wexp < kMinAssembleExp || wexp > 0) return false;
+  const int rows = fx::tanh_rows(h->dim, wexp);
+  // warps a block: those that put most of the 16 that the registers allow on an SM
+  // (a block has one copy of the table), the larger block where two are equal; fewer
+  // where the tiles would not give every SM a block
+  auto block_smem = [&](int warps) {
+    return (size_t)rows * 3 * sizeof(int4) +
+           warps * 32 * (sizeof(RowTerms) + (size_t)h->nl_max * kFacVals * sizeof(double));
+  };
+  int warps = 0, most = 0;
+  for (int w : {4, 2, 1}) {
+    const int fit = w * (int)std::min<size_t>(220 * 1024 / (block_smem(w) + 1024), 16 / w);
+    if (fit > most || (fit > 0 && h->n_ltiles < 152 * 2 * w)) most = fit, warps = w;
+  }
+  if (warps == 0) return false;
+  const size_t smem = block_smem(warps);
   prof_begin(h, KID_ASSEMBLE, (double)h->NPR * h->K * (8.0 + (panels32 ? 4.0 : 0.0)) +
                                   (double)h->NR * (8.0 * h->dim + 4.0));
 #define ELMFB_K1FX(SP, TWO)                                                                   \

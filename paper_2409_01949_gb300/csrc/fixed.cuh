@@ -52,6 +52,9 @@ FX_FN int64_t mul_add(Val a, Val b, int64_t c) {
   return mad(a.hi, b.hi, c) + (cross >> 31);
 }
 
+// v / 2^n (n >= 0), rounded down
+FX_FN int64_t down(int64_t v, int n) { return v >> (n < 63 ? n : 63); }
+
 // The weight scale a as a power of two: weights and biases are at most
 // 2^wexp(a) in magnitude.  Fixed point is used for kMinExp <= wexp <= kMaxExp:
 // below, FP64's error (relative to its terms) is the smaller one; above, the

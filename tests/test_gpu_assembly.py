@@ -209,3 +209,45 @@ def test_nonfinite_operator_gives_nonfinite_entries():
             M, _ = s.get_rows(np.arange(30))
         inside = np.abs((np.arange(4) + 0.5) / 4 - P.interior.points) < 0.25
         assert not np.isfinite(M.reshape(30, 4, 12)[inside]).any()
+
+
+# operators of one or two terms: with one subdomain over every point the window is
+# 1, and an entry is t (c1 w / sigma - 2 phi c2 (w / sigma)^2) + phi c0 alone, which
+# goes with a feature's weights to zero
+@pytest.mark.parametrize("dim,c0,c1,c2", [
+    (1, 0.0, (0.0, 0.0), (-1.0, 0.0)), (1, 0.0, (1.0, 0.0), (0.0, 0.0)),
+    (1, 0.0, (2.0 ** -9, 0.0), (1.0, 0.0)), (1, 2.0 ** -12, (0.0, 0.0), (-1.0, 0.0)),
+    (2, 0.0, (0.0, 0.0), (-1.0, -1.0)), (2, 0.0, (0.0, 0.0), (1.0, 0.0)),
+    (2, 0.0, (0.0, 1.0), (0.0, 0.0)), (2, 0.0, (1.0, 0.0), (0.0, -(2.0 ** 10)))])
+@pytest.mark.parametrize("a", [1.0, 0.3, 0.07])
+def test_entries_of_small_weights_to_their_own_last_place(dim, c0, c1, c2, a):
+    """Every entry against extended precision, relative to its own terms T and what
+    its argument's rounding does to them, T + |d entry / d s| (|w x| + |b|): 8 units
+    2^-53 of that for the dozen roundings of an FP64 evaluation from exact windows
+    (here 1, with derivatives 0).  Arguments whose own terms are below 2^-6 are
+    left out: phi is held to 2^-60, not to its last place."""
+    Q = np.longdouble
+    n, K = 64, 192
+    r = np.random.default_rng(5)
+    x = r.integers(1, 2 ** 20, (n, dim)) * 2.0 ** -20
+    with E.Solver(dim, (0.0,) * dim, (1.0,) * dim, (1,), 2.0, K, seed=11, weight_scale=a,
+                  precision=E.FP64) as s:
+        W, b = s.params()
+        s.assemble([dict(points=x, rhs=np.zeros(n), c0=c0, c1=c1, c2=c2)])
+        M, _ = s.get_rows(np.arange(n))
+    assert np.abs(W).min() < 2.0 ** -5 * a
+    xt = (x - 0.5).astype(Q)            # mu = 1/2, sigma = 1
+    W, b = W.reshape(K, dim).astype(Q), b.astype(Q)
+    arg = xt @ W.T + b
+    terms = np.abs(xt) @ np.abs(W).T + np.abs(b)
+    phi = np.tanh(arg)
+    t = 1 - phi * phi
+    B, C, aB, aC = 0, 0, 0, 0
+    for i in range(dim):
+        B, aB = B + c1[i] * W[:, i], aB + np.abs(c1[i] * W[:, i])
+        C, aC = C + 2 * c2[i] * W[:, i] ** 2, aC + 2 * np.abs(c2[i]) * W[:, i] ** 2
+    want = (c0 * phi + t * (B - phi * C)) / 8       # row scale 1 / sqrt(64)
+    T = np.abs(c0 * phi) + t * aB + t * np.abs(phi) * aC
+    slope = t * abs(c0) + 2 * np.abs(phi) * t * aB + t * np.abs(1 - 3 * phi * phi) * aC
+    bound = 8 * Q(2) ** -53 * (T + slope * terms) / 8
+    assert np.all((np.abs(M - want) <= bound) | (terms < 2.0 ** -6))
