@@ -153,8 +153,9 @@ __global__ void __launch_bounds__(256) k_eval(const double* __restrict__ xs, int
 // ---- the fixed-point form -------------------------------------------------
 // One column as k_eval_fx reads it: weights, bias and coefficient in fixed
 // point.  The coefficients of a subdomain share an exponent: a = a_fx
-// 2^(ea - 59) with 2^ea above the largest, so that the K terms a_k phi_k are
-// summed as 64-bit integers in units of 2^(ea - 58).
+// 2^(ea - abits) with 2^ea above the largest, and the terms a_k phi_k are summed as
+// 64-bit integers in units of 2^(ea - abits + 1), as fine as a lane's K / 32 terms
+// leave room for (eval_bits).
 struct __align__(16) EvalCol {
   int4 w;    // w0.hi, w0.lo, w1.hi, w1.lo
   int4 ba;   // bias (low, high word), a.hi, a.lo
@@ -168,7 +169,8 @@ constexpr int kNone = kWide + 1;     // all coefficients zero
 __global__ void __launch_bounds__(128) k_eval_pack(const double* __restrict__ W,
                                                    const double* __restrict__ B,
                                                    const double* __restrict__ a, int dim, int K,
-                                                   int wexp, EvalCol* __restrict__ cols,
+                                                   int wexp, int abits,
+                                                   EvalCol* __restrict__ cols,
                                                    int* __restrict__ expo) {
   __shared__ double red[4];
   const int64_t q0 = (int64_t)blockIdx.x * K;
@@ -187,7 +189,7 @@ __global__ void __launch_bounds__(128) k_eval_pack(const double* __restrict__ W,
   bad |= ea < -900 || ea > 900;
   if (threadIdx.x == 0) expo[blockIdx.x] = bad ? kWide : (mx > 0.0 ? ea : kNone);
   const double ws = scalbn(1.0, 61 - wexp), bs = scalbn(1.0, 60 - wexp);
-  const double as = bad ? 0.0 : scalbn(1.0, 59 - ea);
+  const double as = bad ? 0.0 : scalbn(1.0, abits - ea);
   for (int f = threadIdx.x; f < K; f += blockDim.x) {
     const int64_t q = q0 + f;
     const fx::Val w0 = fx::split(__double2ll_rn(W[q * dim] * ws));
@@ -247,14 +249,16 @@ __device__ __forceinline__ int64_t order_key(double v) {
 // cycles of a sub-partition on a warp of terms, almost all in tanh: 262144
 // points of a 7-level 2-D model with K = 64 took 31.2 ms and take 2.85 ms, 1000
 // points of a 1-D model 45 us and 30 us (the whole call); the error against a
-// 113-bit evaluation is the same, 2.3e-16 of the result in the mean (the
-// windows' part of it).
+// 113-bit evaluation is 1.4e-16 to 2.8e-16 of the result in the mean over eight
+// models, without bias, where the FP64 form's was 1.8e-16 to 3.8e-16 (what is left
+// is the windows' part of it).
 template <bool kTwo>
 __global__ void __launch_bounds__(256) k_eval_fx(
     const double* __restrict__ xs, int64_t n, int K, int L, const double* __restrict__ bnd,
     int nc0, int nc1, const SubGeom* __restrict__ sub, const int* __restrict__ cell_level_off,
     const int* __restrict__ cover_sub, const EvalCol* __restrict__ cols,
-    const int* __restrict__ expo, int shift, int rows, int room, const double* __restrict__ W,
+    const int* __restrict__ expo, int shift, int rows, int abits, int room,
+    const double* __restrict__ W,
     const double* __restrict__ B, const double* __restrict__ a, double* __restrict__ out,
     const Ansatz an) {
   constexpr int dim = kTwo ? 2 : 1;
@@ -349,9 +353,11 @@ __global__ void __launch_bounds__(256) k_eval_fx(
     }
     const fx::Val c = {__shfl_sync(0xffffffffu, cm.hi, j), __shfl_sync(0xffffffffu, cm.lo, j)};
     const int d = __shfl_sync(0xffffffffu, down, j);
-    acc += (fx::mul_add(fx::split(sum), c, 0) + (((int64_t)1 << d) >> 1)) >> d;   // to nearest
+    // to nearest, halves up in even lanes and down in odd ones
+    const int64_t half = (((int64_t)1 << d) - (lane & 1)) >> 1;
+    acc += (fx::mul_exact(fx::split(sum), c, lane & 1) + half) >> d;
   }
-  double part = live ? (double)acc * scalbn(1.0, emax - 57 + room) : 0.0;
+  double part = live ? (double)acc * scalbn(1.0, emax - abits + 2 + room) : 0.0;
   if (wide) {   // subdomains whose coefficients have no shared exponent
     for (int j = 0; j < m; ++j) {
       if (!((wide >> j) & 1u)) continue;
@@ -370,13 +376,18 @@ __global__ void __launch_bounds__(256) k_eval_fx(
   if (lane == 0) out[pt] = total * ansatz_value(an, x, dim);
 }
 
-// Bits to keep free below the aligned sums: a term is below 2^58 units, so an
-// entry's K / 32 terms a lane times cm / 2^62 below (K / 32) 2^57, and m
-// entries add up.
-int eval_room(int K, int m) {
-  const int64_t terms = ceil_div(K, 32) * m;
+// Bits of the coefficients: 62 at most (two 31-bit halves), and a lane's ceil(K / 32)
+// terms, each below 2^(abits - 1), stay below 2^62.
+int eval_bits(int K) {
+  int bits = 62;
+  while (ceil_div(K, 32) << (bits - 1) > (int64_t)1 << 62) --bits;
+  return bits;
+}
+// Bits the aligned sums of a point's m entries, each below 2^61, are moved down by to
+// stay below 2^63.
+int eval_room(int m) {
   int room = 0;
-  while ((int64_t)64 << room < terms) ++room;
+  while ((4 << room) < m) ++room;
   return room;
 }
 
@@ -466,7 +477,7 @@ void eval_model(elmfb_ctx* h, const double* xs, int64_t n, double* out) {
   const double a = h->cfg.weight_scale;
   const int wexp = a > 0.0 ? fx::weight_exp(a) : fx::kMinExp - 1;
   if (h->max_cover <= 32 && wexp >= fx::kMinExp && wexp <= fx::kMaxExp) {
-    const int rows = fx::tanh_rows(h->dim, wexp);
+    const int rows = fx::tanh_rows(h->dim, wexp), abits = eval_bits(h->K);
     const size_t smem = (size_t)rows * 3 * sizeof(int4);
     // columns, then exponents: a workspace of the handle, rewritten on each call
     h->d_eval.alloc((size_t)h->NPhi * sizeof(EvalCol) + (size_t)h->n_sub * sizeof(int), st);
@@ -474,7 +485,7 @@ void eval_model(elmfb_ctx* h, const double* xs, int64_t n, double* out) {
     int* const expo = reinterpret_cast<int*>(cols + h->NPhi);
     k_eval_pack<<<(unsigned)h->n_sub, 128, 0, st>>>(
         h->d_W64.as<double>(), h->d_b64.as<double>(), h->d_a.as<double>(), h->dim, h->K, wexp,
-        cols, expo);
+        abits, cols, expo);
     // few points: half-size blocks, so that they spread over more SMs
     const int threads = n < 152 * 16 ? 128 : 256;
 #define ELMFB_EVAL_FX(TWO)                                                                     \
@@ -483,7 +494,7 @@ void eval_model(elmfb_ctx* h, const double* xs, int64_t n, double* out) {
     k_eval_fx<TWO><<<(unsigned)ceil_div(n * 32, threads), threads, smem, st>>>(                \
         x, n, h->K, h->L, h->d_bnd.as<double>(), h->nc[0], h->nc[1], h->d_sub.as<SubGeom>(),   \
         h->d_cell_level_off.as<int>(), h->d_cover_sub.as<int>(), cols, expo, 54 - wexp, rows,  \
-        eval_room(h->K, h->max_cover), h->d_W64.as<double>(), h->d_b64.as<double>(),           \
+        abits, eval_room(h->max_cover), h->d_W64.as<double>(), h->d_b64.as<double>(),           \
         h->d_a.as<double>(), o, make_ansatz(h->cfg));                                          \
   } while (0)
     if (h->dim == 2) ELMFB_EVAL_FX(true);

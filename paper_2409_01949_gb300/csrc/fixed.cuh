@@ -11,7 +11,7 @@
 //
 // A value v is held as v = hi 2^31 + lo, 0 <= lo < 2^31, so that every partial
 // product is one signed multiply-add; the lo x lo product (less than one unit
-// after the shift) is left out.
+// after the shift, a quarter in the mean) is left out.
 #pragma once
 
 #include <math.h>
@@ -44,12 +44,22 @@ FX_FN int64_t mad(int a, int b, int64_t c) {
 
 FX_FN Val split(int64_t v) { return {(int)(v >> 31), (int)(v & 0x7fffffff)}; }
 
-// c + a b / 2^62, to the nearest unit (but for the lo x lo product): rounding
-// down would put half a unit of the same sign on every one of the thousands of
-// terms of a sum
+// c + a b / 2^62, to the nearest unit but for the lo x lo product: rounding down
+// would put half a unit of the same sign on every one of the thousands of terms of
+// a sum.  The quarter unit that the left-out product takes in the mean has one sign
+// too: sums hold their terms in units well below their own last place.
 FX_FN int64_t mul_add(Val a, Val b, int64_t c) {
   const int64_t cross = mad(a.hi, b.lo, mad(a.lo, b.hi, 1 << 30));
   return mad(a.hi, b.hi, c) + (cross >> 31);
+}
+
+// a b / 2^62, to the nearest unit, a half to either side by `odd`: where b has few
+// bits halves are common, and a sum that rounds half of its terms each way has no
+// bias
+FX_FN int64_t mul_exact(Val a, Val b, int odd) {
+  const int64_t low = (int64_t)(((uint64_t)(uint32_t)a.lo * (uint32_t)b.lo) >> 31);
+  const int64_t cross = mad(a.hi, b.lo, mad(a.lo, b.hi, (1 << 30) - odd + low));
+  return mad(a.hi, b.hi, cross >> 31);
 }
 
 // v / 2^n (n >= 0), rounded down

@@ -114,3 +114,30 @@ def test_points_and_results_in_place_overlapping_or_unaligned():
         raw = torch.zeros(301 * 8 + 4, dtype=torch.uint8, device="cuda")
         assert L.elmfb_eval(s.h, C.c_void_p(x.data_ptr()), 301, C.c_void_p(raw.data_ptr() + 4)) == E.OK
         assert np.array_equal(raw[4:].cpu().numpy().tobytes(), ref.tobytes())
+
+
+@pytest.mark.parametrize("levels,K,delta", [((16,), 64, 2.0), ((1, 2, 4, 8), 33, 2.9)])
+def test_evaluation_has_no_bias(levels, K, delta):
+    """The mean error over 512 points against extended precision.  A point's error
+    is about 2e-16 of the model's size (the windows' part of it, independent from
+    point to point), so that of the mean is about 1e-17: 2^-54 is five of those.
+    Sums whose terms are all rounded to the same side lie above 1e-16."""
+    Q = np.longdouble
+    P = WL.poisson1d(levels=levels, features=K, n_interior=50, delta=delta)
+    r = np.random.default_rng(9)
+    a, x = r.standard_normal(P.n_columns), r.random(512)
+    with E.Solver.from_problem(P) as s:
+        s.set_coeffs(a)
+        W, b = s.params()
+        u = s.eval(x[:, None])
+    W, b, c, t = W.reshape(-1, K).astype(Q), b.reshape(-1, K).astype(Q), a.reshape(-1, K), 0
+    pi, off = 2 * np.arccos(Q(0)), 0
+    for n in levels:
+        d = (x.astype(Q)[:, None] - (np.arange(n) + Q(1) / 2) / n) * n / (Q(delta) / 2)
+        w = np.where(np.abs(d) < 1, np.sin(pi / 2 * (1 - np.minimum(np.abs(d), 1))) ** 4, 0)
+        w = w / w.sum(axis=1, keepdims=True)
+        for j in range(n):
+            t = t + w[:, j] * (np.tanh(d[:, j:j + 1] * W[off + j] + b[off + j]) @ c[off + j].astype(Q))
+        off += n
+    t = t / len(levels)
+    assert abs(np.mean(u - t)) <= 2.0 ** -54 * np.sqrt(np.mean(t * t))
