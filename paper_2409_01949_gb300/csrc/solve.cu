@@ -37,6 +37,7 @@
 #include <type_traits>
 
 #include "elmfb_internal.cuh"
+#include "ring.cuh"
 #include "sm100_ptx.cuh"
 
 namespace {
@@ -553,39 +554,42 @@ __global__ void __launch_bounds__(320) k_gram_diag_fp32(const __grid_constant__ 
     sm100::fence_mbar_init();
   }
   __syncthreads();
-  bool ok = true;
   if (warp == consumers) {
-    const uint32_t step_bytes = (uint32_t)(16 * K * sizeof(float));
-    int st = 0, ph = 1;
-    for (int q0 = 0; q0 < nsteps; q0 += 32) {
-      // 32 steps looked up at once, one a lane
-      int mine_m = 1, mine_x = 0, mine_y = 0;
-      if (q0 + lane < nsteps) {
-        const DiagStepRows sr =
-            diag_step(steps, entry_base, entry_cell, cover_off, ch.y + q0 + lane, K);
-        mine_m = (int)(sr.mK / K);
-        mine_y = (int)(sr.row0 / mine_m);
-        mine_x = (int)(sr.row0 - (int64_t)mine_y * mine_m) * K;
+    struct Io {
+      float* ring;
+      const DiagMaps& maps;
+      uint64_t *full, *empty;
+      const int2* steps;
+      const int64_t* entry_base;
+      const int* entry_cell;
+      const int* cover_off;
+      int K, first, n, lane;
+      int mine_m, mine_x, mine_y;   // of 32 steps looked up at once, one a lane
+      __device__ bool wait_empty(int st, int ph) const {
+        return __all_sync(0xffffffffu, sm100::mbar_wait(&empty[st], ph));
       }
-      const int n = min(32, nsteps - q0);
-      for (int q = 0; q < n; ++q) {
-        const int m = __shfl_sync(0xffffffffu, mine_m, q);
-        const int x = __shfl_sync(0xffffffffu, mine_x, q);
-        const int y = __shfl_sync(0xffffffffu, mine_y, q);
-        if (!sm100::mbar_wait(&empty[st], ph, ok ? sm100::kSpinLimit : 4u)) ok = false;
+      __device__ bool wait_full(int st, int ph) const { return sm100::mbar_wait(&full[st], ph); }
+      __device__ void issue(int q, int st) {
+        if ((q & 31) == 0 && q + lane < n) {
+          const DiagStepRows sr =
+              diag_step(steps, entry_base, entry_cell, cover_off, first + q + lane, K);
+          mine_m = (int)(sr.mK / K);
+          mine_y = (int)(sr.row0 / mine_m);
+          mine_x = (int)(sr.row0 - (int64_t)mine_y * mine_m) * K;
+        }
+        __syncwarp();
+        const int m = __shfl_sync(0xffffffffu, mine_m, q & 31);
+        const int x = __shfl_sync(0xffffffffu, mine_x, q & 31);
+        const int y = __shfl_sync(0xffffffffu, mine_y, q & 31);
         if (lane == 0) {
           sm100::fence_proxy_async_smem();
-          sm100::mbar_arrive_expect_tx(&full[st], step_bytes);
+          sm100::mbar_arrive_expect_tx(&full[st], (uint32_t)(16 * K * sizeof(float)));
           sm100::tma_load_2d(ring + (int64_t)st * 16 * K, &maps.of[m - 1], x, y, &full[st]);
         }
         __syncwarp();
-        if (++st == kDiagRing) {
-          st = 0;
-          ph ^= 1;
-        }
       }
-    }
-    if (!ok && lane == 0) atomicOr(&flags[3], 1);
+    } io{ring, maps, full, empty, steps, entry_base, entry_cell, cover_off, K, ch.y, nsteps, lane, 1, 0, 0};
+    if (!ring_produce(nsteps, kDiagRing, io)) atomicOr(&flags[3], 1);
     return;
   }
   // tile (ti, tj): rows 4 ti .. + 3, columns 8 tj .. + 7 of the upper triangle
@@ -614,7 +618,10 @@ __global__ void __launch_bounds__(320) k_gram_diag_fp32(const __grid_constant__ 
     for (int b = 0; b < 4; ++b) hi[a][b] = lo[a][b] = 0;
   int st = 0, ph = 0;
   for (int q = 0; q < nsteps; ++q) {
-    if (!sm100::mbar_wait(&full[st], ph, ok ? sm100::kSpinLimit : 4u)) ok = false;
+    if (!__all_sync(0xffffffffu, sm100::mbar_wait(&full[st], ph))) {
+      if (lane == 0) atomicOr(&flags[3], 1);   // the result is not used
+      break;
+    }
     if (ti >= 0) {
       const float* sm = ring + (int64_t)st * 16 * K;
       uint64_t acc[4][4];
@@ -654,7 +661,6 @@ __global__ void __launch_bounds__(320) k_gram_diag_fp32(const __grid_constant__ 
       ph ^= 1;
     }
   }
-  if (!ok && lane == 0) atomicOr(&flags[3], 1);
   if (ti < 0) return;
   const int KT = K * (K + 1) / 2;
   double* out = partial + (int64_t)blockIdx.x * KT;
