@@ -431,9 +431,11 @@ int elmfb_batch_solve(int n, const elmfb_batch_item* items, const elmfb_solve_op
                       int n_workers, elmfb_batch_result* results);
 
 /* The autotuner's record (not in the paper).  A shape class is (panel
- * precision, K, most covering panels of a cell, floor(log2 padded rows)); for
- * each class seen by a solve with `autotune`, the fused LSQR pass was timed at
- * three work-unit sizes (the heuristic size, half and twice it) and the
+ * precision, K, most covering panels of a cell, floor(log2 padded rows), and
+ * for FP64-accurate panels whether the heuristic size is the one of systems
+ * with few units, which the entry does not show); for each class seen by a
+ * solve with `autotune`, the fused LSQR pass was timed at three work-unit sizes
+ * (the heuristic size, half and twice it) and the
  * fastest is used from then on.  Writes up to `max` entries and returns the
  * number of classes (negative status on a bad argument). */
 typedef struct {

@@ -2567,7 +2567,8 @@ struct SolveLayout {
 }  // namespace
 
 // Heuristic rows per fused-pass work unit (see build_fused_plan).
-int64_t fused_unit_target(const elmfb_ctx* h) {
+int64_t fused_unit_target(const elmfb_ctx* h, bool* few) {
+  if (few) *few = false;
   // rows per work unit: about NR / 608 (4 waves of one-CTA-per-SM units), but
   // at least the rows of about 2 MB of covering panels, so that a unit's
   // start-up (barrier set-up, the first copies in flight) stays small next to
@@ -2591,6 +2592,7 @@ int64_t fused_unit_target(const elmfb_ctx* h) {
   for (int c = 0; c < h->n_cells; ++c)
     units += ceil_div(h->cell_pstart[c + 1] - h->cell_pstart[c], target);
   if (2 * units >= 152) return target;
+  if (few) *few = true;
   return std::min(target, (ceil_div(h->NR, 152) + 7) & ~int64_t(7));
 }
 
@@ -3129,7 +3131,8 @@ namespace {
 
 // ---- autotuner of the fused pass's work-unit size --------------------------
 // Shape class: panel precision, K, covering panels per cell, log2 of the
-// padded rows.  The first solve of a class with `autotune` times the fused
+// padded rows, and which rule gives the heuristic size (fused_unit_target: it
+// goes by the cells, which the rest of the class does not know).  The first solve of a class with `autotune` times the fused
 // pass (mode 1, t = 0, CUDA events on the handle's stream, one warm-up and
 // three timed launches each) at the heuristic unit size and at half and twice
 // it (half and a quarter where twice would pass the 1024-row cap), keeps the
@@ -3138,8 +3141,10 @@ namespace {
 // several workers only look the choices up (tune_lookup_only).
 struct TuneKey {
   int prec, K, cover, rows_log2;
+  bool few;   // few units: about one per SM
   bool operator<(const TuneKey& o) const {
-    return std::tie(prec, K, cover, rows_log2) < std::tie(o.prec, o.K, o.cover, o.rows_log2);
+    return std::tie(prec, K, cover, rows_log2, few) <
+           std::tie(o.prec, o.K, o.cover, o.rows_log2, o.few);
   }
 };
 std::mutex g_tune_mu;
@@ -3149,7 +3154,9 @@ template <class T>
 int autotune_unit_rows(elmfb_ctx* h) {
   int lg = 0;
   while ((int64_t(1) << (lg + 1)) <= h->NR) ++lg;
-  const TuneKey key{h->cfg.precision, h->K, h->max_cover, lg};
+  bool few;
+  const int64_t t0 = fused_unit_target(h, &few);
+  const TuneKey key{h->cfg.precision, h->K, h->max_cover, lg, few};
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune.find(key);
@@ -3160,7 +3167,6 @@ int autotune_unit_rows(elmfb_ctx* h) {
   if (h->tune_lookup_only) return 0;
   cudaStream_t st = h->stream;
   // half the heuristic, the heuristic, twice it; at the cap a quarter instead of twice
-  const int64_t t0 = fused_unit_target(h);
   const int64_t t_hi = 2 * t0 <= kMaxUnitRows ? 2 * t0 : t0;
   const int64_t t_lo = 2 * t0 <= kMaxUnitRows ? t0 / 2 : t0 / 4;
   int cand[3] = {(int)std::max<int64_t>(8, t_lo & ~7), (int)std::max<int64_t>(8, (t0 / 2) & ~7),

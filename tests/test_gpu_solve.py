@@ -544,3 +544,21 @@ def test_block_jacobi_factors_over_feature_counts(K):
         s.solve(max_iter=1, atol=0.0, btol=0.0, shift=1e-2, check_every=1)
         a = s.coeffs()
     assert np.linalg.norm(a - a_ref) <= 1e-4 * np.linalg.norm(a_ref)
+
+
+def test_autotuned_units_do_not_depend_on_other_systems():
+    """Two FP64 systems of one precision, K, covering panels and log2 of the rows:
+    17 cells (few units: about one per SM, 8 to 32 rows) and 81 cells of 48 rows
+    (every candidate, 256 rows and more, makes a cell one unit).  Tuned after the
+    first, the second solves bit for bit as untuned."""
+    P = [WL.poisson1d(levels=(n,), features=56, n_interior=r) for n, r in ((16, 2000), (80, 3300))]
+    out = []
+    for tune in (0, 1):
+        for p in P[1 - tune:]:
+            with E.Solver.from_problem(p, precision=E.FP64) as s:
+                s.assemble_problem(p)
+                s.solve(preconditioner=E.PREC_NONE, max_iter=12, atol=0.0, btol=0.0, autotune=tune)
+                out.append(s.coeffs())
+    assert np.array_equal(out[0], out[2])
+    tuned = [e for e in E.tuning_table() if e["precision"] == E.FP64 and e["features"] == 56]
+    assert len({e["rows_log2"] for e in tuned}) == 1 and len(tuned) == 2
