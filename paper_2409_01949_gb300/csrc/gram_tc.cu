@@ -69,6 +69,9 @@ __host__ __device__ constexpr int gram_tile_bytes(int K) {
   return gram_box_rows(K) / 16 * gram_block_bytes(K);
 }
 
+// device memory that blocks on their way to the host pass through
+constexpr int64_t kGramStaging = 32 << 20;
+
 // tasks: (first run, end run, 2 boxes + diagonal, block of G)
 __global__ void __launch_bounds__(kGramThreads, 1)
     k_gram_tc(const uint8_t* __restrict__ pt, const int4* __restrict__ tasks,
@@ -430,22 +433,27 @@ int elmfb_get_gram(elmfb_t h, int64_t n, const int* ij, double* out) {
       const bool found = it != h->gram_pair_ij.end() && *it == std::make_pair(i, j);
       which[q] = make_int2(found ? (int)(it - h->gram_pair_ij.begin()) : -1, tr);
     }
-    // in place in device memory, else through a staging buffer
+    // in place in device memory, else through a staging buffer, a slice at a time
     cudaStream_t st = h->stream;
-    const size_t bytes = (size_t)n * K * K * sizeof(double);
+    const int64_t KK = (int64_t)K * K;
+    const bool direct = usable_in_place(h, out, sizeof(double));
+    const int64_t slice = std::min<int64_t>(
+        n, direct ? int64_t(1) << 24 : std::max<int64_t>(1, kGramStaging / (KK * sizeof(double))));
     DevBuf dw, dout;
-    dw.alloc(n * sizeof(int2), st);
-    CUDA_CHECK(cudaMemcpyAsync(dw.p, which.data(), n * sizeof(int2), cudaMemcpyHostToDevice, st));
-    double* o = out;
-    if (!usable_in_place(h, out, sizeof(double))) {
-      dout.alloc(bytes, st);
-      o = dout.as<double>();
+    dw.alloc(slice * sizeof(int2), st);
+    if (!direct) dout.alloc(slice * KK * sizeof(double), st);
+    for (int64_t q = 0; q < n; q += slice) {
+      const int64_t c = std::min(slice, n - q);
+      double* const o = direct ? out + q * KK : dout.as<double>();
+      CUDA_CHECK(cudaMemcpyAsync(dw.p, which.data() + q, c * sizeof(int2), cudaMemcpyHostToDevice,
+                                 st));
+      k_gram_blocks<<<dim3((unsigned)c, (unsigned)ceil_div(KK, 256)), 256, 0, st>>>(
+          dw.as<int2>(), K, h->d_gram.as<float>(), o);
+      check_launch("k_gram_blocks");
+      count_launch(h);
+      if (!direct)
+        CUDA_CHECK(cudaMemcpyAsync(out + q * KK, o, c * KK * sizeof(double), cudaMemcpyDefault, st));
     }
-    k_gram_blocks<<<dim3((unsigned)n, (unsigned)ceil_div(K * K, 256)), 256, 0, st>>>(
-        dw.as<int2>(), K, h->d_gram.as<float>(), o);
-    check_launch("k_gram_blocks");
-    count_launch(h);
-    if (dout.p) CUDA_CHECK(cudaMemcpyAsync(out, dout.p, bytes, cudaMemcpyDefault, st));
     stream_sync(h);
     return ELMFB_OK;
   } catch (const elmfb_error& e) {

@@ -168,3 +168,22 @@ def test_gram_block_depends_on_its_own_rows_only(K, n):
         steps = np.count_nonzero(np.abs(bi).any(1) & np.abs(bj).any(1)) / 16 + 16
         mag = np.abs(bi).T @ np.abs(bj)
         assert np.all(np.abs(out[0][q] - bi.T @ bj) <= steps * 2.0 ** -22 * mag)
+
+
+def test_blocks_to_the_host_take_little_device_memory():
+    """600 MB of blocks asked for into host memory pass through a bounded buffer
+    (32 MB; the library's pool keeps what it has taken, so the free memory shows it)."""
+    torch = pytest.importorskip("torch")
+    P = WL.poisson2d(levels=(2,), features=128, n_side=12, n_boundary_side=4)
+    pairs = [(q % 4, (q // 4) % 4) for q in range(4601)]
+    with E.Solver.from_problem(P, precision=E.MIXED) as s:
+        s.assemble_problem(P)
+        s.compute_gram()
+        few = s.gram_blocks(pairs[:16])
+        E.trim_memory()
+        before = torch.cuda.mem_get_info()[0]
+        got = s.gram_blocks(pairs)
+        taken = before - torch.cuda.mem_get_info()[0]
+    assert taken <= 128 << 20
+    for q in range(0, 4601, 16):
+        assert np.array_equal(got[q:q + 16], few[:4601 - q])
