@@ -433,8 +433,11 @@ int elmfb_get_gram(elmfb_t h, int64_t n, const int* ij, double* out) {
       const bool found = it != h->gram_pair_ij.end() && *it == std::make_pair(i, j);
       which[q] = make_int2(found ? (int)(it - h->gram_pair_ij.begin()) : -1, tr);
     }
-    // in place in device memory, else through a staging buffer, a slice at a time
-    cudaStream_t st = h->stream;
+    // In place in device memory, else through a staging buffer, a slice at a time; on
+    // the legacy stream, as a plain copy to `out` would be, so that work on `out` that
+    // is pending there or on blocking streams comes first (the blocks themselves were
+    // complete when compute_gram returned).
+    cudaStream_t st = cudaStreamLegacy;
     const int64_t KK = (int64_t)K * K;
     const bool direct = usable_in_place(h, out, sizeof(double));
     const int64_t slice = std::min<int64_t>(
@@ -454,7 +457,7 @@ int elmfb_get_gram(elmfb_t h, int64_t n, const int* ij, double* out) {
       if (!direct)
         CUDA_CHECK(cudaMemcpyAsync(out + q * KK, o, c * KK * sizeof(double), cudaMemcpyDefault, st));
     }
-    stream_sync(h);
+    CUDA_CHECK(cudaStreamSynchronize(st));
     return ELMFB_OK;
   } catch (const elmfb_error& e) {
     h->err = e.msg;

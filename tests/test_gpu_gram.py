@@ -187,3 +187,23 @@ def test_blocks_to_the_host_take_little_device_memory():
     assert taken <= 128 << 20
     for q in range(0, 4601, 16):
         assert np.array_equal(got[q:q + 16], few[:4601 - q])
+
+
+def test_blocks_in_place_come_after_pending_work_on_the_buffer():
+    """A handle on a stream of its own writes blocks into a device buffer that the
+    default stream is still to fill: the blocks are what remains, as after a copy."""
+    torch = pytest.importorskip("torch")
+    P = WL.poisson2d(levels=(2,), features=64, n_side=12, n_boundary_side=4)
+    p = np.array([(0, 0), (0, 3), (1, 2)], dtype=np.int32)
+    side = torch.cuda.Stream()
+    with E.Solver.from_problem(P, precision=E.MIXED, stream=side.cuda_stream) as s:
+        s.assemble_problem(P)
+        s.compute_gram()
+        want = s.gram_blocks(p)
+        out = torch.zeros((3, 64, 64), dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        torch.cuda._sleep(100_000_000)   # some 50 ms
+        out.fill_(7.0)
+        assert E.lib().elmfb_get_gram(s.h, 3, p.ctypes.data, out.data_ptr()) == E.OK
+        torch.cuda.synchronize()
+    assert np.array_equal(out.cpu().numpy(), want)
