@@ -216,3 +216,34 @@ def test_gnn_gradient_at_ragged_sizes(K, B):
     assert np.allclose(Y, Yo, rtol=0, atol=1e-4 * np.abs(Yo).max())
     assert loss == pytest.approx(Lo.item(), rel=1e-4)
     assert np.allclose(grad, go, rtol=0, atol=1e-4 * np.abs(go).max())
+
+
+def test_message_layer_sums_each_weight_by_itself():
+    """A message layer adds two FP32 sums of 64 products, self and neighbours, the
+    bias with the first: one sum of 128 has 1.4 times the rounding error.  A network
+    whose other layers pass small integers through unchanged shows one layer's
+    rounding: all outputs (but for double roundings of this FP64 emulation of fused
+    multiply-adds, one in 10^6) have the bits of that order of the sums."""
+    K = H = 64
+    P = WL.poisson2d(levels=(1, 4), features=K, n_side=24, n_boundary_side=12)
+    rng = np.random.default_rng(3)
+    ws, wn = (rng.standard_normal((2, H, H)) / 8).astype(np.float32)
+    b = rng.standard_normal(H).astype(np.float32)
+    eye, zero = np.eye(H, dtype=np.float32), np.zeros((H, H), dtype=np.float32)
+    z = np.zeros(H, dtype=np.float32)
+    w = np.concatenate([v.ravel() for v in (eye, z, eye, zero, z, eye, zero, z, ws, wn, b, eye, z)])
+    X = rng.integers(0, 16, (4, P.n_subdomains, K)).astype(np.float32)
+    with E.Solver.from_problem(P, precision=E.FP32) as s:
+        s.assemble_problem(P)
+        nbrs = s.gnn_graph()
+        s.gnn_set_weights(w)
+        Y, _, _ = s.gnn_eval(X)
+    mean = np.stack([X[:, nb].sum(axis=1) / np.float32(len(nb)) for nb in nbrs], axis=1)
+
+    def chain(A, W):
+        v = np.zeros(A.shape, dtype=np.float32)
+        for k in range(H):
+            v = (A[..., k:k + 1].astype(np.float64) * W[:, k] + v).astype(np.float32)
+        return v
+    want = np.maximum(chain(mean, wn) + (chain(X, ws) + b), 0)
+    assert np.mean(Y == want) >= 0.999
