@@ -15,7 +15,10 @@ import shutil
 import subprocess
 import sys
 
-from . import tanh_table
+if __package__:
+    from . import tanh_table
+else:   # run as a script: python paper_2409_01949_gb300/build.py
+    import tanh_table
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -76,5 +79,5 @@ def build(verbose: bool = False, force: bool = False, extra_flags=()) -> str:
     return LIB
 
 
-if __name__ == "__main__":   # python -m paper_2409_01949_gb300.build
+if __name__ == "__main__":
     print(build(verbose="-v" in sys.argv, force="-f" in sys.argv))

@@ -6,6 +6,8 @@ import ctypes
 import os
 import re
 import shutil
+import subprocess
+import sys
 
 import pytest
 
@@ -51,3 +53,10 @@ def test_default_solve_options_without_gpu(libpath):
     import paper_2409_01949_gb300 as E
     o = E.default_solve_opts()
     assert o.method == E.SOLVE_LSQR and o.max_iter == 15000 and o.check_every == 50
+
+
+def test_build_runs_as_a_script_and_as_a_module(libpath):
+    for args in (["paper_2409_01949_gb300/build.py"], ["-m", "paper_2409_01949_gb300.build"]):
+        out = subprocess.run([sys.executable, *args], cwd=ROOT, capture_output=True, text=True)
+        assert out.returncode == 0, out.stderr
+        assert os.path.samefile(out.stdout.split()[-1], libpath)
