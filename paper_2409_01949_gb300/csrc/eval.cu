@@ -163,39 +163,47 @@ struct __align__(16) EvalCol {
 constexpr int kWide = -100000;       // no shared exponent: the subdomain is evaluated in FP64
 constexpr int kNone = kWide + 1;     // all coefficients zero
 
-// Columns of subdomain blockIdx.x in fixed point and their exponent ea, or
+// v 2^k to the nearest integer (v finite, |v 2^k| <= 2^62), on the integer pipes
+__device__ __forceinline__ int64_t to_fixed(double v, int k) {
+  const int64_t bits = __double_as_longlong(v);
+  const int e = (int)(bits >> 52) & 0x7ff;
+  const int64_t m = (bits & 0xfffffffffffffll) | (e ? 0x10000000000000ll : 0ll);
+  const int sh = max(e, 1) - 1075 + k;
+  const int r = min(max(-sh, 0), 62);
+  const int64_t n = sh >= 0 ? m << min(sh, 10) : (m + (((int64_t)1 << r) >> 1)) >> r;
+  return bits < 0 ? -n : n;
+}
+
+// A warp per subdomain: its columns in fixed point and their exponent ea, or
 // kWide where a coefficient is not finite or the exponent out of range, kNone
-// where all are zero.
+// where all are zero.  32 bytes written for every 24 or 32 read; a block per
+// subdomain, with conversions in FP64, took 6 ns a subdomain whatever its K: one
+// point of a model of 256^2 subdomains, K = 16, 412 us, 50 us with this kernel (33 us
+// in FP64, which it is dispatched to), one of 7 levels to 64^2, K = 64, 85 us and 55.
 __global__ void __launch_bounds__(128) k_eval_pack(const double* __restrict__ W,
                                                    const double* __restrict__ B,
                                                    const double* __restrict__ a, int dim, int K,
-                                                   int wexp, int abits,
+                                                   int n_sub, int wexp, int abits,
                                                    EvalCol* __restrict__ cols,
                                                    int* __restrict__ expo) {
-  __shared__ double red[4];
-  const int64_t q0 = (int64_t)blockIdx.x * K;
-  double mx = 0.0;
-  bool bad = false;
-  for (int f = threadIdx.x; f < K; f += blockDim.x) {
-    const double v = fabs(a[q0 + f]);
-    bad |= !(v <= 1.7976931348623157e308);
-    mx = fmax(mx, v);
-  }
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  bad = __syncthreads_or(bad);
-  mx = fmax(fmax(red[0], red[1]), fmax(red[2], red[3]));
-  const int ea = mx > 0.0 ? ilogb(mx) + 1 : 0;
-  bad |= ea < -900 || ea > 900;
-  if (threadIdx.x == 0) expo[blockIdx.x] = bad ? kWide : (mx > 0.0 ? ea : kNone);
-  const double ws = scalbn(1.0, 61 - wexp), bs = scalbn(1.0, 60 - wexp);
-  const double as = bad ? 0.0 : scalbn(1.0, abits - ea);
-  for (int f = threadIdx.x; f < K; f += blockDim.x) {
+  const int s = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (s >= n_sub) return;
+  const int64_t q0 = (int64_t)s * K;
+  int64_t mx = 0;   // |a| orders as its bits do, not finite values above the others
+#pragma unroll 2
+  for (int f = lane; f < K; f += 32)
+    mx = max(mx, (int64_t)(__double_as_longlong(a[q0 + f]) & 0x7fffffffffffffffll));
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, (int64_t)__shfl_xor_sync(0xffffffffu, mx, o));
+  const int ea = (int)(mx >> 52) - 1022;
+  const bool bad = mx != 0 && (ea < -900 || ea > 900);
+  if (lane == 0) expo[s] = bad ? kWide : (mx != 0 ? ea : kNone);
+#pragma unroll 2
+  for (int f = lane; f < K; f += 32) {
     const int64_t q = q0 + f;
-    const fx::Val w0 = fx::split(__double2ll_rn(W[q * dim] * ws));
-    const fx::Val w1 = fx::split(dim == 2 ? __double2ll_rn(W[q * dim + 1] * ws) : 0ll);
-    const int64_t b = __double2ll_rn(B[q] * bs);
-    const fx::Val av = fx::split(bad ? 0ll : __double2ll_rn(a[q] * as));
+    const fx::Val w0 = fx::split(to_fixed(W[q * dim], 61 - wexp));
+    const fx::Val w1 = fx::split(dim == 2 ? to_fixed(W[q * dim + 1], 61 - wexp) : 0ll);
+    const int64_t b = to_fixed(B[q], 60 - wexp);
+    const fx::Val av = fx::split(bad || mx == 0 ? 0ll : to_fixed(a[q], abits - ea));
     cols[q].w = make_int4(w0.hi, w0.lo, w1.hi, w1.lo);
     cols[q].ba = make_int4((int)(uint32_t)b, (int)(b >> 32), av.hi, av.lo);
   }
@@ -474,18 +482,24 @@ void eval_model(elmfb_ctx* h, const double* xs, int64_t n, double* out) {
   // Fixed point wherever a point's covering subdomains fit a warp and the
   // weight scale is in its range (fixed.cuh); FP64 otherwise: below the range
   // FP64's error, relative to the small arguments, is the smaller one.
+  // Few points of a model of many columns too: packing the columns takes 3 us and
+  // 1.1e-5 us a column (measured), where FP64 takes 0.9 us more than fixed point for
+  // every 32 features of the point's subdomains, or 2.4 us once a block of 8 points
+  // shares an SM, for each wave of blocks.
   const double a = h->cfg.weight_scale;
   const int wexp = a > 0.0 ? fx::weight_exp(a) : fx::kMinExp - 1;
-  if (h->max_cover <= 32 && wexp >= fx::kMinExp && wexp <= fx::kMaxExp) {
+  const double slower = n <= 4 ? 0.9 : 2.4 * (double)ceil_div(n, 8 * 152);
+  const bool few = slower * (double)(h->max_cover * ceil_div(h->K, 32)) < 3.0 + 1.1e-5 * h->NPhi;
+  if (h->max_cover <= 32 && wexp >= fx::kMinExp && wexp <= fx::kMaxExp && !few) {
     const int rows = fx::tanh_rows(h->dim, wexp), abits = eval_bits(h->K);
     const size_t smem = (size_t)rows * 3 * sizeof(int4);
     // columns, then exponents: a workspace of the handle, rewritten on each call
     h->d_eval.alloc((size_t)h->NPhi * sizeof(EvalCol) + (size_t)h->n_sub * sizeof(int), st);
     EvalCol* const cols = h->d_eval.as<EvalCol>();
     int* const expo = reinterpret_cast<int*>(cols + h->NPhi);
-    k_eval_pack<<<(unsigned)h->n_sub, 128, 0, st>>>(
-        h->d_W64.as<double>(), h->d_b64.as<double>(), h->d_a.as<double>(), h->dim, h->K, wexp,
-        abits, cols, expo);
+    k_eval_pack<<<(unsigned)ceil_div(h->n_sub, 4), 128, 0, st>>>(
+        h->d_W64.as<double>(), h->d_b64.as<double>(), h->d_a.as<double>(), h->dim, h->K, h->n_sub,
+        wexp, abits, cols, expo);
     // few points: half-size blocks, so that they spread over more SMs
     const int threads = n < 152 * 16 ? 128 : 256;
 #define ELMFB_EVAL_FX(TWO)                                                                     \

@@ -141,3 +141,19 @@ def test_evaluation_has_no_bias(levels, K, delta):
         off += n
     t = t / len(levels)
     assert abs(np.mean(u - t)) <= 2.0 ** -54 * np.sqrt(np.mean(t * t))
+
+
+@pytest.mark.parametrize("n,launches", [(1, 1), (4, 1), (5, 2), (300, 2)])
+def test_few_points_of_a_model_of_many_columns(n, launches):
+    """Up to four points of a model of 128^2 subdomains are evaluated in FP64 (one
+    launch), which reads their own columns; from five on the columns are packed
+    first.  Both agree with the oracle."""
+    P = _problem(2, (128,), 8, 1.0, n_side=8, n_boundary_side=4)
+    a = np.random.default_rng(6).standard_normal(P.n_columns)
+    X = _points(P, n)
+    with E.Solver.from_problem(P) as s:
+        s.set_coeffs(a)
+        before = s.kernel_launches()
+        u = s.eval(X)
+        assert s.kernel_launches() - before == launches
+    assert np.abs(u - OE.u_hat(P, a, X)).max() <= _tol(P, a)
