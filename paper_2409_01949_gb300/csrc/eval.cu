@@ -490,11 +490,21 @@ void eval_model(elmfb_ctx* h, const double* xs, int64_t n, double* out) {
   const int wexp = a > 0.0 ? fx::weight_exp(a) : fx::kMinExp - 1;
   const double slower = n <= 4 ? 0.9 : 2.4 * (double)ceil_div(n, 8 * 152);
   const bool few = slower * (double)(h->max_cover * ceil_div(h->K, 32)) < 3.0 + 1.1e-5 * h->NPhi;
-  if (h->max_cover <= 32 && wexp >= fx::kMinExp && wexp <= fx::kMaxExp && !few) {
+  bool fixed = h->max_cover <= 32 && wexp >= fx::kMinExp && wexp <= fx::kMaxExp && !few;
+  if (fixed) {
+    // columns, then exponents: a workspace of the handle, rewritten on each call; FP64
+    // needs none, so a device that is full does not fail the call
+    try {
+      h->d_eval.alloc((size_t)h->NPhi * sizeof(EvalCol) + (size_t)h->n_sub * sizeof(int), st);
+    } catch (const elmfb_error& e) {
+      if (e.code != ELMFB_ERR_OOM) throw;
+      cudaGetLastError();
+      fixed = false;
+    }
+  }
+  if (fixed) {
     const int rows = fx::tanh_rows(h->dim, wexp), abits = eval_bits(h->K);
     const size_t smem = (size_t)rows * 3 * sizeof(int4);
-    // columns, then exponents: a workspace of the handle, rewritten on each call
-    h->d_eval.alloc((size_t)h->NPhi * sizeof(EvalCol) + (size_t)h->n_sub * sizeof(int), st);
     EvalCol* const cols = h->d_eval.as<EvalCol>();
     int* const expo = reinterpret_cast<int*>(cols + h->NPhi);
     k_eval_pack<<<(unsigned)ceil_div(h->n_sub, 4), 128, 0, st>>>(

@@ -157,3 +157,32 @@ def test_few_points_of_a_model_of_many_columns(n, launches):
         u = s.eval(X)
         assert s.kernel_launches() - before == launches
     assert np.abs(u - OE.u_hat(P, a, X)).max() <= _tol(P, a)
+
+
+def test_evaluation_on_a_full_device():
+    """A model of 8.4 million columns: its packed columns take 270 MB.  With less
+    than that free the points are evaluated in FP64, which takes no memory of its
+    own, to the same values within the tolerance."""
+    import torch
+    P = _problem(2, (256,), 128, 1.0, n_side=8, n_boundary_side=4)
+    a = np.random.default_rng(8).standard_normal(P.n_columns)
+    x = torch.from_numpy(_points(P, 5000)).cuda()
+    out = torch.empty((2, 5000), dtype=torch.float64, device="cuda")
+    fill = None
+    for k in range(2):
+        with E.Solver.from_problem(P) as s:
+            s.set_coeffs(a)
+            torch.cuda.synchronize()
+            if k:
+                E.trim_memory()
+                torch.cuda.empty_cache()
+                fill = torch.empty(torch.cuda.mem_get_info()[0] - (160 << 20), dtype=torch.uint8,
+                                   device="cuda")
+            before = s.kernel_launches()
+            s.eval(x, out[k])
+            assert s.kernel_launches() - before == (1 if k else 2)
+            del fill
+            fill = None
+        E.trim_memory()
+    torch.cuda.empty_cache()
+    assert float((out[0] - out[1]).abs().max()) <= 2 * _tol(P, a)
