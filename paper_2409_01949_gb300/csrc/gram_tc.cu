@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kGramThreads, 1)
       const int buf = q & 1;
       const int4 task = tasks[t];
       // a pair is one chain: the wait grows with its boxes (each within the limits above)
-      const uint32_t limit = sm100::kSpinLimit + 256u * (uint32_t)(task.z >> 1);
+      const uint32_t limit = sm100::kSpinLimit + 256u * min((uint32_t)(task.z >> 1), 1u << 22);
       if (!sm100::mbar_wait(&acc_full[buf], (q >> 1) & 1, limit)) {
         ok = false;
         break;
