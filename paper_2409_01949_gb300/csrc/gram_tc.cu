@@ -38,12 +38,9 @@
 //
 // Every mbarrier wait is bounded; a timeout raises flags[2].
 #include <algorithm>
-#include <cmath>
 #include <cstring>
 #include <functional>
-#include <numeric>
 #include <queue>
-#include <unordered_map>
 
 #include <new>
 #include <stdexcept>
@@ -260,59 +257,67 @@ void gram_build_pairs(elmfb_ctx* h) {
   struct Run {
     int a, b, len;   // panel rows of i and j
   };
-  // pairs numbered as the cells meet them, then sorted by (i, j)
-  std::unordered_map<uint64_t, int> number;
-  std::vector<uint64_t> keys;
-  std::vector<std::vector<Run>> runs_of;
-  std::vector<int> first_cell;
-  number.reserve(16 * (size_t)h->n_sub);
-  for (int c = 0; c < h->n_cells; ++c) {
-    if (h->cell_count[c] == 0) continue;
-    const int pad = h->cell_pstart[c + 1] - h->cell_pstart[c];
-    for (int e1 = h->cover_off[c]; e1 < h->cover_off[c + 1]; ++e1)
-      for (int e2 = e1; e2 < h->cover_off[c + 1]; ++e2) {
-        const int s1 = h->cover_sub[e1], s2 = h->cover_sub[e2];
-        const int a = (int)(h->panel_off[s1] + h->cover_start[e1]);
-        const int b = (int)(h->panel_off[s2] + h->cover_start[e2]);
-        const uint64_t key = ((uint64_t)(uint32_t)s1 << 32) | (uint32_t)s2;
-        const auto [it, fresh] = number.try_emplace(key, (int)keys.size());
-        if (fresh) {
-          keys.push_back(key);
-          runs_of.emplace_back();
-          first_cell.push_back(c);
-        }
-        auto& v = runs_of[it->second];
-        if (!v.empty() && v.back().a + v.back().len == a && v.back().b + v.back().len == b)
-          v.back().len += pad;
-        else
-          v.push_back({a, b, pad});
-      }
-  }
-  std::vector<int> order(keys.size());
-  std::iota(order.begin(), order.end(), 0);
-  std::sort(order.begin(), order.end(), [&](int x, int y) { return keys[x] < keys[y]; });
-  h->gram_pair_ij.clear();
   struct Task {
     int4 t;
     int at;   // the pair's first cell
     int boxes;
   };
+  // the entries of every subdomain, in cell order
+  const int ne = (int)h->cover_sub.size();
+  std::vector<int> off(h->n_sub + 1, 0), ent(ne);
+  for (int e = 0; e < ne; ++e) off[h->cover_sub[e] + 1]++;
+  for (int s = 0; s < h->n_sub; ++s) off[s + 1] += off[s];
+  {
+    std::vector<int> fill(off.begin(), off.end() - 1);
+    for (int e = 0; e < ne; ++e) ent[fill[h->cover_sub[e]]++] = e;
+  }
+  h->gram_pair_ij.clear();
   std::vector<Task> tasks;
   std::vector<int4> runs;
   int64_t total = 0;
-  for (size_t p = 0; p < order.size(); ++p) {
-    const uint64_t key = keys[order[p]];
-    h->gram_pair_ij.push_back({(int)(key >> 32), (int)(uint32_t)key});
-    const int diag = (key >> 32) == (uint32_t)key;
-    const int r0 = (int)runs.size();
-    int boxes = 0;
-    for (const Run& r : runs_of[order[p]]) {
-      runs.push_back(make_int4(r.a, r.b, r.len, 0));
-      boxes += (int)ceil_div(r.len, gram_box_rows(h->K));
+  // subdomain by subdomain, its pairs' runs gathered by the partner
+  std::vector<int> slot(h->n_sub, -1), partners, first_cell;
+  std::vector<std::vector<Run>> runs_of;
+  for (int s1 = 0; s1 < h->n_sub; ++s1) {
+    partners.clear();
+    first_cell.clear();
+    for (int q = off[s1]; q < off[s1 + 1]; ++q) {
+      const int e1 = ent[q], c = h->entry_cell[e1];
+      if (h->cell_count[c] == 0) continue;
+      const int pad = h->cell_pstart[c + 1] - h->cell_pstart[c];
+      const int a = (int)(h->panel_off[s1] + h->cover_start[e1]);
+      for (int e2 = e1; e2 < h->cover_off[c + 1]; ++e2) {
+        const int s2 = h->cover_sub[e2];
+        const int b = (int)(h->panel_off[s2] + h->cover_start[e2]);
+        if (slot[s2] < 0) {
+          slot[s2] = (int)partners.size();
+          partners.push_back(s2);
+          first_cell.push_back(c);
+          if (runs_of.size() < partners.size()) runs_of.emplace_back();
+          runs_of[slot[s2]].clear();
+        }
+        auto& v = runs_of[slot[s2]];
+        if (!v.empty() && v.back().a + v.back().len == a && v.back().b + v.back().len == b)
+          v.back().len += pad;
+        else
+          v.push_back({a, b, pad});
+      }
     }
-    tasks.push_back({make_int4(r0, (int)runs.size(), 2 * boxes + diag, (int)p),
-                     first_cell[order[p]], boxes});
-    total += boxes;
+    std::sort(partners.begin(), partners.end());
+    for (int s2 : partners) {
+      const int k = slot[s2], r0 = (int)runs.size();
+      slot[s2] = -1;
+      int boxes = 0;
+      for (const Run& r : runs_of[k]) {
+        runs.push_back(make_int4(r.a, r.b, r.len, 0));
+        boxes += (int)ceil_div(r.len, gram_box_rows(h->K));
+      }
+      tasks.push_back({make_int4(r0, (int)runs.size(), 2 * boxes + (s1 == s2),
+                                 (int)h->gram_pair_ij.size()),
+                       first_cell[k], boxes});
+      h->gram_pair_ij.push_back({s1, s2});
+      total += boxes;
+    }
   }
   int sms = 0;
   CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
@@ -350,7 +355,7 @@ void gram_build_pairs(elmfb_ctx* h) {
   CUDA_CHECK(cudaMemcpyAsync(h->d_gram_task_off.p, task_off.data(), task_off.size() * sizeof(int),
                              cudaMemcpyHostToDevice, h->stream));
   h->gram_ctas = ctas;
-  h->n_gram_pairs = (int64_t)order.size();
+  h->n_gram_pairs = (int64_t)h->gram_pair_ij.size();
   auto up = [&](DevBuf& d, const std::vector<int4>& v) {
     d.alloc(std::max<size_t>(v.size(), 1) * sizeof(int4), h->stream);
     if (!v.empty())
