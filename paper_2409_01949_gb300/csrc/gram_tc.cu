@@ -34,7 +34,8 @@
 // the CTA with the least work so far, so that all CTAs are in the same place at the
 // same time and the panels stay in L2.  400^2 points, levels 1..16, K = 128 (6297
 // pairs), against one CTA per pair, pair after pair: 1.64 -> 0.79 ms, 330 -> 690
-// TFLOP/s.
+// TFLOP/s; 2048^2, levels 1..64, K = 64: 49.6 -> 33.8 ms, 170 -> 249 TFLOP/s (half of
+// each MMA's rows are past K there).
 //
 // Every mbarrier wait is bounded; a timeout raises flags[2].
 #include <algorithm>
@@ -60,7 +61,7 @@ constexpr size_t kGramSmem = kGramRing + 16 * 1024 + 1024;
 // cycles whatever its size (boxes of 64 rows took the same time at K = 64 and K =
 // 128, and half the ring cost 4%), so it is as large as leaves three stages or more
 // of the ring: 64 -> 128 rows took 0.94 -> 0.75 ms at K = 128, 45.6 -> 33.4 ms at K =
-// 64 on the workloads above.
+// 64 on the workloads above (with their pairs cut).
 __host__ __device__ constexpr int gram_box_rows(int K) { return K <= 32 ? 256 : 128; }
 __host__ __device__ constexpr int gram_tile_bytes(int K) {
   return gram_box_rows(K) / 16 * gram_block_bytes(K);

@@ -522,9 +522,8 @@ __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
 // rows of a cell with m covering panels are m K elements apart, so the whole panel
 // array is described once per m as a matrix of rows m K wide, and a step starts at
 // (row % m) K of row / m (0.5 ms less than 16 bulk copies of 256 bytes a step on
-// the large 2-D workload).  Block-Jacobi LSQR of 20 steps at 400^2, K = 128: 8.25 ->
-// 7.91 ms, all of it these blocks (1.96 -> 1.6 ms); at K = 64 (72 of 96 lanes hold a
-// tile) the two forms take the same time.
+// the large 2-D workload).  400^2, levels 1..16, K = 128: 1.96 -> 1.39 ms; 2048^2,
+// levels 1..64, K = 64 (72 of 96 lanes hold a tile): 17.6 -> 14.8 ms.
 constexpr int kDiagRing = 8;
 constexpr int kDiagMaps = 32;   // covering panels of a cell, at most
 struct DiagMaps {
