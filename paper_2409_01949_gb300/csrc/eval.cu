@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(256) k_eval_fx(
 // terms, each below 2^(abits - 1), stay below 2^62.
 int eval_bits(int K) {
   int bits = 62;
-  while (ceil_div(K, 32) << (bits - 1) > (int64_t)1 << 62) --bits;
+  while (ceil_div(K, 32) > (int64_t)1 << (63 - bits)) --bits;
   return bits;
 }
 // Bits the aligned sums of a point's m entries, each below 2^61, are moved down by to

@@ -186,3 +186,21 @@ def test_evaluation_on_a_full_device():
         E.trim_memory()
     torch.cuda.empty_cache()
     assert float((out[0] - out[1]).abs().max()) <= 2 * _tol(P, a)
+
+
+@pytest.mark.parametrize("K", [1, 32, 33, 64, 65, 96, 97, 128, 129, 160, 255, 256])
+@pytest.mark.parametrize("dim,levels,delta", [(1, (5,), 2.0), (1, (1, 2, 4, 8, 16, 32), 2.9),
+                                              (2, (1, 2, 4), 2.9)])
+def test_sums_of_largest_terms(K, dim, levels, delta):
+    """Every term at its largest and of one sign: the coefficients just below a
+    power of two, with the sign of their features, which a weight scale of 64
+    saturates nearly everywhere.  A lane's sums and those over the covering
+    subdomains come as close to their bounds as they can."""
+    P = _problem(dim, levels, K, 64.0, delta=delta)
+    X = np.random.default_rng(2).random((400, dim))
+    with E.Solver.from_problem(P) as s:
+        _, b = s.params()
+        a = np.nextafter(2.0, 0.0) * np.sign(b)
+        for v in (a, -a, np.abs(a)):
+            s.set_coeffs(v)
+            assert np.abs(s.eval(X) - OE.u_hat(P, v, X)).max() <= _tol(P, v)
