@@ -801,7 +801,7 @@ __global__ void __launch_bounds__(128, 4) k_assemble_fx(
       fx::Val w0, w1, u0, u1, q0, q1;
       int s0, s1;
       auto weight = [&](double v, fx::Val& w, fx::Val& u, fx::Val& sq, int& sh) {
-        sh = v == 0.0 ? 0 : max(wexp - 1 - ilogb(v), 0);
+        sh = v == 0.0 ? 200 : max(wexp - 1 - ilogb(v), 0);   // zero: no part in the exponent
         w = fx::split(__double2ll_rn(v * w_in));
         u = fx::split(__double2ll_rn(scalbn(v * w_in, sh)));
         sq = fx::split(fx::mul_add(u, u, 0) << 1);
