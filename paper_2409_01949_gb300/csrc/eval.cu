@@ -257,9 +257,9 @@ __device__ __forceinline__ int64_t order_key(double v) {
 // cycles of a sub-partition on a warp of terms, almost all in tanh: 262144
 // points of a 7-level 2-D model with K = 64 took 31.2 ms and take 2.82 ms, 1000
 // points of a 1-D model 45 us and 29 us (the whole call); the error against a
-// 113-bit evaluation is 1.4e-16 to 2.8e-16 of the result in the mean over eight
-// models, without bias, where the FP64 form's was 1.8e-16 to 3.8e-16 (what is left
-// is the windows' part of it).
+// 113-bit evaluation is 1.4e-16 to 2.8e-16 of the result in the mean square over
+// eight models, its mean below 1e-16, where the FP64 form's was 1.8e-16 to 3.8e-16
+// (what is left is the windows' part of it).
 template <bool kTwo>
 __global__ void __launch_bounds__(256) k_eval_fx(
     const double* __restrict__ xs, int64_t n, int K, int L, const double* __restrict__ bnd,
